@@ -153,91 +153,101 @@ __device__ __forceinline__ float transpose_reduce(float (&v)[NV]) {
     return r;
 }
 
-// Tokens per TMA chunk starting at token `tok`, index `pos` within its
-// frame: never crosses a frame boundary or the end of the range.
-__device__ __forceinline__ int chunk_len(int pos, int64_t tok, int64_t end, int N, int CH) {
-    return (int)min((int64_t)min(CH, N - pos), end - tok);
-}
-
-constexpr int kRelStages = 3;
-constexpr int kRelMaxConsumers = 512;
+constexpr int kRelMaxStages = 16;
+constexpr int kRelMaxWarps = 24;         // consumer warps of a CTA (all groups)
+constexpr int kRelWindow = 128;          // tokens per cross-warp reduction
+constexpr int kRelGroupTokens = 8;       // tokens per warp transpose-reduction
+constexpr size_t kRelSmem = 224 * 1024;   // dynamic shared memory of a CTA (at most)
 constexpr uint64_t kRelTimeoutNs = 2000000000ull;
 
+// Launch shape of the relevance pass (relevance_config).
+struct RelShape {
+    int ch;        // tokens per chunk (a multiple of kRelGroupTokens unless the row is long)
+    int stages;    // ring stages: a multiple of groups, so that a stage always serves the same
+                   // group and that group's warps see every phase of its barrier
+    int groups;    // consumer groups; chunk k of the CTA goes to group k mod groups
+    int gthreads;  // threads of a group (a multiple of 32)
+    int wpart_off, csum_off;   // byte offsets of the window and of the groups' column sums
+};
+
 // One CTA streams tokens [blockIdx.x*L1, +L1) of the flattened [V*T*N] index.
-// The last warp copies chunks of CH consecutive tokens (contiguous in HBM)
-// into a 3-stage shared-memory ring with cp.async.bulk; the other warps
-// (NC threads, VPT 16-byte vectors each) read them from shared memory.  Each
-// consumer warp waits for a chunk itself and hands it back itself; per-token
-// partial dots and norms go to a shared window that all consumers reduce
-// together once per <= 64 tokens, so block barriers are rare.
-template <typename T, int VPT>
-__global__ void __launch_bounds__(kRelMaxConsumers + 32, 1) relevance_pass_kernel(Ctx c, int CH) {
+// The last warp copies chunks of consecutive tokens (contiguous in HBM, never
+// across a frame) into a shared-memory ring with cp.async.bulk.  The other
+// warps form `groups` groups, each wide enough for one token row (VPT 16-byte
+// vectors per thread); a group takes every groups-th chunk, waits for it,
+// hands it back, and keeps its own column sums of the open frame, so a row of
+// few vectors still occupies 15 to 24 warps.  Per-token partial dots and norms
+// go to a window that all consumers reduce together once per <= 128 tokens;
+// the groups' column sums are added (in group order) when the frame ends.
+template <typename T, int VPT, int MAXTHREADS>
+__global__ void __launch_bounds__(MAXTHREADS, 1) relevance_pass_kernel(Ctx c, RelShape sh) {
     // The producer streams only the features, which the kernels before this
     // one do not write, so it starts before the wait for the previous grid
     // (the query pooling) and fills the ring meanwhile; the consumers wait
     // for it before they read u_q or write anything.
     pdl_trigger();
     constexpr int VEC = VecOf<T>::kElems;
-    constexpr int GROUP = 8;                 // tokens per warp transpose-reduction
+    constexpr int GROUP = kRelGroupTokens;
     constexpr int NV = 2 * GROUP;            // GROUP dots + GROUP squared norms
-    constexpr int WIN = 128;                 // tokens per cross-warp reduction
-    constexpr int NWMAX = kRelMaxConsumers / 32;
     extern __shared__ __align__(128) uint8_t rsm[];
-    __shared__ float wpart[2][NWMAX][2][WIN];
-    __shared__ float qsum[NWMAX];
-    __shared__ uint64_t full[kRelStages], empty[kRelStages];
+    __shared__ float qsum[kRelMaxWarps];
+    __shared__ uint64_t full[kRelMaxStages], empty[kRelMaxStages];
     __shared__ volatile int abort_flag;
     const int NC = blockDim.x - 32;          // consumer threads
-    const int nw = NC >> 5;
+    const int nwg = sh.gthreads >> 5;        // warps of a group
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int n_vec = c.D / VEC;
+    const int N = c.N, CH = sh.ch;
     const bool maxsim = c.relevance_mode == WZ_RELEVANCE_MAXSIM;
-    const size_t rowb = (size_t)c.D * sizeof(T);
-    const size_t stage_bytes = (size_t)CH * rowb;
-    const int64_t total = (int64_t)c.V * c.T * c.N;
+    const uint32_t rowb = (uint32_t)c.D * (uint32_t)sizeof(T);
+    const uint32_t stage_bytes = (uint32_t)CH * rowb;
+    const int64_t total = (int64_t)c.V * c.T * N;
     const int64_t start = (int64_t)blockIdx.x * c.L1;
-    const int64_t end = min(start + c.L1, total);
+    const int len = start < total ? (int)min(c.L1, total - start) : 0;   // tokens of this CTA (grid <= 2048 CTAs)
     if (threadIdx.x == 0) {
-        for (int s = 0; s < kRelStages; ++s) {
+        for (int s = 0; s < sh.stages; ++s) {
             ptx::mbar_init(&full[s], 1);
-            ptx::mbar_init(&empty[s], (uint32_t)nw);
+            ptx::mbar_init(&empty[s], (uint32_t)nwg);
         }
         abort_flag = 0;
         ptx::fence_barrier_init();
         ptx::fence_proxy_async_smem();
     }
     __syncthreads();
-    if (start >= end) return;
+    if (len <= 0) return;
+    const int64_t f0 = start / N;
+    const int pos0 = (int)(start - f0 * N);   // token index within its frame
 
-    if (warp == nw) {
+    if (threadIdx.x >= NC) {
         // ---------------- producer ----------------
         if (lane == 0) {
             const uint64_t pol = ptx::policy_evict_first();
-            const char *X = static_cast<const char *>(c.X);
+            const char *src = static_cast<const char *>(c.X) + (size_t)start * rowb;
             int s = 0;
             uint32_t ph = 0;
-            int issued[kRelStages] = {-1, -1, -1};
-            int pos = (int)(start % c.N);   // token index within its frame
-            for (int64_t tok = start; tok < end && !abort_flag;) {
-                const int n = chunk_len(pos, tok, end, c.N, CH);
+            uint32_t issued = 0, par = 0;    // per stage: copied to, parity of the last copy
+            for (int tok = 0, pos = pos0; tok < len && !abort_flag;) {
+                const int n = min(min(CH, N - pos), len - tok);
                 if (!ptx::mbar_wait(&empty[s], ph ^ 1u, kRelTimeoutNs)) {
                     atomicOr(c.status, 16);
                     abort_flag = 1;
                     break;
                 }
-                ptx::mbar_arrive_expect_tx(&full[s], (uint32_t)(n * rowb));
-                ptx::bulk_load(rsm + s * stage_bytes, X + (size_t)tok * rowb, (uint32_t)(n * rowb), &full[s], pol);
-                issued[s] = (int)ph;
+                ptx::mbar_arrive_expect_tx(&full[s], (uint32_t)n * rowb);
+                ptx::bulk_load(rsm + s * stage_bytes, src, (uint32_t)n * rowb, &full[s], pol);
+                issued |= 1u << s;
+                par = (par & ~(1u << s)) | (ph << s);
+                src += (size_t)n * rowb;
                 tok += n;
                 pos += n;
-                if (pos == c.N) pos = 0;
-                if (++s == kRelStages) {
+                if (pos == N) pos = 0;
+                if (++s == sh.stages) {
                     s = 0;
                     ph ^= 1u;
                 }
             }
-            for (int k = 0; k < kRelStages; ++k)
-                if (issued[k] >= 0) ptx::mbar_wait(&full[k], (uint32_t)issued[k], kRelTimeoutNs);
+            for (int k = 0; k < sh.stages; ++k)
+                if (issued >> k & 1u) ptx::mbar_wait(&full[k], par >> k & 1u, kRelTimeoutNs);
         }
         return;
     }
@@ -246,27 +256,30 @@ __global__ void __launch_bounds__(kRelMaxConsumers + 32, 1) relevance_pass_kerne
     pdl_wait();
     auto consumer_sync = [&]() { asm volatile("bar.sync 1, %0;" ::"r"(NC) : "memory"); };
     constexpr int NP = VEC / 2;                  // packed pairs per 16-byte vector
-    constexpr int SHIFT = 1;                     // lane l holds reduced value l >> 1
-    int cur_v = -1;
-    f2_t q[VPT][NP];
+    const int grp = (int)threadIdx.x / sh.gthreads;
+    const int gtid = (int)threadIdx.x - grp * sh.gthreads;
+    const int gwarp = gtid >> 5;
+    // window: [2 buffers][nwg][dot, norm][kRelWindow]
+    float *const wpart = reinterpret_cast<float *>(rsm + sh.wpart_off);
+    const int wbuf = nwg * 2 * kRelWindow;
+    float *const csum = reinterpret_cast<float *>(rsm + sh.csum_off);   // [groups - 1][D]
+    // one group: two sets of column sums by token parity (shorter dependent chains)
+    constexpr int CSP = VPT == 1 && MAXTHREADS <= 544 ? 2 : 1;
+    f2_t q[VPT][NP], cs[CSP][VPT][NP];
     float qn = 0.f;
-    // column sums, split by token parity when registers allow (two shorter
-    // dependent chains per group)
-    constexpr int CSP = VPT == 1 ? 2 : 1;
-    f2_t cs[CSP][VPT][NP];
-    int s = 0;
-    uint32_t ph = 0;
+    const uint32_t ring = ptx::smem_u32(rsm) + (uint32_t)gtid * 16u;
     bool dead = false;
-    int buf = 0, wcount = 0;
-    int64_t wbase = start;
-    // frame f, its position t in the video v, and the token index within the
-    // frame are carried along: no 64-bit divisions inside the loop
-    int64_t f = start / c.N;
-    int pos = (int)(start - f * c.N);
-    int tf = (int)(f % c.T), v = (int)(f / c.T);
+    // chunk counter modulo the groups, and the stage and phase of the chunk
+    int turn = 0, s = 0;
+    uint32_t ph = 0;
+    int buf = 0, wcount = 0, wbase = 0;
+    bool csum_read = false;                  // group 0 may still be reading csum
+    int64_t f = f0;
+    int pos = pos0;
+    int tf = (int)(f0 % c.T), v = (int)(f0 / c.T), cur_v = -1;
     bool frame_new = true;
-    for (int64_t tok = start; tok < end;) {
-        const int n = chunk_len(pos, tok, end, c.N, CH);
+    for (int tok = 0; tok < len;) {
+        const int n = min(min(CH, N - pos), len - tok);
         if (frame_new) {
             frame_new = false;
             if (v != cur_v) {
@@ -274,7 +287,7 @@ __global__ void __launch_bounds__(kRelMaxConsumers + 32, 1) relevance_pass_kerne
                 float qq = 0.f;
 #pragma unroll
                 for (int vi = 0; vi < VPT; ++vi) {
-                    const int vidx = threadIdx.x + vi * NC;
+                    const int vidx = gtid + vi * sh.gthreads;
 #pragma unroll
                     for (int e = 0; e < NP; ++e) {
                         const float q0 = vidx < n_vec ? c.qbar32[(size_t)v * c.D + vidx * VEC + 2 * e] : 0.f;
@@ -288,7 +301,7 @@ __global__ void __launch_bounds__(kRelMaxConsumers + 32, 1) relevance_pass_kerne
                 if (lane == 0) qsum[warp] = qq;
                 consumer_sync();
                 qq = 0.f;
-                for (int w = 0; w < nw; ++w) qq += qsum[w];
+                for (int w = 0; w < nwg; ++w) qq += qsum[w];
                 qn = sqrtf(qq);
             }
 #pragma unroll
@@ -296,90 +309,108 @@ __global__ void __launch_bounds__(kRelMaxConsumers + 32, 1) relevance_pass_kerne
 #pragma unroll
                 for (int e = 0; e < NP; ++e) cs[0][vi][e] = cs[CSP - 1][vi][e] = 0ull;
         }
-        // this warp waits for the chunk itself (bounded)
-        int ok = 1;
-        if (lane == 0 && !dead) ok = ptx::mbar_wait(&full[s], ph, kRelTimeoutNs) ? 1 : 0;
-        ok = __shfl_sync(0xffffffffu, ok, 0);
-        if (!ok && !dead) {
-            dead = true;
-            if (lane == 0) {
-                abort_flag = 1;
-                atomicOr(c.status, 32);
+        if (turn == grp) {
+            // this warp waits for the chunk itself (bounded; one verdict per warp)
+            if (!dead && !__all_sync(0xffffffffu, ptx::mbar_wait(&full[s], ph, kRelTimeoutNs))) {
+                dead = true;
+                if (lane == 0) {
+                    abort_flag = 1;
+                    atomicOr(c.status, 32);
+                }
             }
-        }
-        const int nt = (int)n;
-        if (!dead) {
-            ptx::mbar_wait(&full[s], ph, kRelTimeoutNs);   // completed: acquire for this thread
-            const uint32_t st32 = ptx::smem_u32(rsm) + (uint32_t)(s * stage_bytes);
-            const uint32_t rowb32 = (uint32_t)rowb;
-            for (int g0 = 0; g0 < nt; g0 += GROUP) {
-                float acc[NV];
-                const bool full_group = nt - g0 >= GROUP;
+            if (!dead) {
+                float *const wp = wpart + buf * wbuf + gwarp * 2 * kRelWindow;
+                uint32_t row = ring + (uint32_t)s * stage_bytes;
+                for (int g0 = 0; g0 < n; g0 += GROUP) {
+                    float acc[NV];
+                    const int left = n - g0;
 #pragma unroll
-                for (int k = 0; k < GROUP; ++k) {
-                    f2_t dd = 0ull, nn = 0ull;
-                    if (full_group || g0 + k < nt) {
-                        const uint32_t row = st32 + (uint32_t)(g0 + k) * rowb32;
+                    for (int k = 0; k < GROUP; ++k) {
+                        f2_t dd = 0ull, nn = 0ull;
+                        if (k < left) {
 #pragma unroll
-                        for (int vi = 0; vi < VPT; ++vi) {
-                            const int vidx = threadIdx.x + vi * NC;
-                            if (vidx < n_vec) {
-                                const uint4 raw = ptx::lds128(row + (uint32_t)vidx * 16u);
-                                f2_t x[NP];
-                                unpack_pairs(raw, x, (T *)nullptr);
+                            for (int vi = 0; vi < VPT; ++vi) {
+                                if (gtid + vi * sh.gthreads < n_vec) {
+                                    const uint4 raw = ptx::lds128(row + (uint32_t)(vi * sh.gthreads) * 16u);
+                                    f2_t x[NP];
+                                    unpack_pairs(raw, x, (T *)nullptr);
 #pragma unroll
-                                for (int e = 0; e < NP; ++e) {
-                                    cs[k & (CSP - 1)][vi][e] = add2(cs[k & (CSP - 1)][vi][e], x[e]);
-                                    dd = fma2(x[e], q[vi][e], dd);
-                                    nn = fma2(x[e], x[e], nn);
+                                    for (int e = 0; e < NP; ++e) {
+                                        cs[k & (CSP - 1)][vi][e] = add2(cs[k & (CSP - 1)][vi][e], x[e]);
+                                        dd = fma2(x[e], q[vi][e], dd);
+                                        nn = fma2(x[e], x[e], nn);
+                                    }
                                 }
                             }
                         }
+                        row += rowb;
+                        const float2 d2 = unpack2(dd), n2 = unpack2(nn);
+                        acc[k] = d2.x + d2.y;
+                        acc[k + GROUP] = n2.x + n2.y;
                     }
-                    const float2 d2 = unpack2(dd), n2 = unpack2(nn);
-                    acc[k] = d2.x + d2.y;
-                    acc[k + GROUP] = n2.x + n2.y;
+                    const float tot = transpose_reduce<NV>(acc);
+                    const int kk = (lane >> 1) & (GROUP - 1);   // lane l holds value l >> 1: token kk, dot or norm
+                    if ((lane & 1) == 0 && kk < left) wp[(lane >> 4) * kRelWindow + wcount + g0 + kk] = tot;
                 }
-                const float tot = transpose_reduce<NV>(acc);
-                const int idx = lane >> SHIFT;              // value held by this lane
-                const int kk = idx & (GROUP - 1);
-                if ((lane & 1) == 0 && g0 + kk < nt)
-                    wpart[buf][warp][idx >> 3][wcount + g0 + kk] = tot;
             }
+            // hand the stage back once this warp's reads are done
+            __syncwarp();
+            if (lane == 0) ptx::mbar_arrive(&empty[s]);
         }
-        // hand the stage back once this warp's reads are done
-        __syncwarp();
-        if (lane == 0) ptx::mbar_arrive(&empty[s]);
-        if (++s == kRelStages) {
+        if (++turn == sh.groups) turn = 0;
+        if (++s == sh.stages) {
             s = 0;
             ph ^= 1u;
         }
         tok += n;
         pos += n;
-        wcount += nt;
-        const bool frame_done = pos == c.N || tok >= end;
-        if (frame_done && !dead &&
-            wz_in_range(c.status, (int64_t)blockIdx.x + (int64_t)f < (int64_t)c.G1 + (int64_t)c.V * c.T)) {
+        wcount += n;
+        if (pos == N || tok >= len) {
             // column partial of frame f from this CTA: slot blockIdx.x + f
-            float *dst = c.part + ((size_t)blockIdx.x + (size_t)f) * c.D;
+            if (CSP == 2)
 #pragma unroll
-            for (int vi = 0; vi < VPT; ++vi) {
-                const int vidx = threadIdx.x + vi * NC;
-                if (vidx < n_vec) {
+                for (int vi = 0; vi < VPT; ++vi)
 #pragma unroll
-                    for (int e = 0; e < NP; e += 2) {
-                        f2_t s0 = cs[0][vi][e], s1 = cs[0][vi][e + 1];
-                        if (CSP == 2) {
-                            s0 = add2(s0, cs[CSP - 1][vi][e]);
-                            s1 = add2(s1, cs[CSP - 1][vi][e + 1]);
+                    for (int e = 0; e < NP; ++e) cs[0][vi][e] = add2(cs[0][vi][e], cs[CSP - 1][vi][e]);
+            if (sh.groups > 1) {
+                if (csum_read) consumer_sync();
+                if (grp > 0) {
+#pragma unroll
+                    for (int vi = 0; vi < VPT; ++vi) {
+                        const int vidx = gtid + vi * sh.gthreads;
+                        if (vidx < n_vec) {
+                            float *dst = csum + (size_t)(grp - 1) * c.D + vidx * VEC;
+#pragma unroll
+                            for (int e = 0; e < NP; ++e) *reinterpret_cast<f2_t *>(dst + 2 * e) = cs[0][vi][e];
                         }
-                        const float2 a = unpack2(s0), b = unpack2(s1);
-                        *reinterpret_cast<float4 *>(dst + vidx * VEC + 2 * e) = make_float4(a.x, a.y, b.x, b.y);
+                    }
+                }
+                consumer_sync();
+                csum_read = true;
+            }
+            if (grp == 0 && !dead &&
+                wz_in_range(c.status, (int64_t)blockIdx.x + f < (int64_t)c.G1 + (int64_t)c.V * c.T)) {
+                float *dst = c.part + ((size_t)blockIdx.x + (size_t)f) * c.D;
+#pragma unroll
+                for (int vi = 0; vi < VPT; ++vi) {
+                    const int vidx = gtid + vi * sh.gthreads;
+                    if (vidx < n_vec) {
+                        for (int g = 0; g < sh.groups - 1; ++g) {
+                            const float *src = csum + (size_t)g * c.D + vidx * VEC;
+#pragma unroll
+                            for (int e = 0; e < NP; ++e)
+                                cs[0][vi][e] = add2(cs[0][vi][e], *reinterpret_cast<const f2_t *>(src + 2 * e));
+                        }
+#pragma unroll
+                        for (int e = 0; e < NP; e += 2) {
+                            const float2 a = unpack2(cs[0][vi][e]), b = unpack2(cs[0][vi][e + 1]);
+                            *reinterpret_cast<float4 *>(dst + vidx * VEC + 2 * e) = make_float4(a.x, a.y, b.x, b.y);
+                        }
                     }
                 }
             }
         }
-        if (pos == c.N) {
+        if (pos == N) {
             pos = 0;
             ++f;
             frame_new = true;
@@ -388,21 +419,21 @@ __global__ void __launch_bounds__(kRelMaxConsumers + 32, 1) relevance_pass_kerne
                 ++v;
             }
         }
-        // reduce the window across warps: when it is full, at the end of the
-        // range, and before a new video changes u_q
-        const bool new_video = tok < end && v != cur_v;
-        if (tok >= end || wcount + CH > WIN || new_video) {
+        // reduce the window across a group's warps: when it is full, at the end
+        // of the range, and before a new video changes u_q
+        if (tok >= len || wcount + CH > kRelWindow || v != cur_v) {
             consumer_sync();
-            if (abort_flag) break;
-            if (!wz_in_range(c.status, wbase + wcount <= total)) wcount = 0;
-            for (int t = threadIdx.x; t < wcount; t += NC) {
+            csum_read = false;   // group 0 arrived here after its reads
+            if (!wz_in_range(c.status, start + wbase + wcount <= total)) wcount = 0;
+            const float *w0 = wpart + buf * wbuf;
+            for (int t = threadIdx.x; t < wcount && !dead; t += NC) {
                 float dot = 0.f, nrm = 0.f;
-                for (int w = 0; w < nw; ++w) {
-                    dot += wpart[buf][w][0][t];
-                    nrm += wpart[buf][w][1][t];
+                for (int w = 0; w < nwg; ++w) {
+                    dot += w0[2 * w * kRelWindow + t];
+                    nrm += w0[(2 * w + 1) * kRelWindow + t];
                 }
-                c.a[wbase + t] = maxsim ? sqrtf(nrm)   // ||u||, divided out by the row-max GEMM
-                                        : (nrm > 0.f && qn > 0.f) ? dot / (sqrtf(nrm) * qn) : 0.f;
+                c.a[start + wbase + t] = maxsim ? sqrtf(nrm)   // ||u||, divided out by the row-max GEMM
+                                         : (nrm > 0.f && qn > 0.f) ? dot / (sqrtf(nrm) * qn) : 0.f;
             }
             buf ^= 1;
             wbase = tok;
@@ -706,23 +737,61 @@ namespace {
 struct RelCfg {
     const void *fn = nullptr;
     int threads = 0;     // consumers + one producer warp
-    int CH = 0;          // tokens per chunk
+    RelShape sh{};
     size_t smem = 0;
 };
 
+// Shape for one CTA per SM.  A row of w warps gets the most groups that fit 16
+// warps when those come to at least 15, else 24: too few warps leave the
+// shared-memory and barrier latencies exposed, more than needed cost
+// registers and barrier arrivals.  Whole wz_relevance calls on about 0.55 GB
+// (16 x 16 maps), one group / 16 / 24 warps: D = 512: 181 / 119 / 120 us;
+// 1152: 212 / 161 / 158; 2304: 146 / - / 122; 2816: 127 / - / 116; 3072 (12
+// warps a row): 120.3 / - / 120.1.  A thread holds at most 8 elements of a row
+// in groups of more than one.  CTAs of fewer than 64 tokens (short clips) stay
+// with one group: the groups' column sums cost more than they save there (16
+// frames of 13 x 13 x 896: 27 us with one group, 30 us with three).
 template <typename T, int VPT>
 void relevance_config(const Ctx &c, RelCfg &r) {
-    r.fn = (const void *)relevance_pass_kernel<T, VPT>;
     constexpr int VEC = VecOf<T>::kElems;
+    constexpr bool kNarrow = VPT * VEC <= 8;
     const int n_vec = c.D / VEC;
-    const int nc = std::max(32, ((n_vec + VPT - 1) / VPT + 31) / 32 * 32);
-    r.threads = nc + 32;
     const size_t rowb = (size_t)c.D * sizeof(T);
-    int ch = (int)std::max<size_t>(1, (56 * 1024) / rowb);
-    ch = std::min(ch, 32);
-    if (ch >= 8) ch = ch / 8 * 8;
-    r.CH = ch;
-    r.smem = (size_t)kRelStages * ch * rowb;
+    RelShape &sh = r.sh;
+    sh.gthreads = std::max(32, ((n_vec + VPT - 1) / VPT + 31) / 32 * 32);
+    const int w = sh.gthreads / 32;
+    sh.groups = 1;
+    if (kNarrow) sh.groups = std::max(1, (16 / w) * w >= 15 ? 16 / w : kRelMaxWarps / w);
+    const int64_t per_cta = ((int64_t)c.V * c.T * c.N + 151) / 152;
+    sh.groups = (int)std::min<int64_t>(sh.groups, std::max<int64_t>(1, per_cta / 32));
+    const size_t wpart = (size_t)2 * w * 2 * kRelWindow * 4;
+    size_t csum = 0, ring = 0;
+    for (; sh.groups > 1; --sh.groups) {
+        // chunks of 8 tokens (up to 32 and 8 KB: short rows), at least two
+        // stages per group
+        csum = (size_t)(sh.groups - 1) * c.D * 4;
+        ring = kRelSmem - wpart - csum;
+        sh.ch = 8 * (int)std::max<size_t>(1, std::min<size_t>(4, 8192 / (8 * rowb)));
+        sh.stages = (int)std::min<size_t>(kRelMaxStages, ring / (sh.ch * rowb)) / sh.groups * sh.groups;
+        if (sh.stages >= 2 * sh.groups) break;
+    }
+    if (sh.groups == 1) {   // three stages of up to 56 KB, 32 tokens
+        csum = 0;
+        ring = kRelSmem - wpart;
+        sh.ch = (int)std::max<size_t>(1, std::min<size_t>(32, std::min<size_t>(56 * 1024, ring / 3) / rowb));
+        if (sh.ch >= 8) sh.ch = sh.ch / 8 * 8;
+        sh.stages = 3;
+    }
+    const int cons = sh.groups * sh.gthreads;
+    r.threads = cons + 32;
+    if constexpr (kNarrow)
+        r.fn = cons <= 512 ? (const void *)relevance_pass_kernel<T, VPT, 512 + 32>
+                           : (const void *)relevance_pass_kernel<T, VPT, kRelMaxWarps * 32 + 32>;
+    else
+        r.fn = (const void *)relevance_pass_kernel<T, VPT, 512 + 32>;
+    sh.wpart_off = (int)(((size_t)sh.stages * sh.ch * rowb + 127) / 128 * 128);
+    sh.csum_off = sh.wpart_off + (int)wpart;
+    r.smem = (size_t)sh.csum_off + csum;
 }
 
 template <typename T>
@@ -765,8 +834,7 @@ cudaError_t launch_relevance_pass(const Ctx &c, cudaStream_t s) {
     if (!pick_any(c, r)) return cudaErrorInvalidValue;
     cudaError_t e = cudaFuncSetAttribute(r.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)r.smem);
     if (e != cudaSuccess) return e;
-    int CH = r.CH;
-    void *args[] = {const_cast<Ctx *>(&c), &CH};
+    void *args[] = {const_cast<Ctx *>(&c), &r.sh};
     return launch_kernel(r.fn, dim3(c.G1), dim3(r.threads), r.smem, s, args, c.pdl != 0);
 }
 
