@@ -775,10 +775,10 @@ void relevance_config(const Ctx &c, RelCfg &r) {
         sh.stages = (int)std::min<size_t>(kRelMaxStages, ring / (sh.ch * rowb)) / sh.groups * sh.groups;
         if (sh.stages >= 2 * sh.groups) break;
     }
-    if (sh.groups == 1) {   // three stages of up to 56 KB, 32 tokens
+    if (sh.groups == 1) {   // three stages of up to 8 tokens (32: short rows)
         csum = 0;
         ring = kRelSmem - wpart;
-        sh.ch = (int)std::max<size_t>(1, std::min<size_t>(32, std::min<size_t>(56 * 1024, ring / 3) / rowb));
+        sh.ch = (int)std::max<size_t>(1, std::min<size_t>(32, ring / 3 / rowb));
         if (sh.ch >= 8) sh.ch = sh.ch / 8 * 8;
         sh.stages = 3;
     }
