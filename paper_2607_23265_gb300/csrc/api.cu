@@ -372,36 +372,54 @@ int run_condense(const CondenseRequest &r) {
         return r.events ? cudaEventRecord((cudaEvent_t)r.events[k], r.stream) : cudaSuccess;
     };
     Nvtx whole("wz::condense");
+    // max-over-query scorer: one pass over the features computes the token
+    // norms, the channel sums and the token x query-row maxima where it applies
+    // and the videos' unit query rows have room: in their own buffer, in the
+    // partial slots past the ones in use, or in the operator's memory (written
+    // by the spatial kernel, later)
+    const bool maxsim = c.relevance_mode == WZ_RELEVANCE_MAXSIM;
+    const int Lq_max = *std::max_element(r.Lq.begin(), r.Lq.end()), Lqp_max = (Lq_max + 15) / 16 * 16;
+    bool fused_maxsim = false;
+    const int64_t qrows = qhl_row(qrow, r.V);   // rows of all videos
+    if (maxsim && maxsim_pass_supported(c, Lqp_max)) {
+        const size_t need = (size_t)qrows * s.D * 2;
+        const size_t used = align_up(((size_t)c.G1 + (size_t)s.V * s.T) * s.D * 4);
+        if (need <= (size_t)2 * WZ_MAX_LQ_MAXSIM * s.D * 2) fused_maxsim = true;
+        else if (L.part + used + need <= L.fr) {
+            c.qhl = reinterpret_cast<__nv_bfloat16 *>(ws.ptr + L.part + used);
+            fused_maxsim = true;
+        } else if (L.Wop + need <= L.total) {
+            c.qhl = reinterpret_cast<__nv_bfloat16 *>(ws.ptr + L.Wop);
+            fused_maxsim = true;
+        }
+    }
     WZ_CUDA(mark(2 * WZ_KERNEL_QUERY_POOL));
-    {
+    if (fused_maxsim) {   // needs no pooled query
+        Nvtx n_("wz::query_rows");
+        WZ_CUDA(launch_query_rows(c, par.data(), 0, r.V, Lqp_max, true, r.stream));
+    } else {
         Nvtx n_("wz::query_pool");
         WZ_CUDA(launch_query_pool(c, par.data(), r.stream));
     }
     WZ_CUDA(mark(2 * WZ_KERNEL_QUERY_POOL + 1));
-    // max-over-query scorer of one video: one pass over the features computes
-    // the token norms, the channel sums and the token x query-row maxima
-    const int Lqp0 = (r.Lq[0] + 15) / 16 * 16;
-    const bool fused_maxsim = c.relevance_mode == WZ_RELEVANCE_MAXSIM && maxsim_pass_supported(c, Lqp0);
+    WZ_CUDA(mark(2 * WZ_KERNEL_RELEVANCE));
     if (fused_maxsim) {
         Nvtx n_("wz::maxsim_pass");
-        WZ_CUDA(launch_query_rows(c, 0, par[0].q_row0, r.Lq[0], Lqp0, r.stream));
-        WZ_CUDA(mark(2 * WZ_KERNEL_RELEVANCE));
-        WZ_CUDA(launch_maxsim_pass(c, r.Lq[0], Lqp0, r.stream));
-        WZ_CUDA(mark(2 * WZ_KERNEL_RELEVANCE + 1));
+        WZ_CUDA(launch_maxsim_pass(c, Lqp_max, qrows, r.stream));
     } else {
-        WZ_CUDA(mark(2 * WZ_KERNEL_RELEVANCE));
         Nvtx n_("wz::relevance_pass");
         WZ_CUDA(launch_relevance_pass(c, r.stream));
-        WZ_CUDA(mark(2 * WZ_KERNEL_RELEVANCE + 1));
     }
-    if (c.relevance_mode == WZ_RELEVANCE_MAXSIM && !fused_maxsim) {
+    WZ_CUDA(mark(2 * WZ_KERNEL_RELEVANCE + 1));
+    if (maxsim && !fused_maxsim) {
         // the token x query-row cosines on the tensor cores, video by video
         // (the relevance pass left ||u|| in c.a)
         Nvtx n_("wz::maxsim");
         for (int v = 0; v < r.V; ++v) {
             const int Lq = r.Lq[v], Lqp = (Lq + 15) / 16 * 16;
             const int64_t tok = (int64_t)s.T * s.N;
-            WZ_CUDA(launch_query_rows(c, v, par[v].q_row0, Lq, Lqp, r.stream));
+            c.qhl_row0 = qhl_row(par[v].q_row0, v);
+            WZ_CUDA(launch_query_rows(c, par.data(), v, 1, Lqp, false, r.stream));
             WZ_CUDA(launch_maxsim_gemm(static_cast<const char *>(r.features) + (size_t)v * tok * s.D * 2, (int)tok,
                                        s.D, c.qhl, Lq, Lqp, c.a + v * tok, c.status, c.pdl != 0, r.stream));
         }

@@ -1,24 +1,27 @@
 // Max-over-query relevance in one pass over the features (the scorer of
-// reading R22 for a single video): the token x query-row cosines on the
+// reading R22): the token x query-row cosines on the
 // 5th-generation tensor cores, and, from the same shared-memory tiles, each
 // token's norm and the per-frame channel sums that the frame statistics
 // (r_t, delta_t; Section 3.2.1, Eq. 7) need.
 //
 //   a_{t,n} = max_{j < Lq} <u_{t,n}, q_j / ||q_j||> / ||u_{t,n}||
 //
-// Token tiles of 128 rows (M) x K steps of 64 channels: A = the features,
-// K-major with 128-byte swizzle; B = the unit query rows as bf16 hi rows then
-// lo rows (query_rows_kernel), N = 2 Lqp <= 256.  A stage holds G
-// consecutive K steps, loaded by one 3D TMA box ({64, 128, G} for the
-// features, {64, 2 Lqp, G} for the query rows): a token row arrives as G * 128
+// Token tiles of 128 rows (M; fewer at the end of a video or of the CTA's
+// range) x K steps of 64 channels: A = the features, K-major with 128-byte
+// swizzle; B = the unit query rows of the tile's video as bf16 hi rows then lo
+// rows (query_rows_kernel), N = 2 Lqp <= 256.  A feature stage holds G
+// consecutive K steps, a query-row stage as many as it has room for (gb(Lqp):
+// 1, 2 or 4, at most G), each loaded by one 3D TMA box ({64, 128, G} and {64,
+// 2 Lqp, gb}, one tensor map per Lqp): a token row arrives as G * 128
 // contiguous bytes per load, not 128, which keeps HBM reads efficient.  The
-// features and the query rows have rings of their own, so the query rows
-// (read from L2 for every tile) take two stages and the rest of shared memory
-// keeps feature reads in flight.  fp32 accumulators in tensor memory, two
-// buffers, so the epilogue of a tile overlaps the main loop of the next.
-// CTA c covers the tokens [c L1, (c+1) L1), exactly as the relevance pass
-// does, and writes its channel sums of every frame it touches into partial
-// slot c + t, so frame_stats_kernel reads them unchanged.
+// features and the query rows have rings of their own; the query rows (read
+// from L2 for every tile) take about kXBFlight bytes and the rest of shared
+// memory keeps feature reads in flight.  fp32 accumulators in tensor
+// memory, two buffers, so the epilogue of a tile overlaps the main loop of the
+// next.  CTA c covers the tokens [c L1, (c+1) L1) of the flattened [V*T*N]
+// index, exactly as the relevance pass does, and writes its channel sums of
+// every frame f it touches into partial slot c + f, where the frame statistics
+// expect them.
 //   warp 0       TMA producer of the features (one thread)
 //   warp 1       TMEM allocation and the MMA issuer (one thread)
 //   warps 2-9    channel sums and token norms: 4 channel pairs per warp, a
@@ -37,9 +40,16 @@
 //   warp 10      TMA producer of the query rows (one thread)
 // Every mbarrier wait is bounded; on a timeout the kernel records a status
 // bit, drains what it issued, frees tensor memory and exits.
+// HBM bound up to Lq = 64 (256 frames of 27 x 27 x 3584: 0.243 ms at Lq = 16,
+// 0.26 at 64), then by the query rows' L2 reads (0.306 at 128).  On 8 videos of
+// 64 frames of 13 x 13 x 3584 and 8 to 119 rows one pass takes 0.185 ms where
+// the relevance pass and one GEMM launch per video took 0.38; frame ends fall
+// inside most tiles there.  Measured and not taken: 16 channel-sum warps (0.196),
+// the sums in packed pairs (0.315), more query-row bytes in flight (0.19).
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
+#include <algorithm>
 #include <cstring>
 
 #include "wz_internal.cuh"
@@ -52,10 +62,13 @@ namespace {
 constexpr int kXM = 128, kXK = 64;
 constexpr int kXABytes = kXM * kXK * 2;             // 16 KB
 constexpr int kXMaxStages = 8;
-constexpr int kXGroups = 4;                         // K steps per ring stage (at most)
+constexpr int kXGroups = 4;                         // K steps per feature stage (at most)
 constexpr int kXMinStages = 2;
+constexpr int kXRowMaps = kXM / 32;                 // feature boxes: 32, 64, 96, 128 rows
+constexpr int kXMaps = WZ_MAX_LQ_MAXSIM / 16;       // query-row boxes: Lqp = 16, 32, ..
 constexpr int kXThreads = 11 * 32;
-constexpr int kXBStages = 2;                        // query-row stages (their own ring)
+constexpr int kXMaxBStages = 8;                     // query-row stages (their own ring)
+constexpr int kXBFlight = 64 * 1024;                // query-row bytes to keep in flight (L2 latency)
 constexpr int kXAccCols = 256;
 constexpr uint64_t kXTimeoutNs = 2000000000ull;
 constexpr int kXReaders = 8;                        // channel-sum warps reading each stage
@@ -63,8 +76,8 @@ constexpr int kXReaders = 8;                        // channel-sum warps reading
 struct XShared {
     uint64_t full[kXMaxStages];    // feature ring
     uint64_t empty[kXMaxStages];
-    uint64_t bfull[kXBStages];     // query-row ring
-    uint64_t bempty[kXBStages];
+    uint64_t bfull[kXMaxBStages];  // query-row ring
+    uint64_t bempty[kXMaxBStages];
     uint64_t tfull[2], tempty[2];
     uint64_t csync[2];
     uint64_t drain;
@@ -74,37 +87,68 @@ struct XShared {
 };
 
 struct XMaps {
-    CUtensorMap a, b;
+    CUtensorMap a[kXRowMaps];   // boxes of 32 (k + 1) token rows
+    CUtensorMap b[kXMaps];      // boxes of 2 Lqp rows, Lqp = 16 (k + 1)
 };
 
 struct XArgs {
-    int stages, stage_stride;   // feature ring: stages and bytes per stage (G A tiles)
-    int b_off, b_stride;        // query-row ring (kXBStages stages of G B tiles): byte offset, bytes per stage
-    int Lq, Lqp;
+    int stages, stage_stride;             // feature ring: stages and bytes per stage (G A tiles)
+    int bstages, b_off, b_stride;         // query-row ring: stages, byte offset, bytes per stage
     int acc_off;                // byte offset of the two channel-sum buffers (2 x D floats)
     int shared_off;             // byte offset of XShared
 };
+
+// K steps of 2 Lqp query rows in a stage of `bytes`, at most G.
+__host__ __device__ __forceinline__ int xgb(int Lqp, int bytes, int G) {
+    int gb = G;
+    while (gb > 1 && gb * 2 * Lqp * kXK * 2 > bytes) gb >>= 1;
+    return gb;
+}
 
 __device__ __forceinline__ void xfail(const Ctx &c, volatile int *abort_flag, int code) {
     *abort_flag = 1;
     atomicOr(c.status, code);
 }
 
-// Token tile `it` of this CTA: first token and valid rows.
-__device__ __forceinline__ void xtile(const Ctx &c, int it, int64_t &base, int &nr) {
-    const int64_t total = (int64_t)c.T * c.N;
-    const int64_t beg = (int64_t)blockIdx.x * c.L1;
-    const int64_t end = min(total, beg + c.L1);
-    base = beg + (int64_t)it * kXM;
-    nr = (int)min((int64_t)kXM, end - base);
-}
+// The token tiles of this CTA in order: at most 128 rows, none across a video.
+// A tile's feature boxes have its rows rounded up to 32; the rows past them in
+// shared memory are stale, and nothing reads the results of rows >= nr.
+struct XTile {
+    int64_t base, end, vend;   // first token; end of the CTA's range and of the video
+    int nr, v;                 // rows, video
+    int Lq, Lqp, qrow;         // the video's query rows: valid, padded to 16, first row of qhl
 
-__device__ __forceinline__ int xtiles(const Ctx &c) {
-    const int64_t total = (int64_t)c.T * c.N;
-    const int64_t beg = (int64_t)blockIdx.x * c.L1;
-    const int64_t end = min(total, beg + c.L1);
-    return beg < end ? (int)((end - beg + kXM - 1) / kXM) : 0;
-}
+    __device__ __forceinline__ int rows() const { return (nr + 31) & ~31; }
+    __device__ __forceinline__ void query(const Ctx &c) {
+        const VideoPar vp = c.vpar[v];
+        Lq = vp.Lq;
+        Lqp = (Lq + 15) & ~15;
+        qrow = qhl_row(vp.q_row0, v) - c.qhl_row0;
+    }
+    // the first tile; false when the CTA has no tokens
+    __device__ __forceinline__ bool first(const Ctx &c) {
+        const int64_t per = (int64_t)c.T * c.N, total = per * c.V;
+        base = (int64_t)blockIdx.x * c.L1;
+        end = min(total, base + c.L1);
+        if (base >= end) return false;
+        v = (int)(base / per);
+        vend = (v + 1) * per;
+        nr = (int)min((int64_t)kXM, min(end, vend) - base);
+        query(c);
+        return true;
+    }
+    __device__ __forceinline__ bool next(const Ctx &c) {
+        base += nr;
+        if (base >= end) return false;
+        if (base >= vend) {
+            ++v;
+            vend += (int64_t)c.T * c.N;
+            query(c);
+        }
+        nr = (int)min((int64_t)kXM, min(end, vend) - base);
+        return true;
+    }
+};
 
 // The channel sums of this warp's 8 channels of every K step (acc), to the
 // partial slot of frame f, then acc cleared: lane group lane / 8 takes every
@@ -113,14 +157,14 @@ __device__ __forceinline__ void xflush(const Ctx &c, float *acc, int64_t f, int 
     float *dst = c.part + ((size_t)blockIdx.x + (size_t)f) * c.D;
     for (int k0 = (lane >> 3) * kXK; k0 < c.D; k0 += 4 * kXK) {
         const int ch = k0 + ch_lo + (lane & 7);
-        if (wz_in_range(c.status, (int64_t)blockIdx.x + f < (int64_t)c.G1 + c.T)) dst[ch] = acc[ch];
+        if (wz_in_range(c.status, (int64_t)blockIdx.x + f < (int64_t)c.G1 + (int64_t)c.V * c.T)) dst[ch] = acc[ch];
         acc[ch] = 0.f;
     }
 }
 
 }  // namespace
 
-template <int G>   // K steps per ring stage
+template <int G>   // K steps per feature stage
 __global__ void __launch_bounds__(kXThreads, 1) maxsim_pass_kernel(const __grid_constant__ XMaps maps, Ctx c, XArgs p) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t *ring = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -135,7 +179,7 @@ __global__ void __launch_bounds__(kXThreads, 1) maxsim_pass_kernel(const __grid_
             ptx::mbar_init(&S->full[s], 1);
             ptx::mbar_init(&S->empty[s], 1 + kXReaders);
         }
-        for (int s = 0; s < kXBStages; ++s) {
+        for (int s = 0; s < p.bstages; ++s) {
             ptx::mbar_init(&S->bfull[s], 1);
             ptx::mbar_init(&S->bempty[s], 1);
         }
@@ -154,8 +198,7 @@ __global__ void __launch_bounds__(kXThreads, 1) maxsim_pass_kernel(const __grid_
         ptx::tmem_relinquish();
     }
     if (warp == 0 && lane == 0) {
-        ptx::prefetch_tmap(&maps.a);
-        ptx::prefetch_tmap(&maps.b);
+        ptx::prefetch_tmap(&maps.a[kXRowMaps - 1]);
     }
     // channel sums start at zero (shared memory only: before the wait)
     for (int k = threadIdx.x; k < 2 * c.D; k += blockDim.x) acc_buf[k] = 0.f;
@@ -164,21 +207,20 @@ __global__ void __launch_bounds__(kXThreads, 1) maxsim_pass_kernel(const __grid_
     __syncthreads();
     ptx::tc_fence_after();
     const uint32_t tmem = S->tmem_base;
-    const int ntile = xtiles(c);
+    XTile t;
+    const bool any = t.first(c);   // vpar is the previous grid's
     const int KS = c.D / kXK;
 
     if (warp == 0 && lane == 0) {
         // ---------------- TMA producer: features ----------------
         const uint64_t pol_a = ptx::policy_evict_first();
-        const uint32_t stage_bytes = (uint32_t)G * (uint32_t)kXABytes;
         int stage = 0;
         uint32_t phase = 0;
         int issued_parity[kXMaxStages];
         for (int s = 0; s < kXMaxStages; ++s) issued_parity[s] = -1;
-        for (int it = 0; it < ntile && !*abort_flag; ++it) {
-            int64_t base;
-            int nr;
-            xtile(c, it, base, nr);
+        for (bool on = any; on && !*abort_flag; on = t.next(c)) {
+            const CUtensorMap *map = &maps.a[(t.rows() >> 5) - 1];
+            const uint32_t stage_bytes = (uint32_t)(G * t.rows() * kXK * 2);
             bool ok = true;
             for (int ks = 0; ks < KS; ks += G) {
                 if (!ptx::mbar_wait(&S->empty[stage], phase ^ 1u, kXTimeoutNs)) {
@@ -188,7 +230,7 @@ __global__ void __launch_bounds__(kXThreads, 1) maxsim_pass_kernel(const __grid_
                 }
                 uint8_t *st = ring + (size_t)stage * p.stage_stride;
                 ptx::mbar_arrive_expect_tx(&S->full[stage], stage_bytes);
-                ptx::tma_load_3d(st, &maps.a, &S->full[stage], 0, (int)base, ks, pol_a);
+                ptx::tma_load_3d(st, map, &S->full[stage], 0, (int)t.base, ks, pol_a);
                 issued_parity[stage] = (int)phase;
                 if (++stage == p.stages) {
                     stage = 0;
@@ -202,43 +244,44 @@ __global__ void __launch_bounds__(kXThreads, 1) maxsim_pass_kernel(const __grid_
     } else if (warp == 10 && lane == 0) {
         // ---------------- TMA producer: query rows (from L2), K step by K step ----------------
         const uint64_t pol_b = ptx::policy_evict_last();
-        const uint32_t stage_bytes = (uint32_t)G * 2u * (uint32_t)p.Lqp * kXK * 2u;
         int stage = 0;
         uint32_t phase = 0;
-        int issued_parity[kXBStages];
-        for (int s = 0; s < kXBStages; ++s) issued_parity[s] = -1;
-        for (int it = 0; it < ntile && !*abort_flag; ++it) {
+        int issued_parity[kXMaxBStages];
+        for (int s = 0; s < kXMaxBStages; ++s) issued_parity[s] = -1;
+        for (bool on = any; on && !*abort_flag; on = t.next(c)) {
+            const int gb = xgb(t.Lqp, p.b_stride, G);
+            const uint32_t stage_bytes = (uint32_t)gb * 2u * (uint32_t)t.Lqp * kXK * 2u;
+            const CUtensorMap *map = &maps.b[(t.Lqp >> 4) - 1];
             bool ok = true;
-            for (int ks = 0; ks < KS; ks += G) {
+            for (int ks = 0; ks < KS; ks += gb) {
                 if (!ptx::mbar_wait(&S->bempty[stage], phase ^ 1u, kXTimeoutNs)) {
                     xfail(c, abort_flag, 16);
                     ok = false;
                     break;
                 }
                 ptx::mbar_arrive_expect_tx(&S->bfull[stage], stage_bytes);
-                ptx::tma_load_3d(ring + p.b_off + (size_t)stage * p.b_stride, &maps.b, &S->bfull[stage], 0, 0, ks,
+                ptx::tma_load_3d(ring + p.b_off + (size_t)stage * p.b_stride, map, &S->bfull[stage], 0, t.qrow, ks,
                                  pol_b);
                 issued_parity[stage] = (int)phase;
-                if (++stage == kXBStages) {
+                if (++stage == p.bstages) {
                     stage = 0;
                     phase ^= 1u;
                 }
             }
             if (!ok) break;
         }
-        for (int s = 0; s < kXBStages; ++s)
+        for (int s = 0; s < p.bstages; ++s)
             if (issued_parity[s] >= 0) ptx::mbar_wait(&S->bfull[s], (uint32_t)issued_parity[s], kXTimeoutNs);
     } else if (warp == 1 && lane == 0) {
         // ---------------- MMA issuer ----------------
-        const uint32_t idesc = ptx::idesc_bf16(kXM, 2 * p.Lqp, false, false);   // both K-major
         const uint32_t ring32 = ptx::smem_u32(ring);
         const uint64_t a_base = ptx::smem_desc(ring32, 16, 1024, 2);              // 128-B swizzle
         const uint64_t b_base = ptx::smem_desc(ring32 + (uint32_t)p.b_off, 16, 1024, 2);
-        const uint64_t b_sub = (uint64_t)((2 * p.Lqp * kXK * 2) >> 4);   // one K step of B
         const uint64_t stage_desc = (uint64_t)(p.stage_stride >> 4), bstage_desc = (uint64_t)(p.b_stride >> 4);
         int stage = 0, bstage = 0;
         uint32_t phase = 0, bphase = 0;
-        for (int it = 0; it < ntile && !*abort_flag; ++it) {
+        int it = 0;
+        for (bool on = any; on && !*abort_flag; on = t.next(c), ++it) {
             const int b = it & 1;
             const uint32_t use = (uint32_t)(it >> 1);
             if (!ptx::mbar_wait(&S->tempty[b], (use & 1u) ^ 1u, kXTimeoutNs)) {
@@ -247,33 +290,47 @@ __global__ void __launch_bounds__(kXThreads, 1) maxsim_pass_kernel(const __grid_
             }
             ptx::tc_fence_after();
             const uint32_t d = tmem + (uint32_t)(b * kXAccCols);
+            const uint32_t idesc = ptx::idesc_bf16(kXM, 2 * t.Lqp, false, false);   // both K-major
+            const uint64_t b_sub = (uint64_t)((2 * t.Lqp * kXK * 2) >> 4);          // one K step of B
+            const uint64_t a_sub = (uint64_t)((t.rows() * kXK * 2) >> 4);            // and of A
+            const int gb1 = xgb(t.Lqp, p.b_stride, G) - 1;
             bool ok = true;
-            for (int ks = 0; ks < KS; ks += G) {
-                if (!ptx::mbar_wait(&S->full[stage], phase, kXTimeoutNs) ||
-                    !ptx::mbar_wait(&S->bfull[bstage], bphase, kXTimeoutNs)) {
+            for (int ks = 0; ks < KS && ok; ks += G) {
+                if (!ptx::mbar_wait(&S->full[stage], phase, kXTimeoutNs)) {
                     xfail(c, abort_flag, 16);
                     ok = false;
                     break;
                 }
-                ptx::tc_fence_after();
-                const uint64_t so = (uint64_t)stage * stage_desc, sbo = (uint64_t)bstage * bstage_desc;
+                const uint64_t so = (uint64_t)stage * stage_desc;
 #pragma unroll
                 for (int g = 0; g < G; ++g) {
-                    const uint64_t ao = so + (uint64_t)g * (kXABytes >> 4), bo = sbo + (uint64_t)g * b_sub;
+                    if ((g & gb1) == 0) {
+                        if (!ptx::mbar_wait(&S->bfull[bstage], bphase, kXTimeoutNs)) {
+                            xfail(c, abort_flag, 16);
+                            ok = false;
+                            break;
+                        }
+                        ptx::tc_fence_after();
+                    }
+                    const uint64_t ao = so + (uint64_t)g * a_sub;
+                    const uint64_t bo = (uint64_t)bstage * bstage_desc + (uint64_t)(g & gb1) * b_sub;
 #pragma unroll
                     for (int k = 0; k < kXK / 16; ++k)   // K = 16 per MMA: 32 bytes along the swizzled row
                         ptx::mma_bf16(d, a_base + ao + (uint64_t)(2 * k), b_base + bo + (uint64_t)(2 * k), idesc,
                                       (ks | g | k) ? 1u : 0u);
+                    if ((g & gb1) == gb1) {
+                        ptx::mma_commit(&S->bempty[bstage]);
+                        if (++bstage == p.bstages) {
+                            bstage = 0;
+                            bphase ^= 1u;
+                        }
+                    }
                 }
+                if (!ok) break;
                 ptx::mma_commit(&S->empty[stage]);
-                ptx::mma_commit(&S->bempty[bstage]);
                 if (++stage == p.stages) {
                     stage = 0;
                     phase ^= 1u;
-                }
-                if (++bstage == kXBStages) {
-                    bstage = 0;
-                    bphase ^= 1u;
                 }
             }
             if (!ok) break;
@@ -296,14 +353,14 @@ __global__ void __launch_bounds__(kXThreads, 1) maxsim_pass_kernel(const __grid_
         const int cw = wsel * 8 + 2 * p4;               // channels cw, cw + 1 of the K step
         const uint32_t lane_off = (uint32_t)(re * 128) + ((uint32_t)(wsel ^ re) << 4) + (uint32_t)(4 * p4);
         float *acc_open = acc_buf, *acc_next = acc_buf + c.D;
-        int64_t open_f = ntile > 0 ? ((int64_t)blockIdx.x * c.L1) / c.N : 0;
+        int64_t open_f = any ? t.base / c.N : 0;
         bool open_has = false;
         int stage = 0;
         uint32_t phase = 0;
-        for (int it = 0; it < ntile && !*abort_flag; ++it) {
-            int64_t base;
-            int nr;
-            xtile(c, it, base, nr);
+        int it = 0;
+        for (bool on = any; on && !*abort_flag; on = t.next(c), ++it) {
+            const int64_t base = t.base;
+            const int nr = t.nr;
             // a frame starts inside the tile at row rb (frames have >= 128 tokens)
             const int to_end = (int)((int64_t)c.N - base % c.N);
             const int rb = to_end < nr ? to_end : nr;
@@ -311,6 +368,8 @@ __global__ void __launch_bounds__(kXThreads, 1) maxsim_pass_kernel(const __grid_
             float sq[16];                   // squares of this lane's two channels, row 8 i + re
 #pragma unroll
             for (int i = 0; i < 16; ++i) sq[i] = 0.f;
+            const int a_sub = t.rows() * kXK * 2;   // bytes of one K step
+            const int rbl = rb - re, nrl = nr - re;   // row 8 i + re below rb, nr: 8 i < rbl, nrl
             bool ok = true;
             for (int ks = 0; ks < KS; ks += G) {
                 if (!ptx::mbar_wait(&S->full[stage], phase, kXTimeoutNs)) {
@@ -322,14 +381,15 @@ __global__ void __launch_bounds__(kXThreads, 1) maxsim_pass_kernel(const __grid_
                 const uint8_t *st0 = smem_raw + ring_off + (size_t)stage * p.stage_stride;
 #pragma unroll
                 for (int g = 0; g < G; ++g) {
-                    const uint8_t *lb = st0 + g * kXABytes + lane_off;
+                    const uint8_t *lb = st0 + g * a_sub + lane_off;
+                    // s0 the open frame's rows, s1 the next's (whole tiles: even
+                    // and odd rows, shorter dependent chains)
                     float s0x = 0.f, s0y = 0.f, s1x = 0.f, s1y = 0.f;
                     if (whole) {
-                        // even and odd rows in two sums each (shorter dependent chains)
 #pragma unroll
                         for (int i = 0; i < 16; ++i) {
                             const uint32_t wv = *reinterpret_cast<const uint32_t *>(lb + 1024 * i);
-                            const float x = __uint_as_float(wv << 16), y = __uint_as_float(wv & 0xffff0000u);
+                            const float x = bf16_lo(wv), y = bf16_hi(wv);
                             sq[i] = fmaf(x, x, fmaf(y, y, sq[i]));
                             if (i & 1) {
                                 s1x += x;
@@ -345,14 +405,13 @@ __global__ void __launch_bounds__(kXThreads, 1) maxsim_pass_kernel(const __grid_
                     } else {
 #pragma unroll
                         for (int i = 0; i < 16; ++i) {
-                            const int r = 8 * i + re;
                             const uint32_t wv = *reinterpret_cast<const uint32_t *>(lb + 1024 * i);
-                            const float x = __uint_as_float(wv << 16), y = __uint_as_float(wv & 0xffff0000u);
+                            const float x = bf16_lo(wv), y = bf16_hi(wv);
                             sq[i] = fmaf(x, x, fmaf(y, y, sq[i]));
-                            if (r < rb) {
+                            if (8 * i < rbl) {
                                 s0x += x;
                                 s0y += y;
-                            } else if (r < nr) {
+                            } else if (8 * i < nrl) {
                                 s1x += x;
                                 s1y += y;
                             }
@@ -362,21 +421,20 @@ __global__ void __launch_bounds__(kXThreads, 1) maxsim_pass_kernel(const __grid_
                         __syncwarp();
                         if (lane == 0) ptx::mbar_arrive(&S->empty[stage]);
                     }
-#pragma unroll
-                    for (int o = 4; o < 32; o <<= 1) {   // the eight row classes, in a fixed order
-                        s0x += __shfl_xor_sync(0xffffffffu, s0x, o);
-                        s0y += __shfl_xor_sync(0xffffffffu, s0y, o);
-                        s1x += __shfl_xor_sync(0xffffffffu, s1x, o);
-                        s1y += __shfl_xor_sync(0xffffffffu, s1y, o);
-                    }
-                    if (re == 0) {
-                        const int ch = (ks + g) * kXK + cw;
-                        acc_open[ch] += s0x;
-                        acc_open[ch + 1] += s0y;
-                        if (rb < nr) {
-                            acc_next[ch] += s1x;
-                            acc_next[ch + 1] += s1y;
-                        }
+                    // the eight row classes (lane bits 2-4), in a fixed order:
+                    // the values are split over the lanes on the way, so that
+                    // lanes with bit 4 clear end with the open frame's sum and
+                    // those with it set with the next's, of channel cw (bit 3
+                    // clear) or cw + 1
+                    const bool up = (lane & 16) != 0, odd = (lane & 8) != 0;
+                    const float a = (up ? s1x : s0x) + __shfl_xor_sync(0xffffffffu, up ? s0x : s1x, 16);
+                    const float b = (up ? s1y : s0y) + __shfl_xor_sync(0xffffffffu, up ? s0y : s1y, 16);
+                    float r = (odd ? b : a) + __shfl_xor_sync(0xffffffffu, odd ? a : b, 8);
+                    r += __shfl_xor_sync(0xffffffffu, r, 4);
+                    const int ch = (ks + g) * kXK + cw + (odd ? 1 : 0);
+                    if ((lane & 4) == 0 && (!up || rb < nr)) {
+                        float *dst = up ? acc_next : acc_open;
+                        dst[ch] += r;
                     }
                 }
                 if (++stage == p.stages) {
@@ -389,6 +447,12 @@ __global__ void __launch_bounds__(kXThreads, 1) maxsim_pass_kernel(const __grid_
             // one partial per warp and row
             const int b = it & 1;
             const uint32_t use = (uint32_t)(it >> 1);
+            // the rows' partials of the tile before the last have been read
+            // (tiles of few stages let some warps run two tiles ahead)
+            if (!ptx::mbar_wait(&S->tempty[b], (use & 1u) ^ 1u, kXTimeoutNs)) {
+                xfail(c, abort_flag, 32);
+                break;
+            }
 #pragma unroll
             for (int i = 0; i < 16; ++i) {
                 float v = sq[i];
@@ -401,9 +465,9 @@ __global__ void __launch_bounds__(kXThreads, 1) maxsim_pass_kernel(const __grid_
             open_has = true;
             if (rb < nr) {   // the open frame ended inside the tile
                 xflush(c, acc_open, open_f, wsel * 8, lane);
-                float *t = acc_open;
+                float *other = acc_open;
                 acc_open = acc_next;
-                acc_next = t;
+                acc_next = other;
                 ++open_f;
             }
             if ((base + nr) % c.N == 0) {   // and the frame open now ends with the tile
@@ -431,18 +495,18 @@ __global__ void __launch_bounds__(kXThreads, 1) maxsim_pass_kernel(const __grid_
                 const float nrm = sqrtf(t2);
                 const uint32_t tbase = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * kXAccCols);
                 float best = -INFINITY;
-                for (int c0 = 0; c0 < p.Lqp; c0 += 16) {
+                for (int c0 = 0; c0 < t.Lqp; c0 += 16) {
                     uint32_t hi[16], lo[16];
                     ptx::tmem_ld_32x32b_x16(tbase + (uint32_t)c0, hi);
-                    ptx::tmem_ld_32x32b_x16(tbase + (uint32_t)(p.Lqp + c0), lo);
+                    ptx::tmem_ld_32x32b_x16(tbase + (uint32_t)(t.Lqp + c0), lo);
                     ptx::tmem_ld_wait();
                     ptx::reg_fence16(hi);
                     ptx::reg_fence16(lo);
 #pragma unroll
                     for (int j = 0; j < 16; ++j)
-                        if (c0 + j < p.Lq) best = fmaxf(best, __uint_as_float(hi[j]) + __uint_as_float(lo[j]));
+                        if (c0 + j < t.Lq) best = fmaxf(best, __uint_as_float(hi[j]) + __uint_as_float(lo[j]));
                 }
-                if (row < nr && wz_in_range(c.status, base + row < (int64_t)c.T * c.N))
+                if (row < nr && wz_in_range(c.status, base + row < (int64_t)c.V * c.T * c.N))
                     c.a[base + row] = nrm > 0.f ? best / nrm : 0.f;
                 ptx::tc_fence_before();
                 __syncwarp();
@@ -474,29 +538,34 @@ bool xencode(PFN_cuTensorMapEncodeTiled_v12000 enc, CUtensorMap *m, const void *
 }
 
 struct XLayout {
-    int stages, stride, G, b_off, b_stride, acc_off, shared_off;
+    int stages, stride, G, bstages, b_off, b_stride, acc_off, shared_off;
     size_t smem;
 };
 
-// K steps per stage: the most of kXGroups (dividing the D / 64 K steps)
-// that leaves kXMinStages feature stages beside the kXBStages query-row
-// stages.
+// K steps per feature stage (G, at most kXGroups, dividing the D / 64 K
+// steps), the longest reads first, such that kXMinStages feature stages fit
+// beside two query-row stages of one K step of the longest query; then the
+// query-row stages up to kXBFlight bytes (of gb K steps where two such stages
+// fit), then the rest to feature stages.
 XLayout xlayout(int D, int Lqp) {
     XLayout L{};
     const size_t fixed = 1024 + (size_t)2 * D * 4 + (sizeof(XShared) + 127) / 128 * 128;
-    const size_t cap = 227 * 1024;
-    for (int G = kXGroups; G >= 1; G >>= 1) {
-        if ((D / kXK) % G != 0) continue;
-        L.G = G;
-        L.stride = G * kXABytes;
-        L.b_stride = G * 2 * Lqp * kXK * 2;   // multiples of 1 KB (2 Lqp % 16 == 0)
-        const size_t used = fixed + (size_t)kXBStages * L.b_stride;
-        L.stages = used < cap ? (int)((cap - used) / (size_t)L.stride) : 0;
-        if (L.stages >= kXMinStages) break;
+    const int room = (int)((size_t)227 * 1024 - fixed);
+    const int step = 2 * Lqp * kXK * 2;   // one K step of query rows: a multiple of 4 KB
+    for (L.G = kXGroups; L.G >= 1; L.G >>= 1) {
+        if ((D / kXK) % L.G != 0) continue;
+        L.stride = L.G * kXABytes;
+        const int left = room - kXMinStages * L.stride;   // for query rows
+        if (left < 2 * step) continue;
+        int gb = L.G;
+        while (gb > 1 && 2 * gb * step > std::min(left, kXBFlight)) gb >>= 1;
+        L.b_stride = gb * step;
+        L.bstages = std::max(2, std::min(std::min(left, kXBFlight) / L.b_stride, kXMaxBStages));
+        L.stages = std::min((room - L.bstages * L.b_stride) / L.stride, kXMaxStages);
+        break;
     }
-    if (L.stages > kXMaxStages) L.stages = kXMaxStages;
     L.b_off = L.stages * L.stride;
-    L.acc_off = L.b_off + kXBStages * L.b_stride;
+    L.acc_off = L.b_off + L.bstages * L.b_stride;
     L.shared_off = L.acc_off + 2 * D * 4;
     L.smem = 1024 + (size_t)L.shared_off + sizeof(XShared);
     return L;
@@ -504,31 +573,35 @@ XLayout xlayout(int D, int Lqp) {
 
 }  // namespace
 
-// The fused pass applies to one video with frames of at least 128 tokens,
-// D a multiple of 64 up to 4096 and at most 128 query rows (Lqp <= 128).
+// The fused pass applies to frames of at least 128 tokens, D a multiple of 64
+// up to 4096 and at most 128 query rows per video (Lqp <= 128: the longest
+// query, padded to 16).
 bool maxsim_pass_supported(const Ctx &c, int Lqp) {
-    if (c.V != 1 || c.N < kXM || c.D % kXK != 0 || c.D > 4096 || c.dtype != WZ_DTYPE_BF16) return false;
-    if (Lqp < 16 || Lqp > 128 || Lqp % 16 != 0) return false;
-    return xlayout(c.D, Lqp).stages >= 2;
+    if (c.N < kXM || c.D % kXK != 0 || c.D > 4096 || c.dtype != WZ_DTYPE_BF16) return false;
+    if ((int64_t)c.V * c.T * c.N > (int64_t)INT32_MAX) return false;   // token coordinates of the tensor map
+    if (Lqp < 16 || Lqp > WZ_MAX_LQ_MAXSIM || Lqp % 16 != 0) return false;
+    return xlayout(c.D, Lqp).stages >= kXMinStages;
 }
 
-cudaError_t launch_maxsim_pass(const Ctx &c, int Lq, int Lqp, cudaStream_t s) {
-    if (!maxsim_pass_supported(c, Lqp) || Lq < 1 || Lq > Lqp) return cudaErrorInvalidValue;
+// Lqp: the longest query's padded rows; c.qhl holds qrows rows in all.
+cudaError_t launch_maxsim_pass(const Ctx &c, int Lqp, int64_t qrows, cudaStream_t s) {
+    if (!maxsim_pass_supported(c, Lqp)) return cudaErrorInvalidValue;
     auto enc = tmap_encode_fn();
     if (!enc) return cudaErrorNotSupported;
     XMaps maps;
     memset(&maps, 0, sizeof(maps));
     const XLayout L = xlayout(c.D, Lqp);
-    if (!xencode(enc, &maps.a, c.X, (int64_t)c.T * c.N, c.D, kXM, L.G) ||
-        !xencode(enc, &maps.b, c.qhl, 2 * Lqp, c.D, 2 * Lqp, L.G))
-        return cudaErrorInvalidValue;
+    for (int k = 0; k < kXRowMaps; ++k)
+        if (!xencode(enc, &maps.a[k], c.X, (int64_t)c.V * c.T * c.N, c.D, 32 * (k + 1), L.G)) return cudaErrorInvalidValue;
+    for (int k = 0; k < Lqp / 16; ++k)
+        if (!xencode(enc, &maps.b[k], c.qhl, qrows, c.D, 32 * (k + 1), xgb(16 * (k + 1), L.b_stride, L.G)))
+            return cudaErrorInvalidValue;
     XArgs p{};
     p.stages = L.stages;
     p.stage_stride = L.stride;
+    p.bstages = L.bstages;
     p.b_off = L.b_off;
     p.b_stride = L.b_stride;
-    p.Lq = Lq;
-    p.Lqp = Lqp;
     p.acc_off = L.acc_off;
     p.shared_off = L.shared_off;
     const void *fn = L.G == 4 ? (const void *)maxsim_pass_kernel<4>

@@ -29,27 +29,33 @@
 
 namespace wz {
 
+// The videos' parameters in the kernel arguments, in blocks of a few sizes: a
+// launch copies its whole argument block (20 KB at WZ_MAX_VIDEOS).
+template <int N>
 struct VideoParBlock {
-    VideoPar v[WZ_MAX_VIDEOS];
+    VideoPar v[N];
 };
+
+// What every kernel after the first one reads of video v.
+__device__ __forceinline__ void video_init(const Ctx &c, int v, const VideoPar &vp) {
+    c.vpar[v] = vp;
+    if (c.drange) {   // empty range of delta_t, filled by frame_stats
+        c.drange[2 * v] = 0x7ff0000000000000ull;   // +inf
+        c.drange[2 * v + 1] = 0ull;                // +0
+    }
+}
 
 // u_q = mean of the query rows: a block covers 32 channels with 8 row
 // slices; compensated fp32 sums (TwoSum) per slice, combined in a fixed
 // order, stored as fp64 and fp32.
-template <typename T>
-__global__ void __launch_bounds__(256) query_pool_kernel(Ctx c, VideoParBlock par) {
+template <typename T, int NPAR>
+__global__ void __launch_bounds__(256) query_pool_kernel(Ctx c, VideoParBlock<NPAR> par) {
     __shared__ float ps[8][32], pe[8][32];
     pdl_wait();
     pdl_trigger();
     const int v = blockIdx.y;
     const VideoPar vp = par.v[v];
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        c.vpar[v] = vp;
-        if (c.drange) {   // empty range of delta_t, filled by frame_stats
-            c.drange[2 * v] = 0x7ff0000000000000ull;   // +inf
-            c.drange[2 * v + 1] = 0ull;                // +0
-        }
-    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) video_init(c, v, vp);
     const int cl = threadIdx.x & 31, slice = threadIdx.x >> 5;
     const int d = blockIdx.x * 32 + cl;
     float s = 0.f, e = 0.f;
@@ -91,41 +97,74 @@ __global__ void __launch_bounds__(256) query_pool_kernel(Ctx c, VideoParBlock pa
     }
 }
 
-// Query rows of video v for the max-over-query scorer: block j < Lq writes
-// ||q_j|| (fp64 sum of fp32 squares) to qnorm and q_j / ||q_j|| as bf16 hi
-// (row j of qhl) and lo = bf16(x - hi) (row Lqp + j); blocks Lq <= j < Lqp
-// write zero rows, so the GEMM's padding columns are zero.  bf16 rows.
-__global__ void __launch_bounds__(256) query_rows_kernel(Ctx c, int v, int q_row0, int Lq, int Lqp) {
+// Unit query rows for the max-over-query scorer, blockIdx.y = video v0 + y:
+// block j < Lq writes ||q_j|| (fp64 sum of fp32 squares) to qnorm and q_j /
+// ||q_j|| as bf16 hi (row j of the video's rows in qhl, see qhl_row) and lo =
+// bf16(x - hi) (row Lqp + j); blocks Lq <= j < Lqp write zero rows, so the
+// GEMM's padding columns are zero.  bf16 rows, D % 64 == 0, read as 16-byte
+// vectors and kept in registers between the two passes (the first kQRowKeep
+// per thread).  With init != 0 the kernel is the first of the call.
+constexpr int kQRowKeep = 2;
+
+template <int NPAR>
+__global__ void __launch_bounds__(256) query_rows_kernel(Ctx c, VideoParBlock<NPAR> par, int v0, int init) {
     __shared__ double red[33];
     pdl_wait();
     pdl_trigger();
-    const int j = blockIdx.x;
-    const int D = c.D;
-    __nv_bfloat16 *hi = c.qhl + (size_t)j * D;
-    __nv_bfloat16 *lo = c.qhl + (size_t)(Lqp + j) * D;
-    const __nv_bfloat16 zero = __float2bfloat16_rn(0.f);
-    if (j >= Lq) {
-        for (int d = threadIdx.x; d < D; d += blockDim.x) {
-            hi[d] = zero;
-            lo[d] = zero;
-        }
+    const int v = v0 + (int)blockIdx.y, j = blockIdx.x;
+    const VideoPar vp = par.v[blockIdx.y];
+    if (init && j == 0 && threadIdx.x == 0) video_init(c, v, vp);
+    const int Lqp = (vp.Lq + 15) & ~15;
+    if (j >= Lqp) return;
+    const int n8 = c.D / 8;
+    uint4 *hi = reinterpret_cast<uint4 *>(c.qhl + (size_t)(qhl_row(vp.q_row0, v) - c.qhl_row0 + j) * c.D);
+    uint4 *lo = hi + (size_t)Lqp * n8;
+    if (j >= vp.Lq) {
+        for (int i = threadIdx.x; i < n8; i += 256) hi[i] = lo[i] = make_uint4(0u, 0u, 0u, 0u);
         return;
     }
-    const __nv_bfloat16 *q = static_cast<const __nv_bfloat16 *>(c.Q) + (size_t)(q_row0 + j) * D;
+    const uint4 *q = reinterpret_cast<const uint4 *>(static_cast<const __nv_bfloat16 *>(c.Q) +
+                                                     (size_t)(vp.q_row0 + j) * c.D);
+    uint4 keep[kQRowKeep];
     float ss = 0.f;
-    for (int d = threadIdx.x; d < D; d += blockDim.x) {
-        const float x = __bfloat162float(q[d]);
-        ss = fmaf(x, x, ss);
+    auto square = [&](const uint4 &w) {
+        float x[8];
+        unpack(w, x, (__nv_bfloat16 *)nullptr);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) ss = fmaf(x[e], x[e], ss);
+    };
+#pragma unroll
+    for (int k = 0; k < kQRowKeep; ++k) {
+        const int i = (int)threadIdx.x + 256 * k;
+        keep[k] = i < n8 ? q[i] : make_uint4(0u, 0u, 0u, 0u);
     }
+#pragma unroll
+    for (int k = 0; k < kQRowKeep; ++k) square(keep[k]);
+    for (int i = (int)threadIdx.x + 256 * kQRowKeep; i < n8; i += 256) square(q[i]);
     const double qn = sqrt(block_sum((double)ss, red));
     if (threadIdx.x == 0) c.qnorm[(size_t)v * WZ_MAX_LQ_MAXSIM + j] = (float)qn;
     const float inv = qn > 0.0 ? (float)(1.0 / qn) : 0.f;
-    for (int d = threadIdx.x; d < D; d += blockDim.x) {
-        const float x = __bfloat162float(q[d]) * inv;
-        const __nv_bfloat16 h = __float2bfloat16_rn(x);
-        hi[d] = h;
-        lo[d] = __float2bfloat16_rn(x - __bfloat162float(h));
+    auto split = [&](int i, const uint4 &w) {
+        float x[8];
+        unpack(w, x, (__nv_bfloat16 *)nullptr);
+        uint32_t h[4], l[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const float x0 = x[2 * e] * inv, x1 = x[2 * e + 1] * inv;
+            const __nv_bfloat162 hh = __floats2bfloat162_rn(x0, x1);
+            const __nv_bfloat162 ll = __floats2bfloat162_rn(x0 - __low2float(hh), x1 - __high2float(hh));
+            h[e] = *reinterpret_cast<const uint32_t *>(&hh);
+            l[e] = *reinterpret_cast<const uint32_t *>(&ll);
+        }
+        hi[i] = make_uint4(h[0], h[1], h[2], h[3]);
+        lo[i] = make_uint4(l[0], l[1], l[2], l[3]);
+    };
+#pragma unroll
+    for (int k = 0; k < kQRowKeep; ++k) {
+        const int i = (int)threadIdx.x + 256 * k;
+        if (i < n8) split(i, keep[k]);
     }
+    for (int i = (int)threadIdx.x + 256 * kQRowKeep; i < n8; i += 256) split(i, q[i]);
 }
 
 // Reduce the NV values held by every lane across the warp (NV a power of
@@ -444,74 +483,11 @@ __global__ void __launch_bounds__(MAXTHREADS, 1) relevance_pass_kernel(Ctx c, Re
 
 // Gate of the WSM for frame f (Eq. 6, Eq. 12): the saliency map M = min-max
 // normalised a_{t,n} over the frame, average-pooled to the subband grid of
-// each DWT level (hp x wp for the first) and scaled by lambda.  `red` is >= 32
-// floats of shared scratch.
-constexpr int kGatePerThread = WZ_MAX_HW * WZ_MAX_HW / 512;   // a_{t,n} per thread of a 512-thread block
-
-// The frame's a_{t,n} (an external scorer's if given), this thread's share
-// k = threadIdx.x + 512 r, loaded into registers early so that the loads
-// overlap the frame statistics.
-__device__ __forceinline__ void gate_prefetch(const Ctx &c, int64_t f, float (&av)[kGatePerThread]) {
-    const float *a = (c.ext_a ? c.ext_a : c.a) + f * c.N;
-#pragma unroll
-    for (int r = 0; r < kGatePerThread; ++r) {
-        const int k = (int)threadIdx.x + 512 * r;
-        av[r] = k < c.N ? a[k] : 0.f;
-    }
-}
-
-__device__ void frame_gate(const Ctx &c, int64_t f, float *red, const float (&av)[kGatePerThread], float *M) {
-    const int N = c.N, H = c.H, W = c.W;
-    float lo = INFINITY, hi = -INFINITY;
-#pragma unroll
-    for (int r = 0; r < kGatePerThread; ++r) {
-        const int k = (int)threadIdx.x + 512 * r;
-        if (k < N) {
-            M[k] = av[r];
-            lo = fminf(lo, av[r]);
-            hi = fmaxf(hi, av[r]);
-        }
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-        lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
-        hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
-    }
-    __syncthreads();   // red is free (the caller's reads are done)
-    if ((threadIdx.x & 31) == 0) {
-        red[threadIdx.x >> 5] = lo;
-        red[16 + (threadIdx.x >> 5)] = hi;
-    }
-    __syncthreads();
-    lo = INFINITY;
-    hi = -INFINITY;
-    for (int k = 0; k < (int)(blockDim.x >> 5); ++k) {
-        lo = fminf(lo, red[k]);
-        hi = fmaxf(hi, red[16 + k]);
-    }
-    const float rng = hi - lo;
-    for (int k = threadIdx.x; k < N; k += blockDim.x) M[k] = rng > 0.f ? (M[k] - lo) / rng : 0.f;
-    __syncthreads();
-    for (int l = 1; l <= c.wsm_levels; ++l) {
-        const int hp = c.lvl_h[l], wp = c.lvl_w[l];
-        if (!wz_in_range(c.status, c.goff[l - 1] + hp * wp <= c.gate_stride)) break;
-        float *G = c.gate + f * (int64_t)c.gate_stride + c.goff[l - 1];
-        for (int k = threadIdx.x; k < hp * wp; k += blockDim.x) {
-            const int ai = k / wp, bj = k % wp;
-            const int r0 = (ai * H) / hp, r1 = ((ai + 1) * H + hp - 1) / hp;
-            const int c0 = (bj * W) / wp, c1 = ((bj + 1) * W + wp - 1) / wp;
-            float s = 0.f;
-            for (int y = r0; y < r1; ++y)
-                for (int x = c0; x < c1; ++x) s += M[y * W + x];
-            G[k] = c.lambda * (s / (float)((r1 - r0) * (c1 - c0)));
-        }
-    }
-}
-
-// The gate of frame f (as frame_gate) formed by the upper half of
-// frame_stats_kernel's threads (t0 = threadIdx.x - nth, named barrier 2 over
-// nth threads) while the lower half forms the frame statistics: the two
-// chains overlap.
-__device__ void gate_half(const Ctx &c, int64_t f, int t0, int nth, float *M2) {
+// each DWT level (hp x wp for the first) and scaled by lambda.  Formed by nth
+// threads of the block (t0 = 0 .. nth - 1, named barrier 2): half of
+// frame_stats_kernel's, while the other half forms the frame statistics, so
+// the two chains overlap, or a whole CTA's.
+__device__ void frame_gate(const Ctx &c, int64_t f, int t0, int nth, float *M2) {
     __shared__ float red2[32];
     auto sync = [nth] { asm volatile("bar.sync 2, %0;" ::"r"(nth) : "memory"); };
     const int N = c.N, H = c.H, W = c.W, lane = t0 & 31, w = t0 >> 5, nw = nth >> 5;
@@ -557,38 +533,47 @@ __device__ void gate_half(const Ctx &c, int64_t f, int t0, int nth, float *M2) {
     }
 }
 
+// r_t and delta_t of frame f = (v, t), from <v_t,v_t>, <v_t,v_{t-1}>,
+// <v_{t-1},v_{t-1}> (one thread).
+__device__ __forceinline__ void frame_result(const Ctx &c, int64_t f, int v, int t, double r, double vv, double vp,
+                                             double pp) {
+    if (c.ext_r) r = (double)c.ext_r[f];   // an external scorer's r_t
+    double d = 0.0;
+    if (t > 0) {
+        const double den = sqrt(vv * pp);
+        const double cs = den > 0.0 ? vp / den : 0.0;
+        d = fmin(2.0, fmax(0.0, 1.0 - cs)) + 0.0;   // + 0.0: never -0
+    }
+    c.fr[4 * f + 0] = r;
+    c.fr[4 * f + 1] = d;
+    if (c.drange) {   // non-negative doubles order like their bit patterns
+        const unsigned long long bits = (unsigned long long)__double_as_longlong(d);
+        atomicMin(&c.drange[2 * v], bits);
+        atomicMax(&c.drange[2 * v + 1], bits);
+    }
+    if (c.frame_scores) c.frame_scores[f] = (float)r;
+}
+
 // One block per frame: the frame sums (fixed list of CTA partials) for all
 // channels, read as 16-byte vectors; fp32 products summed over each thread's
 // channels and across each warp, the warp totals in fp64; then
 // r_t = cos(v_bar_t, u_q) and delta_t = 1 - cos(v_bar_t, v_bar_{t-1})
 // clamped to [0, 2] (Eq. 7) in fp64.
-//
-// With the max-over-query scorer the frame sums are kept in shared memory
-// (D floats of dynamic shared memory) and every warp takes query rows j:
-// <v_t, q_j> in fp32 (as the per-warp partials of the mean scorer), divided
-// by ||q_j|| in fp64; r_t = max_j of that / ||v_t||.
 __global__ void __launch_bounds__(512) frame_stats_kernel(Ctx c) {
     pdl_wait();
     pdl_trigger();
     __shared__ float wsum[16][5];
-    __shared__ double wmax[16];
-    __shared__ float gate_map[WZ_MAX_HW * WZ_MAX_HW];   // the frame's saliency map (either gate form)
-    extern __shared__ float4 sfs[];   // [D/4] frame sums (max-over-query scorer only)
-    const bool maxsim = c.relevance_mode == WZ_RELEVANCE_MAXSIM;
-    const bool do_gate = c.gate && c.spatial_mode == WZ_SPATIAL_WSM;
+    __shared__ float gate_map[WZ_MAX_HW * WZ_MAX_HW];   // the frame's saliency map
     const int64_t f = blockIdx.x;
-    // with the mean scorer, the upper half of the threads forms the gate
-    // while the lower half forms the statistics; the max-over-query scorer
-    // takes every warp for its query rows and forms the gate after them
-    const bool split = !maxsim && do_gate;
+    // the upper half of the threads forms the gate (where there is one) while
+    // the lower half forms the statistics
+    const bool split = c.gate && c.spatial_mode == WZ_SPATIAL_WSM;
     const int half = (int)blockDim.x / 2;
     if (split && (int)threadIdx.x >= half) {
-        gate_half(c, f, (int)threadIdx.x - half, half, gate_map);
+        frame_gate(c, f, (int)threadIdx.x - half, half, gate_map);
         return;
     }
     const int nst = split ? half : (int)blockDim.x;   // threads forming the statistics
-    float av[kGatePerThread];
-    if (do_gate && !split) gate_prefetch(c, f, av);
     const int t = (int)(f % c.T);
     const int v = (int)(f / c.T);
     const int64_t lo = f * c.N / c.L1;
@@ -615,7 +600,6 @@ __global__ void __launch_bounds__(512) frame_stats_kernel(Ctx c) {
             if (cc + 1 <= hi2) { sp.x += y.x; sp.y += y.y; sp.z += y.z; sp.w += y.w; }
         }
         const float4 q = Qv[i];
-        if (maxsim) sfs[i] = sf;
         if (c.frame_mean) {   // caller's buffer: 4-byte alignment only
             float *fm = c.frame_mean + (size_t)f * c.D + 4 * i;
             fm[0] = sf.x / (float)c.N;
@@ -637,43 +621,6 @@ __global__ void __launch_bounds__(512) frame_stats_kernel(Ctx c) {
         p4 += __shfl_xor_sync(0xffffffffu, p4, o);
     }
     const int warp = threadIdx.x >> 5, nw = nst >> 5;
-    if (maxsim) {
-        __syncthreads();   // sfs complete
-        const int lane = threadIdx.x & 31;
-        const VideoPar vp = c.vpar[v];
-        const int n8 = c.D / 8;
-        double best = -INFINITY;
-        const int rot = (int)(f % vp.Lq);   // frames start on different rows: no hot L2 lines
-        for (int jr = warp; jr < vp.Lq; jr += nw) {
-            const int j = jr + rot < vp.Lq ? jr + rot : jr + rot - vp.Lq;
-            const uint4 *qr = reinterpret_cast<const uint4 *>(static_cast<const __nv_bfloat16 *>(c.Q) +
-                                                              (size_t)(vp.q_row0 + j) * c.D);
-            float acc = 0.f;
-            for (int i0 = lane; i0 < n8; i0 += 32 * 8) {   // 8 loads in flight per lane (L2 latency)
-                uint4 qv[8];
-#pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    const int i = i0 + 32 * u;
-                    qv[u] = i < n8 ? __ldg(qr + i) : make_uint4(0u, 0u, 0u, 0u);
-                }
-#pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    const int i = i0 + 32 * u;
-                    if (i < n8) {
-                        float qf[8];
-                        unpack(qv[u], qf, (__nv_bfloat16 *)nullptr);
-                        const float4 s0 = sfs[2 * i], s1 = sfs[2 * i + 1];
-                        acc = fmaf(s0.x, qf[0], fmaf(s0.y, qf[1], fmaf(s0.z, qf[2], fmaf(s0.w, qf[3],
-                              fmaf(s1.x, qf[4], fmaf(s1.y, qf[5], fmaf(s1.z, qf[6], fmaf(s1.w, qf[7], acc))))))));
-                    }
-                }
-            }
-            for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-            const double qn = (double)c.qnorm[(size_t)v * WZ_MAX_LQ_MAXSIM + j];
-            best = fmax(best, qn > 0.0 ? (double)acc / qn : 0.0);
-        }
-        if (lane == 0) wmax[warp] = best;
-    }
     if ((threadIdx.x & 31) == 0) {
         wsum[warp][0] = p0;
         wsum[warp][1] = p1;
@@ -695,41 +642,209 @@ __global__ void __launch_bounds__(512) frame_stats_kernel(Ctx c) {
         const double pp = __shfl_sync(0xffffffffu, acc, 4);
         if (lane == 0) {
             const double qn = sqrt(qq);
-            double r = (vv > 0.0 && qn > 0.0) ? vq / (sqrt(vv) * qn) : 0.0;
-            if (maxsim) {
-                double best = -INFINITY;
-                for (int w = 0; w < nw; ++w) best = fmax(best, wmax[w]);
-                r = vv > 0.0 ? best / sqrt(vv) : 0.0;
-            }
-            if (c.ext_r) r = (double)c.ext_r[f];   // an external scorer's r_t
-            double d = 0.0;
-            if (t > 0) {
-                const double den = sqrt(vv * pp);
-                const double cs = den > 0.0 ? vp / den : 0.0;
-                d = fmin(2.0, fmax(0.0, 1.0 - cs)) + 0.0;   // + 0.0: never -0
-            }
-            c.fr[4 * f + 0] = r;
-            c.fr[4 * f + 1] = d;
-            if (c.drange) {   // non-negative doubles order like their bit patterns
-                const unsigned long long bits = (unsigned long long)__double_as_longlong(d);
-                atomicMin(&c.drange[2 * v], bits);
-                atomicMax(&c.drange[2 * v + 1], bits);
-            }
-            if (c.frame_scores) c.frame_scores[f] = (float)r;
+            frame_result(c, f, v, t, (vv > 0.0 && qn > 0.0) ? vq / (sqrt(vv) * qn) : 0.0, vv, vp, pp);
         }
     }
-    if (do_gate && !split) frame_gate(c, f, wsum[0], av, gate_map);
 }
 
-cudaError_t launch_query_pool(const Ctx &c, const VideoPar *hpar, cudaStream_t s) {
-    VideoParBlock blk;   // copied into the launch parameters
+// The max-over-query scorer's frame statistics: a CTA takes FPB consecutive
+// frames of one video (ceil(T / FPB) CTAs per video), whose sums stay in shared
+// memory ([FPB][D] floats); r_t = max_j <v_t, q_j> / ||q_j|| / ||v_t|| over the
+// video's query rows: every thread takes 16-byte vectors of the channels,
+// kRowBatch rows at a time (a row is read once for the FPB frames), the rows'
+// partial dots are reduced across the warp by one transpose-reduction, and the
+// warps' partials are added in a tree.  The gates are formed by further CTAs
+// (one per frame) beside them.  Bound by the latency of its steps and by
+// reading the query rows from L2 in every CTA (Lq D bf16 each): 512 frames of
+// 13 x 13 x 3584 and 8 to 119 rows (events around the kernel): 77 us with one
+// frame per CTA, a warp per row and the gate after the dots, 36 us now.
+constexpr int kRowBatch = 8;
+constexpr int kStatsThreads = 256;   // of a maxsim statistics CTA; two per SM
+
+template <int FPB>
+__global__ void __launch_bounds__(kStatsThreads, 2) frame_stats_maxsim_kernel(Ctx c) {
+    constexpr int NW = kStatsThreads / 32;
+    pdl_wait();
+    pdl_trigger();
+    __shared__ float wsum[FPB][NW][3];                       // vv, v.v_prev, v_prev.v_prev
+    __shared__ float part[FPB][NW][WZ_MAX_LQ_MAXSIM];        // per warp: <v_f, q_j>
+    __shared__ double best[FPB][4];
+    __shared__ float gate_map[WZ_MAX_HW * WZ_MAX_HW];
+    extern __shared__ float4 sfs[];   // [FPB][D/4] frame sums
+    const int per_video = (c.T + FPB - 1) / FPB, nstat = c.V * per_video;
+    if ((int)blockIdx.x >= nstat) {
+        frame_gate(c, (int64_t)blockIdx.x - nstat, threadIdx.x, kStatsThreads, gate_map);
+        return;
+    }
+    const int v = (int)blockIdx.x / per_video, t0 = ((int)blockIdx.x - v * per_video) * FPB;
+    const int nf = min(FPB, c.T - t0);
+    const int64_t f0 = (int64_t)v * c.T + t0;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const VideoPar par = c.vpar[v];
+    const int nv = c.D / 4;
+    const float4 *P = reinterpret_cast<const float4 *>(c.part);
+    // the column partials of frame f0 - 1 + k: slots [lo, lo + n)
+    int64_t slot[FPB + 1];
+    int cnt[FPB + 1];
+#pragma unroll
+    for (int k = 0; k <= FPB; ++k) {
+        const int64_t f = f0 - 1 + k;
+        const bool on = (k > 0 || t0 > 0) && k <= nf;
+        const int64_t lo = on ? f * c.N / c.L1 : 0;
+        slot[k] = lo + f;
+        cnt[k] = on ? (int)(min((int64_t)c.G1 - 1, ((f + 1) * c.N - 1) / c.L1) - lo) + 1 : 0;
+    }
+    auto dot4 = [](const float4 &a, const float4 &b, float s) {
+        return fmaf(a.x, b.x, fmaf(a.y, b.y, fmaf(a.z, b.z, fmaf(a.w, b.w, s))));
+    };
+    float vv[FPB], vp[FPB], pp[FPB];
+#pragma unroll
+    for (int k = 0; k < FPB; ++k) vv[k] = vp[k] = pp[k] = 0.f;
+    for (int i = threadIdx.x; i < nv; i += kStatsThreads) {
+        float4 sf[FPB + 1];
+#pragma unroll
+        for (int k = 0; k <= FPB; ++k) {
+            sf[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+            for (int q = 0; q < cnt[k]; q += 2) {   // two partial rows in flight, summed in order
+                const float4 x = P[(size_t)(slot[k] + q) * nv + i];
+                const float4 y = q + 1 < cnt[k] ? P[(size_t)(slot[k] + q + 1) * nv + i] : make_float4(0.f, 0.f, 0.f, 0.f);
+                sf[k].x += x.x; sf[k].y += x.y; sf[k].z += x.z; sf[k].w += x.w;
+                if (q + 1 < cnt[k]) { sf[k].x += y.x; sf[k].y += y.y; sf[k].z += y.z; sf[k].w += y.w; }
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < FPB; ++k) {
+            sfs[k * nv + i] = sf[k + 1];
+            vv[k] = dot4(sf[k + 1], sf[k + 1], vv[k]);
+            vp[k] = dot4(sf[k + 1], sf[k], vp[k]);
+            pp[k] = dot4(sf[k], sf[k], pp[k]);
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < FPB; ++k) {
+        for (int o = 16; o > 0; o >>= 1) {
+            vv[k] += __shfl_xor_sync(0xffffffffu, vv[k], o);
+            vp[k] += __shfl_xor_sync(0xffffffffu, vp[k], o);
+            pp[k] += __shfl_xor_sync(0xffffffffu, pp[k], o);
+        }
+        if (lane == 0) {
+            wsum[k][warp][0] = vv[k];
+            wsum[k][warp][1] = vp[k];
+            wsum[k][warp][2] = pp[k];
+        }
+    }
+    __syncthreads();   // sfs complete
+    const int n8 = c.D / 8;
+    const uint4 *Qr = reinterpret_cast<const uint4 *>(static_cast<const __nv_bfloat16 *>(c.Q) + (size_t)par.q_row0 * c.D);
+    // CTAs start on different rows: no hot L2 lines
+    const int nbatch = (par.Lq + kRowBatch - 1) / kRowBatch, rot = (int)(blockIdx.x % nbatch);
+    for (int bi = 0; bi < nbatch; ++bi) {
+        const int j0 = (bi + rot < nbatch ? bi + rot : bi + rot - nbatch) * kRowBatch;
+        float acc[FPB][kRowBatch];
+#pragma unroll
+        for (int k = 0; k < FPB; ++k)
+#pragma unroll
+            for (int u = 0; u < kRowBatch; ++u) acc[k][u] = 0.f;
+        for (int i = threadIdx.x; i < n8; i += kStatsThreads) {
+            uint4 qv[kRowBatch];
+#pragma unroll
+            for (int u = 0; u < kRowBatch; ++u)
+                qv[u] = j0 + u < par.Lq ? __ldg(Qr + (size_t)(j0 + u) * n8 + i) : make_uint4(0u, 0u, 0u, 0u);
+            float4 s[FPB][2];
+#pragma unroll
+            for (int k = 0; k < FPB; ++k) {
+                s[k][0] = sfs[k * nv + 2 * i];
+                s[k][1] = sfs[k * nv + 2 * i + 1];
+            }
+#pragma unroll
+            for (int u = 0; u < kRowBatch; ++u) {
+                float q[8];
+                unpack(qv[u], q, (__nv_bfloat16 *)nullptr);
+#pragma unroll
+                for (int k = 0; k < FPB; ++k)
+                    acc[k][u] = dot4(s[k][0], make_float4(q[0], q[1], q[2], q[3]),
+                                     dot4(s[k][1], make_float4(q[4], q[5], q[6], q[7]), acc[k][u]));
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < FPB; ++k) {
+            const float tot = transpose_reduce<kRowBatch>(acc[k]);   // lane l holds row l >> 2
+            if ((lane & 3) == 0) part[k][warp][j0 + (lane >> 2)] = tot;
+        }
+    }
+    __syncthreads();
+    // the dots with row j over the warps, over ||q_j||; 128 rows of a frame per
+    // four warps
+    static_assert(WZ_MAX_LQ_MAXSIM == 128 && NW == 8, "two frames per round");
+#pragma unroll
+    for (int k0 = 0; k0 < FPB; k0 += 2) {
+        const int k = k0 + (int)(threadIdx.x >> 7), j = threadIdx.x & 127;
+        if (k < FPB) {
+            double x = -INFINITY;
+            if (k < nf && j < par.Lq) {
+                const double qn = (double)c.qnorm[(size_t)v * WZ_MAX_LQ_MAXSIM + j];
+                const float d = ((part[k][0][j] + part[k][1][j]) + (part[k][2][j] + part[k][3][j])) +
+                                ((part[k][4][j] + part[k][5][j]) + (part[k][6][j] + part[k][7][j]));
+                x = qn > 0.0 ? (double)d / qn : 0.0;
+            }
+            for (int o = 16; o > 0; o >>= 1) x = fmax(x, __shfl_xor_sync(0xffffffffu, x, o));
+            if (lane == 0) best[k][warp & 3] = x;
+        }
+    }
+    __syncthreads();
+    if (warp < nf) {   // a warp per frame: lane q < 3 sums quantity q over the warps
+        double acc = 0.0;
+        if (lane < 3)
+            for (int w = 0; w < NW; ++w) acc += (double)wsum[warp][w][lane];
+        const double s0 = __shfl_sync(0xffffffffu, acc, 0), s1 = __shfl_sync(0xffffffffu, acc, 1);
+        const double s2 = __shfl_sync(0xffffffffu, acc, 2);
+        if (lane == 0) {
+            const double m = fmax(fmax(best[warp][0], best[warp][1]), fmax(best[warp][2], best[warp][3]));
+            frame_result(c, f0 + warp, v, t0 + warp, s0 > 0.0 ? m / sqrt(s0) : 0.0, s0, s1, s2);
+        }
+    }
+}
+
+namespace {
+
+template <int N>
+VideoParBlock<N> par_block(const VideoPar *hpar, int n) {
+    VideoParBlock<N> blk;
     memset(&blk, 0, sizeof(blk));
-    for (int v = 0; v < c.V; ++v) blk.v[v] = hpar[v];
+    for (int v = 0; v < n; ++v) blk.v[v] = hpar[v];
+    return blk;
+}
+
+template <int N>
+cudaError_t query_pool_n(const Ctx &c, const VideoPar *hpar, cudaStream_t s) {
+    VideoParBlock<N> blk = par_block<N>(hpar, c.V);   // copied into the launch parameters
     const dim3 grid((unsigned)((c.D + 31) / 32), (unsigned)c.V);
     void *args[] = {const_cast<Ctx *>(&c), &blk};
-    const void *fn = c.dtype == WZ_DTYPE_BF16 ? (const void *)query_pool_kernel<__nv_bfloat16>
-                                              : (const void *)query_pool_kernel<float>;
+    const void *fn = c.dtype == WZ_DTYPE_BF16 ? (const void *)query_pool_kernel<__nv_bfloat16, N>
+                                              : (const void *)query_pool_kernel<float, N>;
     return launch_kernel(fn, grid, dim3(256), 0, s, args, c.pdl != 0);
+}
+
+template <int N>
+cudaError_t query_rows_n(const Ctx &c, const VideoPar *hpar, int v0, int nv, int Lqp, int init, cudaStream_t s) {
+    VideoParBlock<N> blk = par_block<N>(hpar + v0, nv);
+    void *args[] = {const_cast<Ctx *>(&c), &blk, &v0, &init};
+    return launch_kernel((const void *)query_rows_kernel<N>, dim3((unsigned)Lqp, (unsigned)nv), dim3(256), 0, s, args,
+                         c.pdl != 0);
+}
+
+}  // namespace
+
+cudaError_t launch_query_pool(const Ctx &c, const VideoPar *hpar, cudaStream_t s) {
+    return c.V == 1 ? query_pool_n<1>(c, hpar, s)
+           : c.V <= 32 ? query_pool_n<32>(c, hpar, s) : query_pool_n<WZ_MAX_VIDEOS>(c, hpar, s);
+}
+
+// Videos v0 .. v0 + nv - 1; Lqp: the longest of their queries, padded to 16.
+cudaError_t launch_query_rows(const Ctx &c, const VideoPar *hpar, int v0, int nv, int Lqp, bool init, cudaStream_t s) {
+    return nv == 1 ? query_rows_n<1>(c, hpar, v0, nv, Lqp, init, s)
+           : nv <= 32 ? query_rows_n<32>(c, hpar, v0, nv, Lqp, init, s)
+                      : query_rows_n<WZ_MAX_VIDEOS>(c, hpar, v0, nv, Lqp, init, s);
 }
 
 namespace {
@@ -840,27 +955,30 @@ cudaError_t launch_relevance_pass(const Ctx &c, cudaStream_t s) {
 
 cudaError_t launch_frame_stats(const Ctx &c, cudaStream_t s) {
     void *args[] = {const_cast<Ctx *>(&c)};
-    const size_t smem = c.relevance_mode == WZ_RELEVANCE_MAXSIM ? (size_t)c.D * 4 : 0;
-    if (smem > 0) {
-        const cudaError_t e =
-            cudaFuncSetAttribute((const void *)frame_stats_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
-    // 512 threads a frame (4 CTAs per SM); with the mean scorer's split form
-    // and more frames than one wave of those, 256 (twice the CTAs in flight)
-    const bool split = c.relevance_mode != WZ_RELEVANCE_MAXSIM && c.gate && c.spatial_mode == WZ_SPATIAL_WSM;
     int dev = 0, sms = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
+    if (c.relevance_mode == WZ_RELEVANCE_MAXSIM) {
+        // frames share a CTA's reads of the query rows once every SM has work
+        // without that (and their sums fit)
+        const int64_t frames = (int64_t)c.V * c.T;
+        const int fpb = frames > 4 * (int64_t)sms && c.D <= 8192 ? 4 : frames > sms && c.D <= 16384 ? 2 : 1;
+        const size_t smem = (size_t)fpb * c.D * 4;
+        const void *fn = fpb == 4 ? (const void *)frame_stats_maxsim_kernel<4>
+                         : fpb == 2 ? (const void *)frame_stats_maxsim_kernel<2>
+                                    : (const void *)frame_stats_maxsim_kernel<1>;
+        e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        const int gates = c.gate && c.spatial_mode == WZ_SPATIAL_WSM ? c.V * c.T : 0;
+        return launch_kernel(fn, dim3(c.V * ((c.T + fpb - 1) / fpb) + gates), dim3(kStatsThreads), smem, s, args,
+                             c.pdl != 0);
+    }
+    // 512 threads a frame (4 CTAs per SM); with the gate's split form and more
+    // frames than one wave of those, 256 (twice the CTAs in flight)
+    const bool split = c.gate && c.spatial_mode == WZ_SPATIAL_WSM;
     const int threads = split && (int64_t)c.V * c.T > 4 * (int64_t)sms ? 256 : 512;
-    return launch_kernel((const void *)frame_stats_kernel, dim3(c.V * c.T), dim3(threads), smem, s, args,
-                         c.pdl != 0);
-}
-
-cudaError_t launch_query_rows(const Ctx &c, int v, int q_row0, int Lq, int Lqp, cudaStream_t s) {
-    void *args[] = {const_cast<Ctx *>(&c), &v, &q_row0, &Lq, &Lqp};
-    return launch_kernel((const void *)query_rows_kernel, dim3((unsigned)Lqp), dim3(256), 0, s, args, c.pdl != 0);
+    return launch_kernel((const void *)frame_stats_kernel, dim3(c.V * c.T), dim3(threads), 0, s, args, c.pdl != 0);
 }
 
 }  // namespace wz

@@ -91,7 +91,8 @@ struct Ctx {
     const float *ext_r;   // [V*T] external frame scores, or null
     int relevance_mode;   // WZ_RELEVANCE_*
     float *qnorm;         // [V][WZ_MAX_LQ_MAXSIM] query row norms (max-over-query scorer)
-    __nv_bfloat16 *qhl;   // [2 WZ_MAX_LQ_MAXSIM][D] normalised rows, bf16 hi then lo (one video at a time)
+    __nv_bfloat16 *qhl;   // unit query rows [..][D], per video bf16 hi then lo rows at qhl_row() - qhl_row0
+    int qhl_row0;
     int wta_levels;       // WTA decomposition levels (1 = the paper's single level)
     int wsm_levels;       // WSM decomposition levels
     int gate_stride;      // floats of c.gate per frame: sum over levels of lvl_h * lvl_w
@@ -102,6 +103,11 @@ struct Ctx {
     int wta_F;            // WTA filter taps (temporal DWT, fp64)
     double wta_dec_lo[kMaxTaps], wta_dec_hi[kMaxTaps], wta_rec_lo[kMaxTaps], wta_rec_hi[kMaxTaps];
 };
+
+// First row of video v's unit query rows (2 Lqp of them, Lqp = Lq rounded up to
+// 16) among the videos' in order; q_row0: its first query row.  Linear in what
+// precedes it, and spaced by at least 2 Lqp.
+__host__ __device__ __forceinline__ int qhl_row(int q_row0, int v) { return 2 * ((q_row0 + 15 * v) & ~15); }
 
 // ---- device helpers -------------------------------------------------------
 
@@ -363,14 +369,14 @@ cudaError_t launch_spatial_ml(const Ctx &c, cudaStream_t s);
 size_t spatial_ml_smem_bytes(int H, int W, int F, int J);   // 0 if the layout does not fit
 cudaError_t launch_project_gemm(const void *A, int M, int K, const void *B, int N, const float *bias, void *out,
                                 bool gelu, int *status, bool pdl, cudaStream_t s);
-// Max-over-query relevance of one video in one pass over the features
-// (maxsim.cu): token norms, channel-sum partials and a_{t,n}, in place of the
-// relevance pass and the max-over-query GEMM.
+// Max-over-query relevance in one pass over the features (maxsim.cu): token
+// norms, channel-sum partials and a_{t,n}, in place of the relevance pass and
+// the max-over-query GEMM.
 bool maxsim_pass_supported(const Ctx &c, int Lqp);
-cudaError_t launch_maxsim_pass(const Ctx &c, int Lq, int Lqp, cudaStream_t s);
+cudaError_t launch_maxsim_pass(const Ctx &c, int Lqp, int64_t qrows, cudaStream_t s);
 cudaError_t launch_maxsim_gemm(const void *X, int M, int K, const void *QHL, int Lq, int Lqp, float *a, int *status,
                                bool pdl, cudaStream_t s);
-cudaError_t launch_query_rows(const Ctx &c, int v, int q_row0, int Lq, int Lqp, cudaStream_t s);
+cudaError_t launch_query_rows(const Ctx &c, const VideoPar *hpar, int v0, int nv, int Lqp, bool init, cudaStream_t s);
 cudaError_t launch_condense_simt(const Ctx &c, cudaStream_t s);
 cudaError_t launch_condense_tc(const Ctx &c, cudaStream_t s);
 int relevance_grid(const Ctx &c);   // CTAs for the relevance pass on this device
