@@ -159,11 +159,11 @@ constexpr int kCompactFrames = 2048;   // frames whose work prefix a spatial CTA
 // pre[f] = sum of count(f') over the frames f' < f, pre[F] = the total
 // (F <= kCompactFrames; a block-wide scan, every thread a contiguous range of
 // frames).  The caller synchronises the block before reading pre.
-template <class Count>
+template <int NT = kSpatialThreads, class Count>   // NT: threads of the block; wsum: one int per warp
 __device__ void frame_prefix(int F, int *pre, int *wsum, Count count) {
-    constexpr int kPer = kCompactFrames / kSpatialThreads;
+    constexpr int kPer = kCompactFrames / NT;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int per = (F + kSpatialThreads - 1) / kSpatialThreads;
+    const int per = (F + NT - 1) / NT;
     const int f0 = tid * per;
     int cnt[kPer];
     int sum = 0;
@@ -188,7 +188,7 @@ __device__ void frame_prefix(int F, int *pre, int *wsum, Count count) {
     }
     if (tid == 0) {
         int tot = 0;
-        for (int w = 0; w < kSpatialThreads / 32; ++w) tot += wsum[w];
+        for (int w = 0; w < NT / 32; ++w) tot += wsum[w];
         pre[F] = tot;
     }
 }
