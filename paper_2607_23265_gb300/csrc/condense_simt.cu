@@ -5,11 +5,11 @@
 // TM output rows of a frame x TN channels from a static list (the prefix of
 // the frames' row blocks in shared memory), K in steps of 32 tokens through a
 // ring of kSimtStages cp.async stages; a thread forms RT rows x 4 CG columns,
-// products in f32x2 (column pairs), every output one chain in ascending K.  Bound by latency for
-// few frames and by the FMA pipe (43 of 75 TFLOP/s) for many.  Before, with one
-// unpipelined 16-token step at a time, 64 x 64 tiles and a grid over every
-// possible tile: 64 frames of 13 x 13 x 3584 96 us, 64 of 27 x 27 x 2048 1.07 ms
-// (0.81 now).
+// products in f32x2 (column pairs), every output one chain in ascending K.
+// Bound by latency for few frames and by the FMA pipe (43 of 75 TFLOP/s) for
+// many.  Before, with one unpipelined 16-token step at a time, 64 x 64 tiles
+// and a grid over every possible tile: 64 frames of 13 x 13 x 3584 96 us (57
+// now), 64 of 27 x 27 x 2048 1.07 ms (0.81 now).
 #include <algorithm>
 
 #include "wz_spatial.cuh"

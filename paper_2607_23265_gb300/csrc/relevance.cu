@@ -483,13 +483,12 @@ __global__ void __launch_bounds__(MAXTHREADS, 1) relevance_pass_kernel(Ctx c, Re
 
 // Gate of the WSM for frame f (Eq. 6, Eq. 12): the saliency map M = min-max
 // normalised a_{t,n} over the frame, average-pooled to the subband grid of
-// each DWT level (hp x wp for the first) and scaled by lambda.  Formed by nth
-// threads of the block (t0 = 0 .. nth - 1, named barrier 2): half of
-// frame_stats_kernel's, while the other half forms the frame statistics, so
-// the two chains overlap, or a whole CTA's.
-__device__ void frame_gate(const Ctx &c, int64_t f, int t0, int nth, float *M2) {
+// each DWT level (hp x wp for the first) and scaled by lambda.  Called by a
+// whole CTA beside those that form the frame statistics, so that the two chains
+// overlap.
+__device__ void frame_gate(const Ctx &c, int64_t f, float *M2) {
+    const int t0 = threadIdx.x, nth = blockDim.x;
     __shared__ float red2[32];
-    auto sync = [nth] { asm volatile("bar.sync 2, %0;" ::"r"(nth) : "memory"); };
     const int N = c.N, H = c.H, W = c.W, lane = t0 & 31, w = t0 >> 5, nw = nth >> 5;
     const float *a = (c.ext_a ? c.ext_a : c.a) + f * N;
     float lo = INFINITY, hi = -INFINITY;
@@ -507,7 +506,7 @@ __device__ void frame_gate(const Ctx &c, int64_t f, int t0, int nth, float *M2) 
         red2[w] = lo;
         red2[16 + w] = hi;
     }
-    sync();
+    __syncthreads();
     lo = INFINITY;
     hi = -INFINITY;
     for (int k = 0; k < nw; ++k) {
@@ -516,7 +515,7 @@ __device__ void frame_gate(const Ctx &c, int64_t f, int t0, int nth, float *M2) 
     }
     const float rng = hi - lo;
     for (int k = t0; k < N; k += nth) M2[k] = rng > 0.f ? (M2[k] - lo) / rng : 0.f;
-    sync();
+    __syncthreads();
     for (int l = 1; l <= c.wsm_levels; ++l) {
         const int hp = c.lvl_h[l], wp = c.lvl_w[l];
         if (!wz_in_range(c.status, c.goff[l - 1] + hp * wp <= c.gate_stride)) break;
@@ -533,73 +532,91 @@ __device__ void frame_gate(const Ctx &c, int64_t f, int t0, int nth, float *M2) 
     }
 }
 
-// r_t and delta_t of frame f = (v, t), from <v_t,v_t>, <v_t,v_{t-1}>,
-// <v_{t-1},v_{t-1}> (one thread).
-__device__ __forceinline__ void frame_result(const Ctx &c, int64_t f, int v, int t, double r, double vv, double vp,
-                                             double pp) {
-    if (c.ext_r) r = (double)c.ext_r[f];   // an external scorer's r_t
-    double d = 0.0;
-    if (t > 0) {
-        const double den = sqrt(vv * pp);
-        const double cs = den > 0.0 ? vp / den : 0.0;
-        d = fmin(2.0, fmax(0.0, 1.0 - cs)) + 0.0;   // + 0.0: never -0
+// The column partials of frame f: slots [slot, slot + cnt) (CTA c of the
+// relevance pass holds its tokens [c L1, (c+1) L1) of frame f in slot c + f).
+__device__ __forceinline__ void frame_slots(const Ctx &c, int64_t f, int64_t &slot, int &cnt) {
+    const int64_t n0 = f * c.N, n1 = n0 + c.N - 1;
+    int64_t lo, hi;
+    if (n1 <= (int64_t)UINT32_MAX && c.L1 <= (int64_t)UINT32_MAX) {   // 32-bit divisions
+        lo = (uint32_t)n0 / (uint32_t)c.L1;
+        hi = (uint32_t)n1 / (uint32_t)c.L1;
+    } else {
+        lo = n0 / c.L1;
+        hi = n1 / c.L1;
     }
-    c.fr[4 * f + 0] = r;
-    c.fr[4 * f + 1] = d;
-    if (c.drange) {   // non-negative doubles order like their bit patterns
-        const unsigned long long bits = (unsigned long long)__double_as_longlong(d);
-        atomicMin(&c.drange[2 * v], bits);
-        atomicMax(&c.drange[2 * v + 1], bits);
-    }
-    if (c.frame_scores) c.frame_scores[f] = (float)r;
+    slot = lo + f;
+    cnt = (int)(min((int64_t)c.G1 - 1, hi) - lo) + 1;
 }
 
-// One block per frame: the frame sums (fixed list of CTA partials) for all
-// channels, read as 16-byte vectors; fp32 products summed over each thread's
+// r_t and delta_t of frame f = (v, t) from r's and delta's cosines (lanes 0 and
+// 1 of a warp hold them, so that the two inverse square roots run side by
+// side).
+__device__ __forceinline__ void frame_result(const Ctx &c, int64_t f, int v, int t, int lane, double cosine) {
+    if (lane == 0) {
+        const double r = c.ext_r ? (double)c.ext_r[f] : cosine;   // an external scorer's r_t
+        c.fr[4 * f + 0] = r;
+        if (c.frame_scores) c.frame_scores[f] = (float)r;
+    }
+    if (lane == 1) {
+        const double d = t > 0 ? fmin(2.0, fmax(0.0, 1.0 - cosine)) + 0.0 : 0.0;   // + 0.0: never -0
+        c.fr[4 * f + 1] = d;
+        if (c.drange) {   // non-negative doubles order like their bit patterns
+            const unsigned long long bits = (unsigned long long)__double_as_longlong(d);
+            atomicMin(&c.drange[2 * v], bits);
+            atomicMax(&c.drange[2 * v + 1], bits);
+        }
+    }
+}
+
+// One CTA per frame: the frame sums (fixed list of CTA partials) for all
+// channels, read as 16-byte vectors, up to four partials of the frame and four
+// of the one before it in flight; fp32 products summed over each thread's
 // channels and across each warp, the warp totals in fp64; then
 // r_t = cos(v_bar_t, u_q) and delta_t = 1 - cos(v_bar_t, v_bar_{t-1})
-// clamped to [0, 2] (Eq. 7) in fp64.
-__global__ void __launch_bounds__(512) frame_stats_kernel(Ctx c) {
+// clamped to [0, 2] (Eq. 7) in fp64.  Another CTA per frame forms its gate
+// (where there is one).  Bound by the latency of these steps: 64 frames of
+// 13 x 13 x 3584 take 6.0 us (first CTA past its wait to the last one's end);
+// 8.2 us with the partials of the two frames read one after the other, two at
+// a time, 64-bit divisions, and the gate in the other half of the CTA.
+__global__ void __launch_bounds__(512, 2) frame_stats_kernel(Ctx c) {
     pdl_wait();
     pdl_trigger();
     __shared__ float wsum[16][5];
     __shared__ float gate_map[WZ_MAX_HW * WZ_MAX_HW];   // the frame's saliency map
-    const int64_t f = blockIdx.x;
-    // the upper half of the threads forms the gate (where there is one) while
-    // the lower half forms the statistics
-    const bool split = c.gate && c.spatial_mode == WZ_SPATIAL_WSM;
-    const int half = (int)blockDim.x / 2;
-    if (split && (int)threadIdx.x >= half) {
-        frame_gate(c, f, (int)threadIdx.x - half, half, gate_map);
+    const int64_t VT = (int64_t)c.V * c.T;
+    if ((int64_t)blockIdx.x >= VT) {
+        frame_gate(c, (int64_t)blockIdx.x - VT, gate_map);
         return;
     }
-    const int nst = split ? half : (int)blockDim.x;   // threads forming the statistics
-    const int t = (int)(f % c.T);
-    const int v = (int)(f / c.T);
-    const int64_t lo = f * c.N / c.L1;
-    const int64_t hi = min((int64_t)c.G1 - 1, ((f + 1) * c.N - 1) / c.L1);
-    const int64_t g = f - 1;
-    const int64_t lo2 = t > 0 ? g * c.N / c.L1 : 0;
-    const int64_t hi2 = t > 0 ? min((int64_t)c.G1 - 1, ((g + 1) * c.N - 1) / c.L1) : -1;
+    const int64_t f = blockIdx.x;
+    const int v = (int)blockIdx.x / c.T, t = (int)blockIdx.x - v * c.T;
+    int64_t sf_at, sp_at = 0;
+    int nf, np = 0;
+    frame_slots(c, f, sf_at, nf);
+    if (t > 0) frame_slots(c, f - 1, sp_at, np);
     const int nv = c.D / 4;
-    const float4 *P = reinterpret_cast<const float4 *>(c.part);
+    const float4 *Pf = reinterpret_cast<const float4 *>(c.part) + (size_t)sf_at * nv;
+    const float4 *Pp = reinterpret_cast<const float4 *>(c.part) + (size_t)sp_at * nv;
     const float4 *Qv = reinterpret_cast<const float4 *>(c.qbar32 + (size_t)v * c.D);
     float p0 = 0.f, p1 = 0.f, p2 = 0.f, p3 = 0.f, p4 = 0.f;
-    for (int i = threadIdx.x; i < nv; i += nst) {
-        float4 sf = make_float4(0.f, 0.f, 0.f, 0.f), sp = sf;
-        for (int64_t cc = lo; cc <= hi; cc += 2) {   // two partial rows in flight, summed in order
-            const float4 x = P[(size_t)(cc + f) * nv + i];
-            const float4 y = cc + 1 <= hi ? P[(size_t)(cc + 1 + f) * nv + i] : make_float4(0.f, 0.f, 0.f, 0.f);
-            sf.x += x.x; sf.y += x.y; sf.z += x.z; sf.w += x.w;
-            if (cc + 1 <= hi) { sf.x += y.x; sf.y += y.y; sf.z += y.z; sf.w += y.w; }
-        }
-        for (int64_t cc = lo2; cc <= hi2; cc += 2) {
-            const float4 x = P[(size_t)(cc + g) * nv + i];
-            const float4 y = cc + 1 <= hi2 ? P[(size_t)(cc + 1 + g) * nv + i] : make_float4(0.f, 0.f, 0.f, 0.f);
-            sp.x += x.x; sp.y += x.y; sp.z += x.z; sp.w += x.w;
-            if (cc + 1 <= hi2) { sp.x += y.x; sp.y += y.y; sp.z += y.z; sp.w += y.w; }
-        }
+    const int nmax = max(nf, np);
+    for (int i = threadIdx.x; i < nv; i += blockDim.x) {
+        const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
         const float4 q = Qv[i];
+        float4 sf = zero, sp = zero;
+        for (int k0 = 0; k0 < nmax; k0 += 4) {
+            float4 x[4], y[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                x[k] = k0 + k < nf ? Pf[(size_t)(k0 + k) * nv + i] : zero;
+                y[k] = k0 + k < np ? Pp[(size_t)(k0 + k) * nv + i] : zero;
+            }
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {   // in slot order
+                if (k0 + k < nf) { sf.x += x[k].x; sf.y += x[k].y; sf.z += x[k].z; sf.w += x[k].w; }
+                if (k0 + k < np) { sp.x += y[k].x; sp.y += y[k].y; sp.z += y[k].z; sp.w += y[k].w; }
+            }
+        }
         if (c.frame_mean) {   // caller's buffer: 4-byte alignment only
             float *fm = c.frame_mean + (size_t)f * c.D + 4 * i;
             fm[0] = sf.x / (float)c.N;
@@ -620,30 +637,28 @@ __global__ void __launch_bounds__(512) frame_stats_kernel(Ctx c) {
         p3 += __shfl_xor_sync(0xffffffffu, p3, o);
         p4 += __shfl_xor_sync(0xffffffffu, p4, o);
     }
-    const int warp = threadIdx.x >> 5, nw = nst >> 5;
-    if ((threadIdx.x & 31) == 0) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    if (lane == 0) {
         wsum[warp][0] = p0;
         wsum[warp][1] = p1;
         wsum[warp][2] = p2;
         wsum[warp][3] = p3;
         wsum[warp][4] = p4;
     }
-    if (split) asm volatile("bar.sync 1, %0;" ::"r"(half) : "memory");   // the statistics' warps only
-    else __syncthreads();
+    __syncthreads();
     if (warp == 0) {
-        // lane k < 5 sums quantity k over the warps in order (one fp64 warp
-        // instruction per warp partial instead of five)
-        const int lane = threadIdx.x & 31;
+        // lane 4 k + h (k < 5) sums quantity k over the warps h, h + 4, ..; the
+        // four parts in a tree
         double acc = 0.0;
-        if (lane < 5)
-            for (int w = 0; w < nw; ++w) acc += (double)wsum[w][lane];
-        const double vq = __shfl_sync(0xffffffffu, acc, 0), vv = __shfl_sync(0xffffffffu, acc, 1);
-        const double vp = __shfl_sync(0xffffffffu, acc, 2), qq = __shfl_sync(0xffffffffu, acc, 3);
-        const double pp = __shfl_sync(0xffffffffu, acc, 4);
-        if (lane == 0) {
-            const double qn = sqrt(qq);
-            frame_result(c, f, v, t, (vv > 0.0 && qn > 0.0) ? vq / (sqrt(vv) * qn) : 0.0, vv, vp, pp);
-        }
+        if (lane < 20)
+            for (int w = lane & 3; w < nw; w += 4) acc += (double)wsum[w][lane >> 2];
+        acc += __shfl_xor_sync(0xffffffffu, acc, 1);
+        acc += __shfl_xor_sync(0xffffffffu, acc, 2);
+        const double vq = __shfl_sync(0xffffffffu, acc, 0), vv = __shfl_sync(0xffffffffu, acc, 4);
+        const double vp = __shfl_sync(0xffffffffu, acc, 8), qq = __shfl_sync(0xffffffffu, acc, 12);
+        const double pp = __shfl_sync(0xffffffffu, acc, 16);
+        const double den2 = vv * (lane == 0 ? qq : pp), num = lane == 0 ? vq : vp;
+        frame_result(c, f, v, t, lane, den2 > 0.0 ? num * rsqrt(den2) : 0.0);
     }
 }
 
@@ -673,7 +688,7 @@ __global__ void __launch_bounds__(kStatsThreads, 2) frame_stats_maxsim_kernel(Ct
     extern __shared__ float4 sfs[];   // [FPB][D/4] frame sums
     const int per_video = (c.T + FPB - 1) / FPB, nstat = c.V * per_video;
     if ((int)blockIdx.x >= nstat) {
-        frame_gate(c, (int64_t)blockIdx.x - nstat, threadIdx.x, kStatsThreads, gate_map);
+        frame_gate(c, (int64_t)blockIdx.x - nstat, gate_map);
         return;
     }
     const int v = (int)blockIdx.x / per_video, t0 = ((int)blockIdx.x - v * per_video) * FPB;
@@ -683,16 +698,13 @@ __global__ void __launch_bounds__(kStatsThreads, 2) frame_stats_maxsim_kernel(Ct
     const VideoPar par = c.vpar[v];
     const int nv = c.D / 4;
     const float4 *P = reinterpret_cast<const float4 *>(c.part);
-    // the column partials of frame f0 - 1 + k: slots [lo, lo + n)
+    // the column partials of frame f0 - 1 + k
     int64_t slot[FPB + 1];
     int cnt[FPB + 1];
 #pragma unroll
     for (int k = 0; k <= FPB; ++k) {
-        const int64_t f = f0 - 1 + k;
-        const bool on = (k > 0 || t0 > 0) && k <= nf;
-        const int64_t lo = on ? f * c.N / c.L1 : 0;
-        slot[k] = lo + f;
-        cnt[k] = on ? (int)(min((int64_t)c.G1 - 1, ((f + 1) * c.N - 1) / c.L1) - lo) + 1 : 0;
+        slot[k] = cnt[k] = 0;
+        if ((k > 0 || t0 > 0) && k <= nf) frame_slots(c, f0 - 1 + k, slot[k], cnt[k]);
     }
     auto dot4 = [](const float4 &a, const float4 &b, float s) {
         return fmaf(a.x, b.x, fmaf(a.y, b.y, fmaf(a.z, b.z, fmaf(a.w, b.w, s))));
@@ -798,10 +810,9 @@ __global__ void __launch_bounds__(kStatsThreads, 2) frame_stats_maxsim_kernel(Ct
             for (int w = 0; w < NW; ++w) acc += (double)wsum[warp][w][lane];
         const double s0 = __shfl_sync(0xffffffffu, acc, 0), s1 = __shfl_sync(0xffffffffu, acc, 1);
         const double s2 = __shfl_sync(0xffffffffu, acc, 2);
-        if (lane == 0) {
-            const double m = fmax(fmax(best[warp][0], best[warp][1]), fmax(best[warp][2], best[warp][3]));
-            frame_result(c, f0 + warp, v, t0 + warp, s0 > 0.0 ? m / sqrt(s0) : 0.0, s0, s1, s2);
-        }
+        const double m = fmax(fmax(best[warp][0], best[warp][1]), fmax(best[warp][2], best[warp][3]));
+        const double den2 = lane == 0 ? s0 : s0 * s2, num = lane == 0 ? m : s1;
+        frame_result(c, f0 + warp, v, t0 + warp, lane, den2 > 0.0 ? num * rsqrt(den2) : 0.0);
     }
 }
 
@@ -974,11 +985,11 @@ cudaError_t launch_frame_stats(const Ctx &c, cudaStream_t s) {
         return launch_kernel(fn, dim3(c.V * ((c.T + fpb - 1) / fpb) + gates), dim3(kStatsThreads), smem, s, args,
                              c.pdl != 0);
     }
-    // 512 threads a frame (4 CTAs per SM); with the gate's split form and more
-    // frames than one wave of those, 256 (twice the CTAs in flight)
-    const bool split = c.gate && c.spatial_mode == WZ_SPATIAL_WSM;
-    const int threads = split && (int64_t)c.V * c.T > 4 * (int64_t)sms ? 256 : 512;
-    return launch_kernel((const void *)frame_stats_kernel, dim3(c.V * c.T), dim3(threads), 0, s, args, c.pdl != 0);
+    // a CTA per frame and one per gate; 256 threads (more CTAs in flight) once
+    // 512 no longer fit in one wave
+    const int64_t ctas = (int64_t)c.V * c.T * (c.gate && c.spatial_mode == WZ_SPATIAL_WSM ? 2 : 1);
+    const int threads = ctas > 2 * (int64_t)sms ? 256 : 512;
+    return launch_kernel((const void *)frame_stats_kernel, dim3((unsigned)ctas), dim3(threads), 0, s, args, c.pdl != 0);
 }
 
 }  // namespace wz
