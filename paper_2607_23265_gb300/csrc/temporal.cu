@@ -12,7 +12,10 @@
 //   units     the tensor-core work list of the frame  (this library)
 //
 // Every reduction runs in a fixed order for a fixed block size, so results
-// do not depend on scheduling.
+// do not depend on scheduling.  One CTA of latency-bound steps: r_t and gamma_t
+// stay in shared memory; barriers and fp64 chains are what remains (64 frames:
+// 8.4 us past its wait; 10.0 with the per-frame state in global memory, one
+// thread per frame and the budget sums on three barriers each).
 #include <cmath>
 
 #include "wz_spatial.cuh"
@@ -98,14 +101,55 @@ __device__ void block_excl_scan(const int (&x)[K], int *ws, int (&excl)[K], int 
 
 
 // h = min(H, ceil(sqrt(n H / W))): a float estimate corrected to the exact
-// smallest h >= 1 with h^2 W >= n H in integers.
+// smallest h >= 1 with h^2 W >= n H in integers (n <= 4096, H, W <= 64: 32 bits).
 __device__ __forceinline__ int grid_h(int n, int H, int W) {
     if (n <= 0) return 0;
-    long long h = (long long)ceilf(sqrtf((float)n * (float)H / (float)W));
+    int h = (int)ceilf(sqrtf((float)(n * H) / (float)W));
     if (h < 1) h = 1;
-    while (h * h * W < (long long)n * H) ++h;
-    while (h > 1 && (h - 1) * (h - 1) * W >= (long long)n * H) --h;
-    return (int)(h < H ? h : H);
+    while (h * h * W < n * H) ++h;
+    while (h > 1 && (h - 1) * (h - 1) * W >= n * H) --h;
+    return h < H ? h : H;
+}
+
+// Block-wide sum of a double in a fixed order, two barriers: warp trees, then
+// warp 0 over the warp totals.  `scratch` holds 33 doubles and serves one call
+// after another (a call's writes follow a barrier after the last one's reads).
+__device__ __forceinline__ double sum_block(double v, double *scratch) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (lane == 0) scratch[warp] = v;
+    __syncthreads();
+    if (warp == 0) {
+        double s = lane < nw ? scratch[lane] : 0.0;
+        for (int o = 8; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);   // nw <= 16
+        if (lane == 0) scratch[32] = s;
+    }
+    __syncthreads();
+    return scratch[32];
+}
+
+// Block-wide sums of two ints (each below 2^31 in total), as above; `scratch`
+// holds 66 ints.
+__device__ __forceinline__ void sum_block2(int &a, int &b, int *scratch) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    a = __reduce_add_sync(0xffffffffu, a);
+    b = __reduce_add_sync(0xffffffffu, b);
+    if (lane == 0) {
+        scratch[warp] = a;
+        scratch[33 + warp] = b;
+    }
+    __syncthreads();
+    if (warp == 0) {
+        const int x = __reduce_add_sync(0xffffffffu, lane < nw ? scratch[lane] : 0);
+        const int y = __reduce_add_sync(0xffffffffu, lane < nw ? scratch[33 + lane] : 0);
+        if (lane == 0) {
+            scratch[32] = x;
+            scratch[65] = y;
+        }
+    }
+    __syncthreads();
+    a = scratch[32];
+    b = scratch[65];
 }
 
 // Shared-memory arrays of one video, indexed by retained frame m (wgt,
@@ -135,10 +179,10 @@ __host__ __device__ inline size_t temporal_smem_bytes(int T, int J) {
     return temporal_smem_offset_coef(T) + sizeof(double) * coef;
 }
 
-// Threads of the CTA: one frame per thread up to 512 frames, at most
-// WZ_MAX_T / kTemporalThreads frames per thread beyond (fp64 work scales with
-// the warps).
-inline int temporal_threads(int T) { return T <= 512 ? (T < 32 ? 32 : (T + 31) / 32 * 32) : 512; }
+// Threads of the CTA: one frame per thread from 128 (the remainder ranking
+// takes several lanes per frame) up to 512, at most WZ_MAX_T / kTemporalThreads
+// frames per thread beyond (fp64 work scales with the warps).
+inline int temporal_threads(int T) { return T <= 512 ? (T < 128 ? 128 : (T + 31) / 32 * 32) : 512; }
 
 // WTA levels 2..J (J > 1): level 1 left its approximation in A0, its gate in
 // G0 and its gated details in dall[0, K1).  Each further level analyses the
@@ -203,33 +247,36 @@ __device__ __noinline__ const double *wta_deeper_levels(const Ctx &c, double *A0
 __global__ void __launch_bounds__(kTemporalThreads) temporal_kernel(Ctx c) {
     pdl_wait();
     pdl_trigger();
-    if ((int)blockIdx.x == c.V) {
-        // the extra CTA: the spatial kernel's row counter, the condensation's
+    if ((int)blockIdx.x >= c.V) {
+        // the extra CTAs: the spatial kernel's row counter, the condensation's
         // unit counter and, with several WSM levels, the multi-level tables
-        // of the spatial operator (the single-level kernel forms its tables
-        // itself)
-        if (threadIdx.x == 0 && c.spatial_next) {
+        // of the spatial operator in four independent parts (the single-level
+        // kernel forms its tables itself)
+        const int part = (int)blockIdx.x - c.V;
+        if (part == 0 && threadIdx.x == 0 && c.spatial_next) {
             c.spatial_next[0] = 0;
             c.spatial_next[1] = 0;
         }
-        if (c.wsm_levels > 1) build_ml_tables(c);
+        if (c.wsm_levels > 1) build_ml_tables(c, part);
         return;
     }
     extern __shared__ __align__(16) unsigned char tsm[];
-    __shared__ double dscr[64];
-    __shared__ long long lscr[66];
+    __shared__ double dscr[33];
+    __shared__ int iscr2[66];
     __shared__ int iscr[4 * 33];
     const int v = blockIdx.x;
     const int T = c.T;
     const int64_t base = (int64_t)v * T;
     const VideoPar vp = c.vpar[v];
-    double *fr = c.fr + base * 4;          // r, delta, gamma, r~
+    const double2 *fr = reinterpret_cast<const double2 *>(c.fr + base * 4);   // r, delta of frame t at 2 t
     double *wgt = reinterpret_cast<double *>(tsm);                        // weight of retained frame m
     unsigned long long *keys = reinterpret_cast<unsigned long long *>(tsm + temporal_smem_keys(T));   // remainder key
     int *lst = reinterpret_cast<int *>(keys + T);                         // retained frames
     int *nb = lst + T;                     // budget of retained frame m; -1 while active
     int *nf = nb + T;                      // budget of frame t
     double *qv = reinterpret_cast<double *>(tsm + temporal_smem_quota(T));   // quota of retained frame m
+    // until the budgets: r of frame t in qv, gamma in keys
+    double *rs = qv, *gam = reinterpret_cast<double *>(keys);
     const int J = c.wta_levels;
     const int KH = temporal_coef_len(T, J);
     double *A0 = reinterpret_cast<double *>(tsm + temporal_smem_offset_coef(T));   // WTA approximation
@@ -241,34 +288,41 @@ __global__ void __launch_bounds__(kTemporalThreads) temporal_kernel(Ctx c) {
     // delta over the video (Eq. 7)
     const double lo = __longlong_as_double((long long)c.drange[2 * v]);
     const double hi = __longlong_as_double((long long)c.drange[2 * v + 1]);
+    const double inv = hi > lo ? 1.0 / (hi - lo) : 0.0;   // (while the frames' values are on their way)
     // gamma_t and the retained set (frame 1 always kept)
     const double tau = (double)c.tau;
     // each thread owns `per` consecutive frames t0 .. t1 - 1;
     // nf[t] holds the frame's keep flag until the retained list is written
     const int per = (T + (int)blockDim.x - 1) / (int)blockDim.x;
     const int t0 = threadIdx.x * per, t1 = min(T, t0 + per);
+    // (delta >= 0: without a positive threshold every frame is retained)
+    const bool all = !(tau > 0.0);
     int cnt = 0;
     for (int t = t0; t < t1; ++t) {
-        const double d = fr[4 * t + 1];
-        const double gm = hi > lo ? (d - lo) / (hi - lo) : 0.0;
-        fr[4 * t + 2] = gm;
-        fr[4 * t + 3] = NAN;
+        const double2 rd = fr[2 * t];
+        const double d = rd.y;
+        const double gm = (d - lo) * inv;
+        rs[t] = rd.x;
+        gam[t] = gm;
         if (c.out_rel) {   // r~ follows with the WTA (NaN: filtered)
             float *orl = c.out_rel + (base + t) * 4;
-            orl[0] = (float)fr[4 * t];
+            orl[0] = (float)rd.x;
             orl[1] = (float)d;
             orl[2] = (float)gm;
-            orl[3] = NAN;
+            if (!all) orl[3] = NAN;
         }
         const int kp = (t == 0 || d >= tau) ? 1 : 0;
-        nf[t] = kp;
+        nf[t] = all ? 0 : kp;
+        if (all) lst[t] = t;
         cnt += kp;
     }
-    int L = 0;
-    int pos = block_excl_scan(cnt, iscr, &L);
-    for (int t = t0; t < t1; ++t) {
-        if (nf[t]) lst[pos++] = t;
-        nf[t] = 0;
+    int L = T;
+    if (!all) {
+        int pos = block_excl_scan(cnt, iscr, &L);
+        for (int t = t0; t < t1; ++t) {
+            if (nf[t]) lst[pos++] = t;
+            nf[t] = 0;
+        }
     }
     __syncthreads();
 
@@ -286,19 +340,20 @@ __global__ void __launch_bounds__(kTemporalThreads) temporal_kernel(Ctx c) {
     for (int k = threadIdx.x; k < K; k += blockDim.x) {
         double ca = 0.0, cd = 0.0;
         for (int j = 0; j < FT; ++j) {
-            const double x = fr[4 * lst[ext_index(2 * k + 1 - j, L, WZ_MODE_SYMMETRIC)]];
+            const double x = rs[lst[ext_index(2 * k + 1 - j, L, WZ_MODE_SYMMETRIC)]];
             ca += c.wta_dec_lo[j] * x;
             cd += c.wta_dec_hi[j] * x;
         }
         const int m0 = ext_index(2 * k, L, WZ_MODE_SYMMETRIC), m1 = ext_index(2 * k + 1, L, WZ_MODE_SYMMETRIC);
-        const double g = 0.5 * (fr[4 * lst[m0] + 2] + fr[4 * lst[m1] + 2]);
+        const double g = 0.5 * (gam[lst[m0]] + gam[lst[m1]]);
         A0[k] = ca;
         dall[k] = g * cd;
         if (J > 1) G0[k] = g;
     }
     __syncthreads();
     const double *ain = J > 1 ? wta_deeper_levels(c, A0, A1, G0, G1, dall, K, J) : A0;
-    int anypos = 0;
+    // (the first round's sum of the weights rides along)
+    double sp = 0.0;
     for (int m = threadIdx.x; m < L; m += blockDim.x) {
         double rt = 0.0;
         const int alo = m >> 1, ahi = min(K - 1, (m + FT - 2) >> 1);
@@ -307,21 +362,14 @@ __global__ void __launch_bounds__(kTemporalThreads) temporal_kernel(Ctx c) {
             rt += c.wta_rec_lo[kk] * ain[ai] + c.wta_rec_hi[kk] * dall[ai];
         }
         const int t = lst[m];
-        fr[4 * t + 3] = rt;
         if (c.out_rel) c.out_rel[(base + t) * 4 + 3] = (float)rt;
         const double wv = c.temporal_mode == WZ_TEMPORAL_WTA ? rt
-                          : c.temporal_mode == WZ_TEMPORAL_RAW ? fr[4 * t] : 1.0;
-        wgt[m] = fmax(wv, 0.0);
-        anypos |= (wv > 0.0);
-    }
-    // uniform weights if none is positive
-    anypos = __syncthreads_or(anypos);
-    for (int m = threadIdx.x; m < L; m += blockDim.x) {
+                          : c.temporal_mode == WZ_TEMPORAL_RAW ? rs[t] : 1.0;
+        const double w = fmax(wv, 0.0);
+        wgt[m] = w;
         nb[m] = -1;
-        if (!anypos) wgt[m] = 1.0;
+        sp += w;
     }
-    __syncthreads();
-
     // Budgets (Eq. 5, Eq. 15): largest-remainder apportionment of B over the
     // weights, frames whose quota exceeds N capped at N and the rest
     // re-apportioned.
@@ -330,32 +378,29 @@ __global__ void __launch_bounds__(kTemporalThreads) temporal_kernel(Ctx c) {
     if ((long long)L * N <= (long long)B) {
         for (int m = threadIdx.x; m < L; m += blockDim.x) nb[m] = N;
     } else {
-        long long remaining = B;
+        int remaining = B;
         for (int round = 0; round <= L; ++round) {
             // candidates: active frames with positive weight, else all active
-            double sp = 0.0;
-            int npos = 0;
-            for (int m = threadIdx.x; m < L; m += blockDim.x)
-                if (nb[m] < 0 && wgt[m] > 0.0) {
-                    sp += wgt[m];
-                    npos = 1;
-                }
-            npos = __syncthreads_or(npos);
-            const bool uniform = (npos == 0);
-            double S = 0.0;
+            // (S > 0 exactly when a weight is); round 0 has the sum already
+            if (round > 0) {
+                sp = 0.0;
+                for (int m = threadIdx.x; m < L; m += blockDim.x)
+                    if (nb[m] < 0) sp += wgt[m];
+            }
+            double S = sum_block(sp, dscr);
+            const bool uniform = !(S > 0.0);
             if (uniform) {
-                int na = 0;
+                int na = 0, none = 0;
                 for (int m = threadIdx.x; m < L; m += blockDim.x) na += (nb[m] < 0);
-                S = (double)block_sum_ll(na, lscr);
-            } else {
-                S = block_sum(sp, dscr);
+                sum_block2(na, none, iscr2);
+                S = (double)na;
             }
             // quota q_m = remaining * w_m / S of every candidate; in the same
             // pass the caps that bind and, for the largest remainder, the
             // floors and the fractional parts (non-negative doubles order like
             // their bit patterns; a candidate's key is its pattern + 1, others
             // 0, so non-candidates rank below every candidate)
-            long long ncap = 0, fsum = 0;
+            int ncap = 0, fsum = 0;
             for (int m = threadIdx.x; m < L; m += blockDim.x) {
                 const double w = uniform ? 1.0 : wgt[m];
                 unsigned long long key = 0ull;
@@ -363,21 +408,20 @@ __global__ void __launch_bounds__(kTemporalThreads) temporal_kernel(Ctx c) {
                     const double q = (double)remaining * w / S;
                     const double fl = floor(q);
                     ncap += (q > (double)N);
-                    fsum += (long long)fl;
+                    fsum += (int)fl;
                     key = (unsigned long long)__double_as_longlong(q - fl) + 1ull;
                     qv[m] = q;
                 }
                 keys[m] = key;
             }
-            block_sum2_ll(ncap, fsum, lscr);
+            sum_block2(ncap, fsum, iscr2);   // (every key is in place after it)
             if (ncap > 0) {
                 for (int m = threadIdx.x; m < L; m += blockDim.x)
                     if (keys[m] != 0ull && qv[m] > (double)N) nb[m] = N;
-                remaining -= (long long)N * ncap;
-                __syncthreads();
+                remaining -= N * ncap;
                 continue;
             }
-            const long long R = remaining - fsum;
+            const int R = remaining - fsum;
             const ulonglong2 *k2 = reinterpret_cast<const ulonglong2 *>(keys);
             // rank = #{k : key_k > key_m, or key_k == key_m and k < m}, counted
             // by gs lanes per frame (the largest power of two <= 32 with
@@ -489,7 +533,7 @@ cudaError_t launch_temporal(const Ctx &c, cudaStream_t s) {
     cudaError_t e = cudaFuncSetAttribute(temporal_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     void *args[] = {const_cast<Ctx *>(&c)};
-    return launch_kernel((const void *)temporal_kernel, dim3(c.V + 1), dim3(temporal_threads(c.T)), smem, s, args,
+    return launch_kernel((const void *)temporal_kernel, dim3(c.V + (c.wsm_levels > 1 ? kMLParts : 1)), dim3(temporal_threads(c.T)), smem, s, args,
                          c.pdl != 0);
 }
 

@@ -479,27 +479,34 @@ struct MLSmem {
     }
 };
 
-// Build the multi-level tables into c.stab (one CTA).  Level l's matrices
-// are formed from level l-1's in global memory; a block barrier separates
-// the levels (global writes of the block are visible to it after the barrier).
-static __device__ __noinline__ void build_ml_tables(const Ctx &c) {
+// Build one of the kMLParts independent parts of the multi-level tables in
+// c.stab (a CTA each): side part & 1 (height, width), analysis rows (part < 2)
+// or synthesis columns.  Level l's matrices are formed from level l-1's in
+// global memory; a block barrier separates the levels (global writes of the
+// block are visible to it after the barrier).
+constexpr int kMLParts = 4;
+
+static __device__ __noinline__ void build_ml_tables(const Ctx &c, int part) {
     MLTables T;
     T.init(c.H, c.W, c.F, c.wsm_levels);
     float *tb = c.stab;
     int *ti = reinterpret_cast<int *>(c.stab);
     const int F = c.F, H = c.H, W = c.W;
-    // supports, gathered with shared-memory atomics while the tables are formed
-    __shared__ int sup[6][kMaxLevels][WZ_MAX_HW];   // blo, bhi (AW rows), slo, shi (SH), xlo, xhi (SW)
+    const int side = part & 1;
+    const bool analysis = part < 2;
+    // supports per level and map row or column, gathered with shared-memory
+    // atomics while the tables are formed: AW rows at a column, SH / SW columns
+    // at a row / column
+    __shared__ int sup[2][kMaxLevels][WZ_MAX_HW];
     for (int k = threadIdx.x; k < kMaxLevels * WZ_MAX_HW; k += blockDim.x) {
-        const int l = k / WZ_MAX_HW, x = k % WZ_MAX_HW;
-        sup[0][l][x] = sup[2][l][x] = sup[4][l][x] = 1 << 30;
-        sup[1][l][x] = sup[3][l][x] = sup[5][l][x] = -1;
+        sup[0][k / WZ_MAX_HW][k % WZ_MAX_HW] = 1 << 30;
+        sup[1][k / WZ_MAX_HW][k % WZ_MAX_HW] = -1;
     }
     __syncthreads();
     for (int l = 0; l < T.J; ++l) {
-        // analysis rows: AX_u^{l+1}[a][i] = sum_j dec_u[j] AX_L^l[ext(2a + 1 - j)][i]
-        for (int side = 0; side < 2; ++side) {
-            const int n = side ? W : H, nin = side ? T.w[l] : T.h[l], nout = side ? T.w[l + 1] : T.h[l + 1];
+        const int n = side ? W : H, nin = side ? T.w[l] : T.h[l], nout = side ? T.w[l + 1] : T.h[l + 1];
+        if (analysis) {
+            // AX_u^{l+1}[a][i] = sum_j dec_u[j] AX_L^l[ext(2a + 1 - j)][i]
             float *lo = tb + (side ? T.AWl[l] : T.AHl[l]), *hi = tb + (side ? T.AWh[l] : T.AHh[l]);
             const float *prev = l ? tb + (side ? T.AWl[l - 1] : T.AHl[l - 1]) : nullptr;
             for (int k = threadIdx.x; k < nout * n; k += blockDim.x) {
@@ -520,7 +527,8 @@ static __device__ __noinline__ void build_ml_tables(const Ctx &c) {
                     atomicMax(&sup[1][l][i], a);
                 }
             }
-            // synthesis columns: SX_u^{l+1}[y][a] = sum_k SX_L^l[y][k] rec_u[k + F - 2 - 2a]
+        } else {
+            // SX_u^{l+1}[y][a] = sum_k SX_L^l[y][k] rec_u[k + F - 2 - 2a]
             float *slo_ = tb + (side ? T.SWl[l] : T.SHl[l]), *shi_ = tb + (side ? T.SWh[l] : T.SHh[l]);
             const float *sprev = l ? tb + (side ? T.SWl[l - 1] : T.SHl[l - 1]) : nullptr;
             for (int k = threadIdx.x; k < n * nout; k += blockDim.x) {
@@ -536,24 +544,22 @@ static __device__ __noinline__ void build_ml_tables(const Ctx &c) {
                 slo_[k] = sl;
                 shi_[k] = sh;
                 if (sl != 0.f || sh != 0.f) {
-                    atomicMin(&sup[side ? 4 : 2][l][y], a);
-                    atomicMax(&sup[side ? 5 : 3][l][y], a);
+                    atomicMin(&sup[0][l][y], a);
+                    atomicMax(&sup[1][l][y], a);
                 }
             }
         }
         __syncthreads();
     }
     // supports (empty: lo = the band length, hi = -1)
+    if (analysis && !side) return;
     for (int l = 0; l < T.J; ++l) {
-        for (int x = threadIdx.x; x < W; x += blockDim.x) {
-            ti[T.blo[l] + x] = min(sup[0][l][x], T.w[l + 1]);
-            ti[T.bhi[l] + x] = sup[1][l][x];
-            ti[T.xlo[l] + x] = min(sup[4][l][x], T.w[l + 1]);
-            ti[T.xhi[l] + x] = sup[5][l][x];
-        }
-        for (int y = threadIdx.x; y < H; y += blockDim.x) {
-            ti[T.slo[l] + y] = min(sup[2][l][y], T.h[l + 1]);
-            ti[T.shi[l] + y] = sup[3][l][y];
+        const int n = side ? W : H, band = side ? T.w[l + 1] : T.h[l + 1];
+        const int lo = analysis ? T.blo[l] : side ? T.xlo[l] : T.slo[l];
+        const int hi = analysis ? T.bhi[l] : side ? T.xhi[l] : T.shi[l];
+        for (int x = threadIdx.x; x < n; x += blockDim.x) {
+            ti[lo + x] = min(sup[0][l][x], band);
+            ti[hi + x] = sup[1][l][x];
         }
     }
 }
