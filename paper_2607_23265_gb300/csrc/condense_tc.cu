@@ -23,8 +23,9 @@
 // one unit overlaps the main loop of the next whenever two fit.  Per chunk,
 // only the operator rows whose grid rows reach that chunk's map rows are
 // loaded and multiplied (Ctx::krange; the first chunk covers every row, so
-// each accumulator column is initialised).  Units are claimed from a global
-// counter, so SMs that drew small units take more of them.  One CTA per SM:
+// each accumulator column is initialised).  CTA b starts with unit b and then
+// claims units from a global counter, so SMs that drew small units take more
+// of them.  One CTA per SM:
 //   warp 0      unit claims and the TMA producer (one thread), 4-stage ring
 //   warp 1      TMEM allocation and the MMA issuer (one thread)
 //   warps 2-13  epilogue, three warps per TMEM lane quadrant: 16x256b
@@ -89,22 +90,27 @@ struct TcMaps {
 };
 
 struct Unit {
-    int f, j0, ct0, nc, cg, kclo, kchi;   // operator chunks [kclo, kchi] (the rest are zero)
-    bool ranged;                          // per-chunk operator rows in c.krange
+    int f, wrow, j0, ct0, nc, cg, kclo, kchi;   // operator chunks [kclo, kchi] (the rest are zero)
+    bool ranged;                                // per-chunk operator rows in c.krange
 };
 
-__device__ __forceinline__ Unit decode_unit(const Ctx &c, const int *vprefix, int u) {
+// The record of unit u of the call (unit_records).
+__device__ __forceinline__ int4 unit_record(const Ctx &c, const int *vprefix, int u) {
     int lo = 0, hi = c.V - 1;
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
         if (vprefix[mid] <= u) lo = mid;
         else hi = mid - 1;
     }
-    const int4 q = c.units[(size_t)lo * c.max_units_v + (u - vprefix[lo])];
+    return c.units[(size_t)lo * c.max_units_v + (u - vprefix[lo])];
+}
+
+__device__ __forceinline__ Unit decode_unit(const int4 &q) {
     Unit r;
     r.f = q.x;
-    r.j0 = q.y;
-    r.ct0 = q.z;
+    r.wrow = q.y;
+    r.j0 = q.z & 0xffff;
+    r.ct0 = q.z >> 16;
     r.nc = q.w & 0x1ff;
     r.cg = (q.w >> 9) & 7;
     r.kclo = (q.w >> 12) & 0xff;
@@ -293,8 +299,9 @@ __device__ __forceinline__ void block_epilogue(uint32_t colb, bool fused, int nc
 
 }  // namespace
 
-// Units are claimed dynamically: the producer thread takes the next unit of
-// the whole call from a global counter (zeroed by the temporal kernel) and
+// Units are claimed dynamically: the producer thread takes unit blockIdx.x and
+// then the next one past gridDim.x from a global counter (zeroed by the temporal
+// kernel) and
 // hands its index to the MMA thread and the epilogue warps through a small
 // queue in shared memory, so CTAs that drew small units take more of them.
 // Accumulator buffers: a unit uses one of the two 256-column buffers when its
@@ -341,7 +348,9 @@ condense_tc_kernel(const __grid_constant__ TcMaps maps, Ctx c) {
     // global memory from here on: the previous grid has completed
     pdl_wait();
     pdl_trigger();
+    int4 first = make_int4(0, 0, 0, 0);   // the first unit's record, read beside the count (one video)
     if (threadIdx.x == 0) {
+        if (c.V == 1 && (int)blockIdx.x < c.max_units_v) first = c.units[blockIdx.x];
         int acc = 0;
         for (int v = 0; v < c.V; ++v) {
             S->vprefix[v] = acc;
@@ -372,24 +381,33 @@ condense_tc_kernel(const __grid_constant__ TcMaps maps, Ctx c) {
                 fail(c, abort_flag, 1);
                 break;
             }
-            int u = *abort_flag ? -1 : atomicAdd(c.spatial_next + 1, 1);
+            int u = *abort_flag ? -1 : k == 0 ? (int)blockIdx.x : (int)gridDim.x + atomicAdd(c.spatial_next + 1, 1);
             if (u >= n_units) u = -1;
             uq[slot] = u;
             ptx::mbar_arrive(&S->qfull[slot]);
             if (u < 0) break;
-            const Unit un = decode_unit(c, S->vprefix, u);
+            const Unit un = decode_unit(k == 0 && c.V == 1 ? first : unit_record(c, S->vprefix, u));
             const UnitShape sh = unit_shape(un, KC);
             if (!sh.valid) {   // not a record the spatial kernel writes
                 fail(c, abort_flag, 4);
                 break;
             }
-            const int64_t wrow0 = (int64_t)c.woff[un.f] + un.j0;     // multiple of 16
-            if (un.ranged) {   // the unit's chunk ranges, loaded together
-                const uint16_t *kr = c.krange + ((size_t)un.f * c.krange_nblk + (un.j0 >> 8)) * KC;
-                for (int kc = un.kclo + 1; kc <= un.kchi; ++kc) S->krow[kc] = kr[kc];
-            }
+            const int64_t wrow0 = un.wrow;     // multiple of 16
             bool ok = true;
             for (int kc = un.kclo; kc <= un.kchi; ++kc) {
+                if (un.ranged && kc == un.kclo + 1) {
+                    // the unit's chunk ranges, eight loads in flight, while
+                    // the first chunk (every row) is on its way
+                    const uint16_t *kr = c.krange + ((size_t)un.f * c.krange_nblk + (un.j0 >> 8)) * KC;
+                    for (int q = kc; q <= un.kchi; q += 8) {
+                        uint16_t r[8];
+#pragma unroll
+                        for (int e = 0; e < 8; ++e) r[e] = q + e <= un.kchi ? kr[q + e] : (uint16_t)0;
+#pragma unroll
+                        for (int e = 0; e < 8; ++e)
+                            if (q + e <= un.kchi) S->krow[q + e] = r[e];
+                    }
+                }
                 uint32_t ja = 0, jb = (uint32_t)sh.ncp;
                 if (un.ranged && kc > un.kclo) {
                     const uint32_t r = S->krow[kc];
@@ -448,7 +466,7 @@ condense_tc_kernel(const __grid_constant__ TcMaps maps, Ctx c) {
             const int u = uq[slot];
             ptx::mbar_arrive(&S->qempty[slot]);
             if (u < 0) break;
-            const Unit un = decode_unit(c, S->vprefix, u);
+            const Unit un = decode_unit(unit_record(c, S->vprefix, u));
             const UnitShape sh = unit_shape(un, KC);
             if (!sh.valid) {
                 fail(c, abort_flag, 4);
@@ -501,7 +519,7 @@ condense_tc_kernel(const __grid_constant__ TcMaps maps, Ctx c) {
             __syncwarp();
             if (lane == 0) ptx::mbar_arrive(&S->qempty[slot]);
             if (u < 0) break;
-            const Unit un = decode_unit(c, S->vprefix, u);
+            const Unit un = decode_unit(unit_record(c, S->vprefix, u));
             const UnitShape sh = unit_shape(un, KC);
             if (!sh.valid) {
                 fail(c, abort_flag, 4);

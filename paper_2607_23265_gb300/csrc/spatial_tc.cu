@@ -46,6 +46,7 @@ struct TcSmem {
     int Q;       // [16][2][BMAX]: Q_L, Q_H of row t's grid column at b = b0(t) + k
     int tok;     // [16][8] int: per row t (see kTok*)
     int stage;   // [2][KC][512] bf16: the group's hi chunks, then its lo chunks
+    int rec;     // [2][kMaxTaps]: the synthesis taps (lanes index them differently)
     int total;
     __host__ __device__ void init(const SpatialSmem &L, int VT, int bmax) {
         int o = L.tables;
@@ -61,6 +62,7 @@ struct TcSmem {
         P = take(kTcRows * 2 * bmax, 4);
         Q = take(kTcRows * 2 * bmax, 4);
         tok = take(kTcRows * 8, 4);
+        rec = take(2 * kMaxTaps, 4);
         stage = take((L.K_pad >> 5) * kTcChunkBytes * 2 / 4, 32);   // 128-byte aligned
         total = o;
     }
@@ -121,11 +123,17 @@ __global__ void __launch_bounds__(kSpatialThreads, BMAX <= 6 ? 3 : 2)
     S.init(L, VT, BMAX);
     // the frame-independent tables come from the kernel parameters alone:
     // formed while the temporal kernel runs
+    float *rec_lo = sm + S.rec, *rec_hi = rec_lo + kMaxTaps;
+    if (tid >= kSpatialThreads - kMaxTaps) {
+        const int k = tid - (kSpatialThreads - kMaxTaps);
+        rec_lo[k] = c.rec_lo[k];
+        rec_hi[k] = c.rec_hi[k];
+    }
     build_spatial_tables_smem(c, L, sm);
     pdl_wait();
-    // thread 0 claims the next group while the current one is formed
-    int claimed = tid == 0 ? atomicAdd(c.spatial_next, 1) : 0;
-    if ((int)blockIdx.x < kTailBlocks) tail_rows(c, (int)blockIdx.x);
+    // thread 0 claims the next group while the current one is formed; the
+    // first one is the CTA's own index
+    int claimed = (int)blockIdx.x;
     int *gpre = reinterpret_cast<int *>(sm + S.gpre), *fdat = reinterpret_cast<int *>(sm + S.fdat);
     // the prefix of the frames' group counts; the frames' budgets, grids and
     // row offsets stay in shared memory (n <= 4096, h, w <= 64)
@@ -151,9 +159,10 @@ __global__ void __launch_bounds__(kSpatialThreads, BMAX <= 6 ? 3 : 2)
     const int stage_words = KC * kTcChunkBytes * 2 / 16;   // uint4 words of the stage
     const int t = tid >> 4, s = tid & 15;   // operator row of the group, slot of the row's work
 
-    // the frames' tensor-core unit records, frame f by CTA f mod gridDim.x
-    // (before the groups: the counter balances the CTAs afterwards)
-    for (int f = blockIdx.x; f < VT; f += gridDim.x) {
+    // the frames' tensor-core unit records, frame f by CTA f mod gridDim.x from
+    // the last CTA down (those without a group of their own when there are few;
+    // before the groups: the counter balances the CTAs afterwards)
+    for (int f = (int)(gridDim.x - 1 - blockIdx.x); f < VT; f += gridDim.x) {
         const int nhw = fdat[3 * f], n = nhw & 8191;
         if (n > 0) unit_records(c, f, n, (nhw >> 13) & 127, nhw >> 20, ilo, ihi);
     }
@@ -162,7 +171,7 @@ __global__ void __launch_bounds__(kSpatialThreads, BMAX <= 6 ? 3 : 2)
         __syncthreads();   // the previous group's reads of shared memory
         if (tid == 0) {
             const int it = claimed;
-            if (it < items) claimed = atomicAdd(c.spatial_next, 1);
+            if (it < items) claimed = (int)gridDim.x + atomicAdd(c.spatial_next, 1);
             int fi = 0;
             if (it < items) {
                 // the last frame whose first group is <= it (frames without
@@ -209,10 +218,10 @@ __global__ void __launch_bounds__(kSpatialThreads, BMAX <= 6 ? 3 : 2)
             if (s < BMAX) {
                 const int a = a0 + s, b = b0 + s;
                 float *P = Pt + t * 2 * BMAX, *Q = Qt + t * 2 * BMAX;
-                P[s] = a <= a1 ? (1.f - ly) * synth(c.rec_lo, F, y0, a) + ly * synth(c.rec_lo, F, y1, a) : 0.f;
-                P[BMAX + s] = a <= a1 ? (1.f - ly) * synth(c.rec_hi, F, y0, a) + ly * synth(c.rec_hi, F, y1, a) : 0.f;
-                Q[s] = b <= b1 ? (1.f - lx) * synth(c.rec_lo, F, x0, b) + lx * synth(c.rec_lo, F, x1, b) : 0.f;
-                Q[BMAX + s] = b <= b1 ? (1.f - lx) * synth(c.rec_hi, F, x0, b) + lx * synth(c.rec_hi, F, x1, b) : 0.f;
+                P[s] = a <= a1 ? (1.f - ly) * synth(rec_lo, F, y0, a) + ly * synth(rec_lo, F, y1, a) : 0.f;
+                P[BMAX + s] = a <= a1 ? (1.f - ly) * synth(rec_hi, F, y0, a) + ly * synth(rec_hi, F, y1, a) : 0.f;
+                Q[s] = b <= b1 ? (1.f - lx) * synth(rec_lo, F, x0, b) + lx * synth(rec_lo, F, x1, b) : 0.f;
+                Q[BMAX + s] = b <= b1 ? (1.f - lx) * synth(rec_hi, F, x0, b) + lx * synth(rec_hi, F, x1, b) : 0.f;
             }
             if (s == 0) {
                 const int na = min(a1 - a0 + 1, BMAX), nb = min(b1 - b0 + 1, BMAX);
@@ -319,6 +328,9 @@ __global__ void __launch_bounds__(kSpatialThreads, BMAX <= 6 ? 3 : 2)
             ptx::bulk_commit();
         }
     }
+    // rows past the produced count (tau > 0)
+    const int tail = (int)(gridDim.x - 1 - blockIdx.x);
+    if (tail < kTailBlocks) tail_rows(c, tail);
     // the operator rows are in global memory before the CTA ends
     if (tid == 0) ptx::bulk_wait();
 }

@@ -212,10 +212,11 @@ __device__ inline void tail_rows(const Ctx &c, int tb) {
 // The tensor-core work units of frame f (the temporal kernel placed them: the
 // first block's units at ustart[f], the later blocks' at ustartB[f]):
 // column blocks of <= 256 tokens, each in groups of unit_tiles(round16(nc))
-// 128-channel tiles, as even as n_ct allows.  A record is (f, j0, first tile,
-// nc | tiles << 9 | kc_lo << 12 | kc_hi << 20 | ranged): the unit's operator
-// rows are zero outside the 32-column chunks [kc_lo, kc_hi] (K_pad <= 4096,
-// so chunks fit 8 bits).  With the row supports ilo / ihi of the height
+// 128-channel tiles, as even as n_ct allows.  A record is (f, first operator
+// row, j0 | first tile << 16, nc | tiles << 9 | kc_lo << 12 | kc_hi << 20 |
+// ranged), all that the condensation needs to start its copies: the unit's
+// operator rows are zero outside the 32-column chunks [kc_lo, kc_hi] (K_pad <=
+// 4096, so chunks fit 8 bits; n <= 4096, at most 256 tiles).  With the row supports ilo / ihi of the height
 // analysis (single-level WSM; h x w the frame's grid) that range is the
 // chunks of the map rows the block's grid rows reach, else every chunk; and
 // for blocks of more than 64 tokens (two MMAs per step, see unit_fused) each
@@ -227,6 +228,7 @@ __device__ inline void unit_records(const Ctx &c, int64_t f, int n, int h = 0, i
     const int v = (int)(f / c.T);
     int4 *units = c.units + (size_t)v * c.max_units_v;
     int u0 = c.ustart[f];
+    const int wrow = c.woff[f];
     const int KC = c.K_pad >> 5;
     for (int j0 = 0; j0 < n; j0 += kColBlock) {
         if (j0 == kColBlock) u0 = c.ustartB[f];   // later blocks: the second part of the list
@@ -310,7 +312,8 @@ __device__ inline void unit_records(const Ctx &c, int64_t f, int n, int h = 0, i
             // tiles of group li: [li * n_ct / cnt, (li + 1) * n_ct / cnt), sizes differing by at most one
             const int ct = li * c.n_ct / cnt, ct1 = (li + 1) * c.n_ct / cnt;
             if (u0 + li < c.max_units_v)
-                units[u0 + li] = make_int4((int)f, j0, ct, nc | ((ct1 - ct) << 9) | (klo << 12) | (khi << 20) | ranged);
+                units[u0 + li] =
+                    make_int4((int)f, wrow + j0, j0 | (ct << 16), nc | ((ct1 - ct) << 9) | (klo << 12) | (khi << 20) | ranged);
         }
         u0 += cnt;
     }
