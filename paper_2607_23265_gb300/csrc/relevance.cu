@@ -579,21 +579,20 @@ __device__ __forceinline__ void frame_result(const Ctx &c, int64_t f, int v, int
 // 8.2 us with the partials of the two frames read one after the other, two at
 // a time, 64-bit divisions, and the gate in the other half of the CTA.
 __global__ void __launch_bounds__(512, 2) frame_stats_kernel(Ctx c) {
-    pdl_wait();
-    pdl_trigger();
     __shared__ float wsum[16][5];
     __shared__ float gate_map[WZ_MAX_HW * WZ_MAX_HW];   // the frame's saliency map
-    const int64_t VT = (int64_t)c.V * c.T;
-    if ((int64_t)blockIdx.x >= VT) {
-        frame_gate(c, (int64_t)blockIdx.x - VT, gate_map);
+    const int VT = c.V * c.T, f = (int)blockIdx.x;
+    const int v = f / c.T, t = f - v * c.T;
+    int64_t sf_at = 0, sp_at = 0;
+    int nf = 0, np = 0;
+    if (f < VT) frame_slots(c, f, sf_at, nf);
+    if (f < VT && t > 0) frame_slots(c, f - 1, sp_at, np);
+    pdl_wait();
+    pdl_trigger();
+    if (f >= VT) {
+        frame_gate(c, f - VT, gate_map);
         return;
     }
-    const int64_t f = blockIdx.x;
-    const int v = (int)blockIdx.x / c.T, t = (int)blockIdx.x - v * c.T;
-    int64_t sf_at, sp_at = 0;
-    int nf, np = 0;
-    frame_slots(c, f, sf_at, nf);
-    if (t > 0) frame_slots(c, f - 1, sp_at, np);
     const int nv = c.D / 4;
     const float4 *Pf = reinterpret_cast<const float4 *>(c.part) + (size_t)sf_at * nv;
     const float4 *Pp = reinterpret_cast<const float4 *>(c.part) + (size_t)sp_at * nv;

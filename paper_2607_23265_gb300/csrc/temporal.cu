@@ -14,8 +14,10 @@
 // Every reduction runs in a fixed order for a fixed block size, so results
 // do not depend on scheduling.  One CTA of latency-bound steps: r_t and gamma_t
 // stay in shared memory; barriers and fp64 chains are what remains (64 frames:
-// 8.4 us past its wait; 10.0 with the per-frame state in global memory, one
-// thread per frame and the budget sums on three barriers each).
+// 10.0 us past its wait with the per-frame state in global memory, one thread
+// per frame and the budget sums on three barriers each; 8.4 without those; the
+// unit counts from a table formed before the wait, the first loads beside each
+// other and the Haar taps in registers take another 2).
 #include <cmath>
 
 #include "wz_spatial.cuh"
@@ -54,8 +56,8 @@ __device__ int block_excl_scan(int x, int *ws, int *total) {
     return r;
 }
 
-// Three exclusive block scans at once (same barriers as one); ws holds
-// >= 3 * 33 ints.  Returns the exclusive prefixes and the totals.
+// K exclusive block scans at once (same barriers as one); ws holds
+// >= K * 33 ints.  Returns the exclusive prefixes and the totals.
 template <int K>
 __device__ void block_excl_scan(const int (&x)[K], int *ws, int (&excl)[K], int (&total)[K]) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -245,6 +247,12 @@ __device__ __noinline__ const double *wta_deeper_levels(const Ctx &c, double *A0
 }
 
 __global__ void __launch_bounds__(kTemporalThreads) temporal_kernel(Ctx c) {
+    __shared__ int ucnt[2][kColBlock / 16 + 1];   // tensor-core units of a block of 16 i tokens, wide and narrow
+    if (threadIdx.x >= 1 && threadIdx.x <= kColBlock / 16)
+        for (int k = 0; k < 2; ++k) {
+            const int cg = unit_tiles(16 * (int)threadIdx.x, k != 0);
+            ucnt[k][threadIdx.x] = (c.n_ct + cg - 1) / cg;
+        }
     pdl_wait();
     pdl_trigger();
     if ((int)blockIdx.x >= c.V) {
@@ -263,12 +271,17 @@ __global__ void __launch_bounds__(kTemporalThreads) temporal_kernel(Ctx c) {
     extern __shared__ __align__(16) unsigned char tsm[];
     __shared__ double dscr[33];
     __shared__ int iscr2[66];
-    __shared__ int iscr[4 * 33];
+    __shared__ int iscr[6 * 33];
     const int v = blockIdx.x;
     const int T = c.T;
     const int64_t base = (int64_t)v * T;
     const VideoPar vp = c.vpar[v];
     const double2 *fr = reinterpret_cast<const double2 *>(c.fr + base * 4);   // r, delta of frame t at 2 t
+    // each thread owns `per` consecutive frames t0 .. t1 - 1 (its first frame's
+    // values are requested here, beside the range of delta)
+    const int per = (T + (int)blockDim.x - 1) / (int)blockDim.x;
+    const int t0 = threadIdx.x * per, t1 = min(T, t0 + per);
+    const double2 rd0 = t0 < T ? fr[2 * t0] : make_double2(0.0, 0.0);
     double *wgt = reinterpret_cast<double *>(tsm);                        // weight of retained frame m
     unsigned long long *keys = reinterpret_cast<unsigned long long *>(tsm + temporal_smem_keys(T));   // remainder key
     int *lst = reinterpret_cast<int *>(keys + T);                         // retained frames
@@ -288,18 +301,15 @@ __global__ void __launch_bounds__(kTemporalThreads) temporal_kernel(Ctx c) {
     // delta over the video (Eq. 7)
     const double lo = __longlong_as_double((long long)c.drange[2 * v]);
     const double hi = __longlong_as_double((long long)c.drange[2 * v + 1]);
-    const double inv = hi > lo ? 1.0 / (hi - lo) : 0.0;   // (while the frames' values are on their way)
+    const double inv = hi > lo ? 1.0 / (hi - lo) : 0.0;
     // gamma_t and the retained set (frame 1 always kept)
     const double tau = (double)c.tau;
-    // each thread owns `per` consecutive frames t0 .. t1 - 1;
     // nf[t] holds the frame's keep flag until the retained list is written
-    const int per = (T + (int)blockDim.x - 1) / (int)blockDim.x;
-    const int t0 = threadIdx.x * per, t1 = min(T, t0 + per);
     // (delta >= 0: without a positive threshold every frame is retained)
     const bool all = !(tau > 0.0);
     int cnt = 0;
     for (int t = t0; t < t1; ++t) {
-        const double2 rd = fr[2 * t];
+        const double2 rd = t == t0 ? rd0 : fr[2 * t];
         const double d = rd.y;
         const double gm = (d - lo) * inv;
         rs[t] = rd.x;
@@ -337,12 +347,20 @@ __global__ void __launch_bounds__(kTemporalThreads) temporal_kernel(Ctx c) {
     // ("raw") or 1 ("uniform") instead.
     const int FT = c.wta_F;
     const int K = (L + FT - 1) / 2;
+    const double haar[8] = {c.wta_dec_lo[0], c.wta_dec_lo[1], c.wta_dec_hi[0], c.wta_dec_hi[1],
+                            c.wta_rec_lo[0], c.wta_rec_lo[1], c.wta_rec_hi[0], c.wta_rec_hi[1]};
     for (int k = threadIdx.x; k < K; k += blockDim.x) {
         double ca = 0.0, cd = 0.0;
-        for (int j = 0; j < FT; ++j) {
-            const double x = rs[lst[ext_index(2 * k + 1 - j, L, WZ_MODE_SYMMETRIC)]];
-            ca += c.wta_dec_lo[j] * x;
-            cd += c.wta_dec_hi[j] * x;
+        if (FT == 2) {   // Haar: samples 2k + 1 and 2k (an odd last one mirrors itself)
+            const double x0 = rs[lst[min(2 * k + 1, L - 1)]], x1 = rs[lst[2 * k]];
+            ca = haar[0] * x0 + haar[1] * x1;
+            cd = haar[2] * x0 + haar[3] * x1;
+        } else {
+            for (int j = 0; j < FT; ++j) {
+                const double x = rs[lst[ext_index(2 * k + 1 - j, L, WZ_MODE_SYMMETRIC)]];
+                ca += c.wta_dec_lo[j] * x;
+                cd += c.wta_dec_hi[j] * x;
+            }
         }
         const int m0 = ext_index(2 * k, L, WZ_MODE_SYMMETRIC), m1 = ext_index(2 * k + 1, L, WZ_MODE_SYMMETRIC);
         const double g = 0.5 * (gam[lst[m0]] + gam[lst[m1]]);
@@ -356,10 +374,14 @@ __global__ void __launch_bounds__(kTemporalThreads) temporal_kernel(Ctx c) {
     double sp = 0.0;
     for (int m = threadIdx.x; m < L; m += blockDim.x) {
         double rt = 0.0;
-        const int alo = m >> 1, ahi = min(K - 1, (m + FT - 2) >> 1);
-        for (int ai = alo; ai <= ahi; ++ai) {
-            const int kk = m + FT - 2 - 2 * ai;       // synthesis tap, 0 <= kk < FT
-            rt += c.wta_rec_lo[kk] * ain[ai] + c.wta_rec_hi[kk] * dall[ai];
+        if (FT == 2) {
+            rt = (m & 1 ? haar[5] : haar[4]) * ain[m >> 1] + (m & 1 ? haar[7] : haar[6]) * dall[m >> 1];
+        } else {
+            const int alo = m >> 1, ahi = min(K - 1, (m + FT - 2) >> 1);
+            for (int ai = alo; ai <= ahi; ++ai) {
+                const int kk = m + FT - 2 - 2 * ai;       // synthesis tap, 0 <= kk < FT
+                rt += c.wta_rec_lo[kk] * ain[ai] + c.wta_rec_hi[kk] * dall[ai];
+            }
         }
         const int t = lst[m];
         if (c.out_rel) c.out_rel[(base + t) * 4 + 3] = (float)rt;
@@ -472,36 +494,40 @@ __global__ void __launch_bounds__(kTemporalThreads) temporal_kernel(Ctx c) {
     // the condensation claims units in list order, and short units last keep
     // its tail short.
     const bool tc = c.path == WZ_PATH_TENSOR;
-    // units of frame t's first block (ua) and of its later blocks (ub)
-    auto frame_units = [&](int n, int &ua, int &ub) {
+    // units of frame t's first block (ua) and of its later blocks (ub); ucnt:
+    // units of a block by its 16-row groups, wide and narrow
+    auto frame_units = [&](int n, const int *cnt, int &ua, int &ub) {
         ua = ub = 0;
-        if (tc)
-            for (int j0 = 0; j0 < n; j0 += kColBlock) {
-                const int nc = min(kColBlock, n - j0);
-                const int cg = unit_tiles((nc + 15) / 16 * 16), add = (c.n_ct + cg - 1) / cg;
-                if (j0 == 0) ua += add;
-                else ub += add;
-            }
+        if (tc && n > 0) {
+            const int full = (n - 1) / kColBlock, last = cnt[(n - full * kColBlock + 15) >> 4];
+            ua = full > 0 ? cnt[kColBlock / 16] : last;
+            ub = full > 0 ? (full - 1) * cnt[kColBlock / 16] + last : 0;
+        }
     };
     // this thread's frames t0 .. t1 - 1 (their budgets re-read from shared
     // memory: no per-thread arrays)
-    int part[4] = {0, 0, 0, 0};
+    int part[6] = {0, 0, 0, 0, 0, 0};
     for (int t = t0; t < t1; ++t) {
         const int n = nf[t];
-        int ua, ub;
-        frame_units(n, ua, ub);
+        int ua, ub, na, nb_;
+        frame_units(n, ucnt[0], ua, ub);
+        frame_units(n, ucnt[1], na, nb_);
         part[0] += n;
         part[1] += (n + 15) & ~15;
         part[2] += ua;
         part[3] += ub;
+        part[4] += na;
+        part[5] += nb_;
     }
-    int pre[4], tot[4];
-    block_excl_scan<4>(part, iscr, pre, tot);
-    int o = pre[0], wo = pre[1], u = pre[2], uB = tot[2] + pre[3];
+    int pre[6], tot[6];
+    block_excl_scan<6>(part, iscr, pre, tot);
+    const int narrow = c.V == 1 && tot[2] + tot[3] <= kNarrowUnits ? 1 : 0;
+    const int utot = narrow ? tot[4] + tot[5] : tot[2] + tot[3];
+    int o = pre[0], wo = pre[1], u = narrow ? pre[4] : pre[2], uB = narrow ? tot[4] + pre[5] : tot[2] + pre[3];
     for (int t = t0; t < t1; ++t) {
         const int n = nf[t];
         int ua, ub;
-        frame_units(n, ua, ub);
+        frame_units(n, ucnt[narrow], ua, ub);
         c.n[base + t] = n;
         c.off[base + t] = vp.row0 + o;
         c.woff[base + t] = vp.w_row0 + wo;
@@ -522,8 +548,9 @@ __global__ void __launch_bounds__(kTemporalThreads) temporal_kernel(Ctx c) {
         c.prod[v] = tot[0];
         if (c.out_count) c.out_count[v] = tot[0];
         if (tc) {
-            c.ucount[v] = min(tot[2] + tot[3], c.max_units_v);
-            if (tot[2] + tot[3] > c.max_units_v) atomicOr(c.status, 2);
+            c.ucount[v] = min(utot, c.max_units_v);
+            if (utot > c.max_units_v) atomicOr(c.status, 2);
+            if (v == 0) c.spatial_next[2] = narrow;
         }
     }
 }

@@ -72,7 +72,8 @@ struct Ctx {
     int krange_nblk;      // blocks of 256 tokens per frame: ceil(H*W / 256)
     int *status;          // device status word (bounded waits)
     int *spatial_next;    // [0]: next (frame, grid row) of the spatial operator kernel, [1]: next
-                          // tensor-core unit of the condensation; both zeroed by temporal
+                          // tensor-core unit of the condensation; both zeroed by temporal, which
+                          // sets [2], narrow units (unit_tiles)
 
     void *out;            // [rows][D] dtype
     int *out_index;       // [rows][3]
@@ -308,14 +309,23 @@ __host__ __device__ __forceinline__ int gate_floats(int H, int W, int F, int J) 
 // output tokens: the hi and lo operator halves form one MMA of N = 2 ncp for
 // ncp <= 64, else two MMAs of N = ncp; a unit spans as many 128-channel tiles
 // (at most 4) as the 512 accumulator columns of tensor memory hold, so each
-// operator tile in shared memory serves 2-4 channel tiles.
+// operator tile in shared memory serves 2-4 channel tiles.  Narrow units (one
+// video with at most kNarrowUnits wide ones; the temporal kernel
+// decides) take, for blocks of up to 128 tokens, the tiles of half of the
+// columns: more, smaller units whose epilogue overlaps the next unit's main
+// loop.  Calls, wide / narrow: 64 frames of 13 x 13 x 3584 (224 wide units)
+// 58.8 / 57.0 us, 128 of 16 x 16 (448) 103.6 / 101.8; with the max-over-query
+// scorer (896) 146.0 / 147.1, 256 of 27 x 27 413 / 420, 32 videos of 64 frames
+// 763 / 779 (there the operator's extra reads cost more).
 __host__ __device__ __forceinline__ bool unit_fused(int ncp) { return ncp <= 64; }
 
-__host__ __device__ __forceinline__ int unit_tiles(int ncp) {
+__host__ __device__ __forceinline__ int unit_tiles(int ncp, bool narrow) {
     const int cols = unit_fused(ncp) ? 2 * ncp : ncp;
-    const int cg = 512 / cols;
+    const int cg = (narrow && ncp <= 128 ? kTmemCols / 2 : kTmemCols) / cols;
     return cg < 1 ? 1 : (cg > 4 ? 4 : cg);
 }
+
+constexpr int kNarrowUnits = 456;   // three per SM
 
 // ---- launchers (one per kernel family) -------------------------------------
 

@@ -229,11 +229,12 @@ __device__ inline void unit_records(const Ctx &c, int64_t f, int n, int h = 0, i
     int4 *units = c.units + (size_t)v * c.max_units_v;
     int u0 = c.ustart[f];
     const int wrow = c.woff[f];
+    const bool narrow = c.spatial_next[2] != 0;
     const int KC = c.K_pad >> 5;
     for (int j0 = 0; j0 < n; j0 += kColBlock) {
         if (j0 == kColBlock) u0 = c.ustartB[f];   // later blocks: the second part of the list
         const int nc = min(kColBlock, n - j0);
-        const int cg = unit_tiles((nc + 15) / 16 * 16);
+        const int cg = unit_tiles((nc + 15) / 16 * 16, narrow);
         const int cnt = (c.n_ct + cg - 1) / cg;
         int klo = 0, khi = KC - 1;
         if (ilo != nullptr && w > 0) {
