@@ -44,7 +44,6 @@ struct TcSmem {
     int G;       // [hp][wp]: the item's frame gate
     int P;       // [16][2][BMAX]: P_L, P_H of row t's grid row at a = a0(t) + k
     int Q;       // [16][2][BMAX]: Q_L, Q_H of row t's grid column at b = b0(t) + k
-    int tok;     // [16][8] int: per row t (see kTok*)
     int stage;   // [2][KC][512] bf16: the group's hi chunks, then its lo chunks
     int rec;     // [2][kMaxTaps]: the synthesis taps (lanes index them differently)
     int total;
@@ -61,15 +60,11 @@ struct TcSmem {
         G = take(L.hp * L.wp, 4);
         P = take(kTcRows * 2 * bmax, 4);
         Q = take(kTcRows * 2 * bmax, 4);
-        tok = take(kTcRows * 8, 4);
         rec = take(2 * kMaxTaps, 4);
         stage = take((L.K_pad >> 5) * kTcChunkBytes * 2 / 4, 32);   // 128-byte aligned
         total = o;
     }
 };
-
-// Per-row ints of TcSmem::tok.
-enum { kTokA0 = 0, kTokNA, kTokB0, kTokNB, kTokZlo, kTokSpan, kTokJ4 };
 
 // Operator entries (row t of the group, columns k ...) as bf16 hi and lo
 // halves in the staged tiled layout: chunk k / 32, then the 8-row group, then
@@ -151,7 +146,6 @@ __global__ void __launch_bounds__(kSpatialThreads, BMAX <= 6 ? 3 : 2)
     const int *jlo = reinterpret_cast<const int *>(sm + L.jlo), *jhi = reinterpret_cast<const int *>(sm + L.jhi);
     const int *ilo = reinterpret_cast<const int *>(sm + L.ilo), *ihi = reinterpret_cast<const int *>(sm + L.ihi);
     float *G = sm + S.G, *Pt = sm + S.P, *Qt = sm + S.Q;
-    int *tok = reinterpret_cast<int *>(sm + S.tok);
     unsigned char *stg = reinterpret_cast<unsigned char *>(sm + S.stage);
     __nv_bfloat16 *shi = reinterpret_cast<__nv_bfloat16 *>(stg);
     const int KC = L.K_pad >> 5, WP4 = L.WP4;
@@ -202,19 +196,24 @@ __global__ void __launch_bounds__(kSpatialThreads, BMAX <= 6 ? 3 : 2)
             const int k = tid + r * kSpatialThreads;
             gr[r] = k < ng ? Gf[k] : 0.f;
         }
+        // row t: token j of the frame, grid cell (p, q); the bilinear row and
+        // column through the synthesis (P_u[p, a], Q_v[q, b] for the na and nb
+        // coefficients from a0, b0) and the map rows zlo .. zlo + span - 1 and
+        // column quads j4lo .. j4hi that the row reaches; every thread of the
+        // row holds these
+        const int j = kTcRows * g + t;
+        const bool valid = j < n;
+        const int p = valid ? j / w : 0, q = valid ? j - p * w : 0;
+        int a0, na, b0, nb, zlo, span, j4lo, j4hi;
         {
-            // row t: token j of the frame, grid cell (p, q); the bilinear row
-            // and column through the synthesis (P_u[p, a], Q_v[q, b]) and the
-            // map rows and columns the row reaches
-            const int j = kTcRows * g + t;
-            const bool valid = j < n;
-            const int p = valid ? j / w : 0, q = valid ? j - p * w : 0;
-            int y0, y1, x0, x1, a0, a1, b0, b1;
+            int y0, y1, x0, x1, a1, b1;
             float ly, lx;
             bilinear_src(p, H, h, y0, y1, ly);
             bilinear_src(q, W, w, x0, x1, lx);
             synth_support(y0, y1, F, hp, a0, a1);
             synth_support(x0, x1, F, wp, b0, b1);
+            na = min(a1 - a0 + 1, BMAX);
+            nb = min(b1 - b0 + 1, BMAX);
             if (s < BMAX) {
                 const int a = a0 + s, b = b0 + s;
                 float *P = Pt + t * 2 * BMAX, *Q = Qt + t * 2 * BMAX;
@@ -223,32 +222,25 @@ __global__ void __launch_bounds__(kSpatialThreads, BMAX <= 6 ? 3 : 2)
                 Q[s] = b <= b1 ? (1.f - lx) * synth(rec_lo, F, x0, b) + lx * synth(rec_lo, F, x1, b) : 0.f;
                 Q[BMAX + s] = b <= b1 ? (1.f - lx) * synth(rec_hi, F, x0, b) + lx * synth(rec_hi, F, x1, b) : 0.f;
             }
-            if (s == 0) {
-                const int na = min(a1 - a0 + 1, BMAX), nb = min(b1 - b0 + 1, BMAX);
-                int zlo = H, zhi = -1, jl = WP4, jh = -1;
-                for (int u = 0; u < na; ++u) {
-                    zlo = min(zlo, ilo[a0 + u]);
-                    zhi = max(zhi, ihi[a0 + u]);
-                }
-                for (int bb = 0; bb < nb; ++bb) {
-                    jl = min(jl, jlo[b0 + bb]);
-                    jh = max(jh, jhi[b0 + bb]);
-                }
-                int *T = tok + 8 * t;
-                T[kTokA0] = a0;
-                T[kTokNA] = na;
-                T[kTokB0] = b0;
-                T[kTokNB] = nb;
-                T[kTokZlo] = zlo;
-                T[kTokSpan] = valid && jh >= 0 ? max(0, zhi - zlo + 1) : 0;
-                T[kTokJ4] = jh >= 0 ? (jl >> 2) | ((jh >> 2) << 16) : 0;
-                const int64_t row = (int64_t)fdat[3 * f + 1] + j;
-                if (valid && wz_in_range(c.status, row < c.rows_total)) {
-                    int *o = c.out_index + (size_t)row * 3;
-                    o[0] = f % c.T;
-                    o[1] = p;
-                    o[2] = q;
-                }
+            // lane s of the row's half-warp holds coefficient s's supports;
+            // first rows and columns and 63 - the last ones as bytes, all
+            // minima (H, W <= 64, an empty support has 63 - last = 64)
+            const int sa = s < na ? a0 + s : a0, sb = s < nb ? b0 + s : b0;
+            uint32_t lim = (uint32_t)ilo[sa] | (uint32_t)(63 - ihi[sa]) << 8 | (uint32_t)jlo[sb] << 16 |
+                           (uint32_t)(63 - jhi[sb]) << 24;
+#pragma unroll
+            for (int o = 8; o > 0; o >>= 1) lim = __vminu4(lim, __shfl_xor_sync(0xffffffffu, lim, o));
+            zlo = (int)(lim & 0xffu);
+            const int zhi = 63 - (int)(lim >> 8 & 0xffu), jl = (int)(lim >> 16 & 0xffu), jh = 63 - (int)(lim >> 24);
+            span = valid && jh >= 0 ? max(0, zhi - zlo + 1) : 0;
+            j4lo = jl >> 2;
+            j4hi = jh >> 2;   // (jh < 0: span is 0)
+            const int64_t row = (int64_t)fdat[3 * f + 1] + j;
+            if (s == 0 && valid && wz_in_range(c.status, row < c.rows_total)) {
+                int *o = c.out_index + (size_t)row * 3;
+                o[0] = f % c.T;
+                o[1] = p;
+                o[2] = q;
             }
         }
 #pragma unroll
@@ -268,10 +260,6 @@ __global__ void __launch_bounds__(kSpatialThreads, BMAX <= 6 ? 3 : 2)
         }
         __syncthreads();   // the stage is clear; G, P, Q and the row data are in place
         {
-            const int *T = tok + 8 * t;
-            const int span = T[kTokSpan];
-            const int a0 = T[kTokA0], na = T[kTokNA], b0 = T[kTokB0], nb = T[kTokNB], zlo = T[kTokZlo];
-            const int j4lo = T[kTokJ4] & 0xffff, j4hi = T[kTokJ4] >> 16;
             const float *P = Pt + t * 2 * BMAX, *Q = Qt + t * 2 * BMAX;
             for (int ri = s; ri < span; ri += 16) {
                 const int i = zlo + ri;
