@@ -347,7 +347,7 @@ int run_condense(const CondenseRequest &r) {
     c.out_count = r.out_count;
     c.out_rel = r.out_relevance;
     if (r.device_status) c.status = r.device_status;
-    else WZ_CUDA(cudaMemsetAsync(c.status, 0, sizeof(int), r.stream));
+    else c.clear_status = 1;
     c.G1 = relevance_grid(c);
     if (c.G1 < 1) {
         cudaGetLastError();
@@ -825,7 +825,7 @@ int wz_relevance(const void *features, int T, int H, int W, int D, int dtype, co
     // a bounded wait that gives up reports to the caller's status word, else
     // to the workspace's, which starts each call at zero
     if (device_status) c.status = device_status;
-    else WZ_CUDA(cudaMemsetAsync(c.status, 0, sizeof(int), cs));
+    else c.clear_status = 1;
     WZ_CUDA(launch_query_pool(c, &par, cs));
     WZ_CUDA(launch_relevance_pass(c, cs));
     WZ_CUDA(launch_frame_stats(c, cs));
@@ -853,13 +853,11 @@ int wz_project(const wz_project_args *a) {
     int st = ws.acquire(a->workspace, a->workspace_bytes, need, s);
     if (st != WZ_OK) return st;
     int *status = a->device_status;
-    if (!status) {
-        status = reinterpret_cast<int *>(ws.ptr + align_up((size_t)a->B * (size_t)a->C * 2));
-        WZ_CUDA(cudaMemsetAsync(status, 0, sizeof(int), s));
-    }
+    const bool own = !status;
+    if (own) status = reinterpret_cast<int *>(ws.ptr + align_up((size_t)a->B * (size_t)a->C * 2));
     const int M = (int)a->B;
-    WZ_CUDA(launch_project_gemm(a->tokens, M, a->D, a->w1, a->C, a->b1, ws.ptr, true, status, false, s));
-    WZ_CUDA(launch_project_gemm(ws.ptr, M, a->C, a->w2, a->E, a->b2, a->out, false, status, true, s));
+    WZ_CUDA(launch_project_gemm(a->tokens, M, a->D, a->w1, a->C, a->b1, ws.ptr, true, status, own, false, s));
+    WZ_CUDA(launch_project_gemm(ws.ptr, M, a->C, a->w2, a->E, a->b2, a->out, false, status, false, true, s));
     return WZ_OK;
 }
 

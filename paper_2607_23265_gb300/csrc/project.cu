@@ -82,6 +82,7 @@ struct PArgs {
     float *a;
     int Lq, Lqp;
     int *status;
+    int clear_status;    // zero it first (a wait that gives up does so seconds later)
 };
 
 __device__ __forceinline__ void pfail(const PArgs &p, volatile int *abort_flag, int code) {
@@ -176,6 +177,7 @@ project_pair_kernel(const __grid_constant__ PMaps maps, PArgs p) {
     }
     pdl_wait();   // A may be the previous grid's output
     pdl_trigger();
+    if (p.clear_status && blockIdx.x == 0 && threadIdx.x == 0) *p.status = 0;
     __syncthreads();
     ptx::cluster_sync();   // both CTAs' barriers are ready
     ptx::tc_fence_after();
@@ -326,6 +328,7 @@ project_gemm_kernel(const __grid_constant__ PMaps maps, PArgs p) {
     }
     pdl_wait();   // A may be the previous grid's output
     pdl_trigger();
+    if (p.clear_status && blockIdx.x == 0 && threadIdx.x == 0) *p.status = 0;
     __syncthreads();
     ptx::tc_fence_after();
     const uint32_t tmem = S->tmem_base;
@@ -503,7 +506,7 @@ PShape project_shape(int M, int N, int sms) {
 // Out[M][N] = act(A[M][K] B[N][K]^T + bias): K and N multiples of 64, 16-byte
 // aligned rows; launched with programmatic stream serialization when pdl.
 cudaError_t launch_project_gemm(const void *A, int M, int K, const void *B, int N, const float *bias, void *out,
-                                bool gelu, int *status, bool pdl, cudaStream_t s) {
+                                bool gelu, int *status, bool clear_status, bool pdl, cudaStream_t s) {
     if (M < 1) return cudaSuccess;
     auto enc = tmap_encode_fn();
     if (!enc) return cudaErrorNotSupported;
@@ -520,6 +523,7 @@ cudaError_t launch_project_gemm(const void *A, int M, int K, const void *B, int 
     PArgs p{};
     p.M = M; p.N = N; p.K = K; p.tileN = shape.tileN;
     p.bias = bias; p.out = static_cast<__nv_bfloat16 *>(out); p.gelu = gelu ? 1 : 0; p.status = status;
+    p.clear_status = clear_status ? 1 : 0;
     void *args[] = {&maps, &p};
     if (shape.pair) {
         e = cudaFuncSetAttribute(project_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPairSmemBytes);

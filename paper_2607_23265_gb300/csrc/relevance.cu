@@ -39,6 +39,7 @@ struct VideoParBlock {
 // What every kernel after the first one reads of video v.
 __device__ __forceinline__ void video_init(const Ctx &c, int v, const VideoPar &vp) {
     c.vpar[v] = vp;
+    if (v == 0 && c.clear_status) *c.status = 0;   // (a wait that gives up does so seconds later)
     if (c.drange) {   // empty range of delta_t, filled by frame_stats
         c.drange[2 * v] = 0x7ff0000000000000ull;   // +inf
         c.drange[2 * v + 1] = 0ull;                // +0

@@ -16,7 +16,7 @@
 // up once per device with cudaGetSymbolAddress (with that device current) on
 // the first call made on that device, and passed to the kernels.  A 16-byte
 // slot of the array is the status word of the bounded waits when the caller
-// passes none; it is zeroed on the stream at every call.
+// passes none; the first kernel of every call zeroes it.
 #include <mutex>
 
 #include "wz_internal.cuh"
@@ -122,8 +122,8 @@ extern "C" int wz_relevance_static(const void *features, int T, int H, int W, in
     c.L1 = ((int64_t)T * c.N + c.G1 - 1) / c.G1;
 
     // Carve the fixed array.  Every byte the kernels read is written earlier
-    // in the same call, except the status word, which is cleared below when
-    // the caller passes none.
+    // in the same call; the status word is cleared there when the caller
+    // passes none.
     const ScratchLayout o = scratch_layout(T, D, c.G1);
     if (o.total > (size_t)WZ_STATIC_SCRATCH_BYTES) return WZ_ERR_WORKSPACE;
 
@@ -138,9 +138,9 @@ extern "C" int wz_relevance_static(const void *features, int T, int H, int W, in
     c.fr = reinterpret_cast<double *>(b + o.fr);
     // The bounded waits of the relevance pass (and the index checks of the
     // checked build) record failures in a status word: the caller's, else
-    // the array's own slot, zeroed on the stream (cudaMemsetAsync allocates
-    // nothing).
+    // the array's own slot, zeroed by the first kernel.
     c.status = device_status ? device_status : reinterpret_cast<int *>(b + o.status);
+    c.clear_status = device_status ? 0 : 1;
     c.X = features;
     c.Q = query;
     c.a = token_scores;
@@ -149,8 +149,7 @@ extern "C" int wz_relevance_static(const void *features, int T, int H, int W, in
 
     const VideoPar par{0, Lq, 0, 0, 0};
     const cudaStream_t s = (cudaStream_t)stream;
-    if ((!device_status && cudaMemsetAsync(c.status, 0, sizeof(int), s) != cudaSuccess) ||
-        launch_query_pool(c, &par, s) != cudaSuccess || launch_relevance_pass(c, s) != cudaSuccess ||
+    if (launch_query_pool(c, &par, s) != cudaSuccess || launch_relevance_pass(c, s) != cudaSuccess ||
         launch_frame_stats(c, s) != cudaSuccess) {
         cudaGetLastError();
         return WZ_ERR_CUDA;

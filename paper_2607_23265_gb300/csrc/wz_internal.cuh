@@ -71,6 +71,7 @@ struct Ctx {
                           // reach a 32-token chunk: [16*(r & 0xff), 16*(r >> 8)) (tensor path)
     int krange_nblk;      // blocks of 256 tokens per frame: ceil(H*W / 256)
     int *status;          // device status word (bounded waits)
+    int clear_status;     // the call's first kernel zeroes it (the workspace's own word)
     int *spatial_next;    // [0]: next (frame, grid row) of the spatial operator kernel, [1]: next
                           // tensor-core unit of the condensation; both zeroed by temporal, which
                           // sets [2], narrow units (unit_tiles)
@@ -340,7 +341,7 @@ PFN_cuTensorMapEncodeTiled_v12000 tmap_encode_fn();
 cudaError_t launch_spatial_ml(const Ctx &c, cudaStream_t s);
 size_t spatial_ml_smem_bytes(int H, int W, int F, int J);   // 0 if the layout does not fit
 cudaError_t launch_project_gemm(const void *A, int M, int K, const void *B, int N, const float *bias, void *out,
-                                bool gelu, int *status, bool pdl, cudaStream_t s);
+                                bool gelu, int *status, bool clear_status, bool pdl, cudaStream_t s);
 // Max-over-query relevance in one pass over the features (maxsim.cu): token
 // norms, channel-sum partials and a_{t,n}, in place of the relevance pass and
 // the max-over-query GEMM.
