@@ -485,12 +485,12 @@ __global__ void __launch_bounds__(MAXTHREADS, 1) relevance_pass_kernel(Ctx c, Re
 // Gate of the WSM for frame f (Eq. 6, Eq. 12): the saliency map M = min-max
 // normalised a_{t,n} over the frame, average-pooled to the subband grid of
 // each DWT level (hp x wp for the first) and scaled by lambda.  Called by a
-// whole CTA beside those that form the frame statistics, so that the two chains
-// overlap.
-__device__ void frame_gate(const Ctx &c, int64_t f, float *M2) {
-    const int t0 = threadIdx.x, nth = blockDim.x;
-    __shared__ float red2[32];
-    const int N = c.N, H = c.H, W = c.W, lane = t0 & 31, w = t0 >> 5, nw = nth >> 5;
+// whole CTA, or by a warp (M2 its own map), beside those that form the frame
+// statistics, so that the two chains overlap.
+template <bool WARP>
+__device__ __forceinline__ void frame_gate(const Ctx &c, int64_t f, float *M2) {
+    const int t0 = WARP ? threadIdx.x & 31 : threadIdx.x, nth = WARP ? 32 : blockDim.x;
+    const int N = c.N, H = c.H, W = c.W;
     const float *a = (c.ext_a ? c.ext_a : c.a) + f * N;
     float lo = INFINITY, hi = -INFINITY;
     for (int k = t0; k < N; k += nth) {
@@ -503,20 +503,25 @@ __device__ void frame_gate(const Ctx &c, int64_t f, float *M2) {
         lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
         hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
     }
-    if (lane == 0) {
-        red2[w] = lo;
-        red2[16 + w] = hi;
-    }
-    __syncthreads();
-    lo = INFINITY;
-    hi = -INFINITY;
-    for (int k = 0; k < nw; ++k) {
-        lo = fminf(lo, red2[k]);
-        hi = fmaxf(hi, red2[16 + k]);
+    if constexpr (!WARP) {
+        __shared__ float red2[32];
+        const int lane = t0 & 31, w = t0 >> 5, nw = nth >> 5;
+        if (lane == 0) {
+            red2[w] = lo;
+            red2[16 + w] = hi;
+        }
+        __syncthreads();
+        lo = INFINITY;
+        hi = -INFINITY;
+        for (int k = 0; k < nw; ++k) {
+            lo = fminf(lo, red2[k]);
+            hi = fmaxf(hi, red2[16 + k]);
+        }
     }
     const float rng = hi - lo;
     for (int k = t0; k < N; k += nth) M2[k] = rng > 0.f ? (M2[k] - lo) / rng : 0.f;
-    __syncthreads();
+    if constexpr (WARP) __syncwarp();
+    else __syncthreads();
     for (int l = 1; l <= c.wsm_levels; ++l) {
         const int hp = c.lvl_h[l], wp = c.lvl_w[l];
         if (!wz_in_range(c.status, c.goff[l - 1] + hp * wp <= c.gate_stride)) break;
@@ -531,6 +536,20 @@ __device__ void frame_gate(const Ctx &c, int64_t f, float *M2) {
             G[k] = c.lambda * (s / (float)((r1 - r0) * (c1 - c0)));
         }
     }
+}
+
+// The gates of a batch of many frames: CTA b of its kernel's gate CTAs forms
+// one, or, where a frame has at most kWarpGateTokens tokens (gate_warps), one
+// per warp.
+constexpr int kWarpGateTokens = 512;
+
+__device__ __forceinline__ void frame_gates(const Ctx &c, int b, int gate_warps, float *map) {
+    if (!gate_warps) {
+        frame_gate<false>(c, b, map);
+        return;
+    }
+    const int warp = threadIdx.x >> 5, f = b * (int)(blockDim.x >> 5) + warp;
+    if (f < c.V * c.T) frame_gate<true>(c, f, map + warp * kWarpGateTokens);
 }
 
 // The column partials of frame f: slots [slot, slot + cnt) (CTA c of the
@@ -569,6 +588,32 @@ __device__ __forceinline__ void frame_result(const Ctx &c, int64_t f, int v, int
     }
 }
 
+// Channels 4 i .. 4 i + 3 of the sums of FPB + 1 frames: the first two partials
+// of every frame in flight together, further ones (frames of more than two
+// CTAs' tokens) after them, in slot order.
+template <int FPB>
+__device__ __forceinline__ void partial_sums(const float4 *P, int nv, int i, const int (&slot)[FPB + 1],
+                                             const int (&cnt)[FPB + 1], float4 (&sf)[FPB + 1]) {
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    float4 y[FPB + 1];
+#pragma unroll
+    for (int k = 0; k <= FPB; ++k) {
+        sf[k] = cnt[k] > 0 ? P[(size_t)slot[k] * nv + i] : zero;
+        y[k] = cnt[k] > 1 ? P[(size_t)(slot[k] + 1) * nv + i] : zero;
+    }
+#pragma unroll
+    for (int k = 0; k <= FPB; ++k) {
+        sf[k].x += y[k].x; sf[k].y += y[k].y; sf[k].z += y[k].z; sf[k].w += y[k].w;
+#pragma unroll 1
+        for (int q = 2; q < cnt[k]; q += 2) {
+            const float4 x = P[(size_t)(slot[k] + q) * nv + i];
+            const float4 z = q + 1 < cnt[k] ? P[(size_t)(slot[k] + q + 1) * nv + i] : zero;
+            sf[k].x += x.x; sf[k].y += x.y; sf[k].z += x.z; sf[k].w += x.w;
+            sf[k].x += z.x; sf[k].y += z.y; sf[k].z += z.z; sf[k].w += z.w;
+        }
+    }
+}
+
 // One CTA per frame: the frame sums (fixed list of CTA partials) for all
 // channels, read as 16-byte vectors, up to four partials of the frame and four
 // of the one before it in flight; fp32 products summed over each thread's
@@ -591,7 +636,7 @@ __global__ void __launch_bounds__(512, 2) frame_stats_kernel(Ctx c) {
     pdl_wait();
     pdl_trigger();
     if (f >= VT) {
-        frame_gate(c, f - VT, gate_map);
+        frame_gate<false>(c, f - VT, gate_map);
         return;
     }
     const int nv = c.D / 4;
@@ -662,6 +707,95 @@ __global__ void __launch_bounds__(512, 2) frame_stats_kernel(Ctx c) {
     }
 }
 
+// The same for many frames: a CTA takes FPB consecutive frames of one video
+// (ceil(T / FPB) CTAs per video), so that a frame's partials are read once
+// instead of twice and the frames' loads are in flight together; the same sums
+// in the same order.  The gates are formed by further CTAs, a warp each where
+// a frame is small.  2048 frames of 13 x 13 x 3584 with gates: 20.5 us (cold),
+// 31.1 with a CTA per frame and per gate (6.7 waves of them).
+constexpr int kStatsThreads = 256;   // of the kernels with several frames per CTA
+constexpr int kStatsFrames = 4;
+
+template <int FPB>
+__global__ void __launch_bounds__(kStatsThreads, 3) frame_stats_many_kernel(Ctx c, int gate_warps) {
+    constexpr int NW = kStatsThreads / 32, NQ = 3 * FPB + 2;   // vq, vv, vp of each frame; qq, the first pp
+    __shared__ float wsum[NW][NQ];
+    __shared__ float gate_map[WZ_MAX_HW * WZ_MAX_HW];
+    static_assert(NW * kWarpGateTokens <= WZ_MAX_HW * WZ_MAX_HW && FPB <= NW, "a map and a frame per warp");
+    const int per_video = (c.T + FPB - 1) / FPB, nstat = c.V * per_video;
+    const int v = (int)blockIdx.x / per_video, t0 = ((int)blockIdx.x - v * per_video) * FPB;
+    const int nf = min(FPB, c.T - t0);
+    const int64_t f0 = (int64_t)v * c.T + t0;
+    // the column partials of frame f0 - 1 + k
+    int slot[FPB + 1], cnt[FPB + 1];
+#pragma unroll
+    for (int k = 0; k <= FPB; ++k) {
+        int64_t at = 0;
+        cnt[k] = 0;
+        if ((int)blockIdx.x < nstat && (k > 0 || t0 > 0) && k <= nf) frame_slots(c, f0 - 1 + k, at, cnt[k]);
+        slot[k] = (int)at;   // < G1 + V T
+    }
+    pdl_wait();
+    pdl_trigger();
+    if ((int)blockIdx.x >= nstat) {
+        frame_gates(c, (int)blockIdx.x - nstat, gate_warps, gate_map);
+        return;
+    }
+    const int nv = c.D / 4;
+    const float4 *P = reinterpret_cast<const float4 *>(c.part);
+    const float4 *Qv = reinterpret_cast<const float4 *>(c.qbar32 + (size_t)v * c.D);
+    float acc[NQ];
+#pragma unroll
+    for (int k = 0; k < NQ; ++k) acc[k] = 0.f;
+    auto dot4 = [](const float4 &a, const float4 &b, float s) {
+        return fmaf(a.x, b.x, fmaf(a.y, b.y, fmaf(a.z, b.z, fmaf(a.w, b.w, s))));
+    };
+#pragma unroll 1
+    for (int i = threadIdx.x; i < nv; i += kStatsThreads) {
+        const float4 q = Qv[i];
+        float4 sf[FPB + 1];
+        partial_sums<FPB>(P, nv, i, slot, cnt, sf);
+#pragma unroll
+        for (int k = 0; k < FPB; ++k) {
+            if (c.frame_mean && k < nf) {   // caller's buffer: 4-byte alignment only
+                float *fm = c.frame_mean + (size_t)(f0 + k) * c.D + 4 * i;
+                fm[0] = sf[k + 1].x / (float)c.N;
+                fm[1] = sf[k + 1].y / (float)c.N;
+                fm[2] = sf[k + 1].z / (float)c.N;
+                fm[3] = sf[k + 1].w / (float)c.N;
+            }
+            acc[3 * k] = dot4(sf[k + 1], q, acc[3 * k]);
+            acc[3 * k + 1] = dot4(sf[k + 1], sf[k + 1], acc[3 * k + 1]);
+            acc[3 * k + 2] = dot4(sf[k + 1], sf[k], acc[3 * k + 2]);
+        }
+        acc[3 * FPB] = dot4(q, q, acc[3 * FPB]);
+        acc[3 * FPB + 1] = dot4(sf[0], sf[0], acc[3 * FPB + 1]);
+    }
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int k = 0; k < NQ; ++k) acc[k] += __shfl_xor_sync(0xffffffffu, acc[k], o);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (lane == 0)
+#pragma unroll
+        for (int k = 0; k < NQ; ++k) wsum[warp][k] = acc[k];
+    __syncthreads();
+    if (warp < nf) {
+        // warp k's frame: lane 4 m + h (m < 5) sums quantity m over the warps h, h + 4
+        const int m = lane >> 2;
+        const int col = m < 3 ? 3 * warp + m : m == 3 ? 3 * FPB : warp == 0 ? 3 * FPB + 1 : 3 * (warp - 1) + 1;
+        double s = 0.0;
+        if (lane < 20)
+            for (int w = lane & 3; w < NW; w += 4) s += (double)wsum[w][col];
+        s += __shfl_xor_sync(0xffffffffu, s, 1);
+        s += __shfl_xor_sync(0xffffffffu, s, 2);
+        const double vq = __shfl_sync(0xffffffffu, s, 0), vv = __shfl_sync(0xffffffffu, s, 4);
+        const double vp = __shfl_sync(0xffffffffu, s, 8), qq = __shfl_sync(0xffffffffu, s, 12);
+        const double pp = __shfl_sync(0xffffffffu, s, 16);
+        const double den2 = vv * (lane == 0 ? qq : pp), num = lane == 0 ? vq : vp;
+        frame_result(c, f0 + warp, v, t0 + warp, lane, den2 > 0.0 ? num * rsqrt(den2) : 0.0);
+    }
+}
+
 // The max-over-query scorer's frame statistics: a CTA takes FPB consecutive
 // frames of one video (ceil(T / FPB) CTAs per video), whose sums stay in shared
 // memory ([FPB][D] floats); r_t = max_j <v_t, q_j> / ||q_j|| / ||v_t|| over the
@@ -674,7 +808,6 @@ __global__ void __launch_bounds__(512, 2) frame_stats_kernel(Ctx c) {
 // 13 x 13 x 3584 and 8 to 119 rows (events around the kernel): 77 us with one
 // frame per CTA, a warp per row and the gate after the dots, 36 us now.
 constexpr int kRowBatch = 8;
-constexpr int kStatsThreads = 256;   // of a maxsim statistics CTA; two per SM
 
 template <int FPB>
 __global__ void __launch_bounds__(kStatsThreads, 2) frame_stats_maxsim_kernel(Ctx c) {
@@ -688,7 +821,7 @@ __global__ void __launch_bounds__(kStatsThreads, 2) frame_stats_maxsim_kernel(Ct
     extern __shared__ float4 sfs[];   // [FPB][D/4] frame sums
     const int per_video = (c.T + FPB - 1) / FPB, nstat = c.V * per_video;
     if ((int)blockIdx.x >= nstat) {
-        frame_gate(c, (int64_t)blockIdx.x - nstat, gate_map);
+        frame_gate<false>(c, (int64_t)blockIdx.x - nstat, gate_map);
         return;
     }
     const int v = (int)blockIdx.x / per_video, t0 = ((int)blockIdx.x - v * per_video) * FPB;
@@ -970,10 +1103,10 @@ cudaError_t launch_frame_stats(const Ctx &c, cudaStream_t s) {
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
+    const int64_t frames = (int64_t)c.V * c.T, gates = c.gate && c.spatial_mode == WZ_SPATIAL_WSM ? frames : 0;
     if (c.relevance_mode == WZ_RELEVANCE_MAXSIM) {
         // frames share a CTA's reads of the query rows once every SM has work
         // without that (and their sums fit)
-        const int64_t frames = (int64_t)c.V * c.T;
         const int fpb = frames > 4 * (int64_t)sms && c.D <= 8192 ? 4 : frames > sms && c.D <= 16384 ? 2 : 1;
         const size_t smem = (size_t)fpb * c.D * 4;
         const void *fn = fpb == 4 ? (const void *)frame_stats_maxsim_kernel<4>
@@ -981,13 +1114,21 @@ cudaError_t launch_frame_stats(const Ctx &c, cudaStream_t s) {
                                     : (const void *)frame_stats_maxsim_kernel<1>;
         e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
-        const int gates = c.gate && c.spatial_mode == WZ_SPATIAL_WSM ? c.V * c.T : 0;
-        return launch_kernel(fn, dim3(c.V * ((c.T + fpb - 1) / fpb) + gates), dim3(kStatsThreads), smem, s, args,
-                             c.pdl != 0);
+        return launch_kernel(fn, dim3((unsigned)(c.V * ((c.T + fpb - 1) / fpb) + gates)), dim3(kStatsThreads), smem,
+                             s, args, c.pdl != 0);
+    }
+    if (frames > 4 * (int64_t)sms && c.T >= kStatsFrames) {
+        // more than two waves of a CTA per frame and gate
+        int gate_warps = c.N <= kWarpGateTokens;
+        const int64_t per = gate_warps ? kStatsThreads / 32 : 1;
+        const int64_t ctas = c.V * (int64_t)((c.T + kStatsFrames - 1) / kStatsFrames) + (gates + per - 1) / per;
+        void *margs[] = {const_cast<Ctx *>(&c), &gate_warps};
+        return launch_kernel((const void *)frame_stats_many_kernel<kStatsFrames>, dim3((unsigned)ctas),
+                             dim3(kStatsThreads), 0, s, margs, c.pdl != 0);
     }
     // a CTA per frame and one per gate; 256 threads (more CTAs in flight) once
     // 512 no longer fit in one wave
-    const int64_t ctas = (int64_t)c.V * c.T * (c.gate && c.spatial_mode == WZ_SPATIAL_WSM ? 2 : 1);
+    const int64_t ctas = frames + gates;
     const int threads = ctas > 2 * (int64_t)sms ? 256 : 512;
     return launch_kernel((const void *)frame_stats_kernel, dim3((unsigned)ctas), dim3(threads), 0, s, args, c.pdl != 0);
 }
