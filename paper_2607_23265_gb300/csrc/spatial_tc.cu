@@ -46,6 +46,7 @@ struct TcSmem {
     int Q;       // [16][2][BMAX]: Q_L, Q_H of row t's grid column at b = b0(t) + k
     int stage;   // [2][KC][512] bf16: the group's hi chunks, then its lo chunks
     int rec;     // [2][kMaxTaps]: the synthesis taps (lanes index them differently)
+    int zero;    // [BMAX] zeros: the gate row of a coefficient outside the support
     int total;
     __host__ __device__ void init(const SpatialSmem &L, int VT, int bmax) {
         int o = L.tables;
@@ -61,6 +62,7 @@ struct TcSmem {
         P = take(kTcRows * 2 * bmax, 4);
         Q = take(kTcRows * 2 * bmax, 4);
         rec = take(2 * kMaxTaps, 4);
+        zero = take(bmax, 4);
         stage = take((L.K_pad >> 5) * kTcChunkBytes * 2 / 4, 32);   // 128-byte aligned
         total = o;
     }
@@ -108,8 +110,8 @@ __global__ void __launch_bounds__(kSpatialThreads, BMAX <= 6 ? 3 : 2)
     spatial_wsm_tc_kernel(const __grid_constant__ CUtensorMap wmap, Ctx c) {
     pdl_trigger();
     extern __shared__ __align__(128) float sm[];
-    __shared__ int s_item, s_f, s_wsum[kSpatialThreads / 32];
-    const int tid = threadIdx.x;
+    __shared__ int s_item, s_wsum[kSpatialThreads / 32];
+    const int tid = threadIdx.x, lane = tid & 31;
     if (tid == 0) ptx::prefetch_tmap(&wmap);
     const int H = c.H, W = c.W, hp = c.hp, wp = c.wp, F = c.F, VT = c.V * c.T;
     SpatialSmem L;
@@ -124,6 +126,8 @@ __global__ void __launch_bounds__(kSpatialThreads, BMAX <= 6 ? 3 : 2)
         rec_lo[k] = c.rec_lo[k];
         rec_hi[k] = c.rec_hi[k];
     }
+    float *zrow = sm + S.zero;
+    if (tid < BMAX) zrow[tid] = 0.f;
     build_spatial_tables_smem(c, L, sm);
     pdl_wait();
     // thread 0 claims the next group while the current one is formed; the
@@ -162,29 +166,26 @@ __global__ void __launch_bounds__(kSpatialThreads, BMAX <= 6 ? 3 : 2)
     }
 
     for (;;) {
-        __syncthreads();   // the previous group's reads of shared memory
+        // the claim of the group after this one is in flight meanwhile (thread 0)
+        int next = 0;
         if (tid == 0) {
-            const int it = claimed;
-            if (it < items) claimed = (int)gridDim.x + atomicAdd(c.spatial_next, 1);
-            int fi = 0;
-            if (it < items) {
-                // the last frame whose first group is <= it (frames without
-                // groups share their successor's prefix)
-                int lo = 0, hi = VT - 1;
-                while (lo < hi) {
-                    const int mid = (lo + hi + 1) >> 1;
-                    if (gpre[mid] <= it) lo = mid;
-                    else hi = mid - 1;
-                }
-                fi = lo;
-            }
-            s_item = it;
-            s_f = fi;
+            s_item = claimed;
+            if (claimed < items) next = (int)gridDim.x + atomicAdd(c.spatial_next, 1);
         }
-        __syncthreads();
+        __syncthreads();   // the item; the previous group's reads of shared memory
         const int item = s_item;
         if (item >= items) break;
-        const int f = s_f, g = item - gpre[f];
+        // the last frame whose first group is <= item (frames without groups
+        // share their successor's prefix): every warp probes 32 places at a time
+        int f = 0;
+        for (int span = VT; span > 1;) {
+            const int step = (span + 31) >> 5, at = f + lane * step;
+            const unsigned le = __ballot_sync(0xffffffffu, lane * step < span && gpre[at] <= item);
+            const int k = 31 - __clz((int)le);   // gpre[f] <= item: le is not 0
+            f += k * step;
+            span = min(step, span - k * step);
+        }
+        const int g = item - gpre[f];
         const int nhw = fdat[3 * f], n = nhw & 8191, h = (nhw >> 13) & 127, w = nhw >> 20;
         // gate G of the frame (Eq. 6, Eq. 12), pooled by frame_stats: loaded
         // into registers here, stored to shared memory after the row setup
@@ -261,47 +262,58 @@ __global__ void __launch_bounds__(kSpatialThreads, BMAX <= 6 ? 3 : 2)
         __syncthreads();   // the stage is clear; G, P, Q and the row data are in place
         {
             const float *P = Pt + t * 2 * BMAX, *Q = Qt + t * 2 * BMAX;
+            const float *Gr[BMAX];   // the gate's rows from b0; zeros past the support
+#pragma unroll
+            for (int u = 0; u < BMAX; ++u) Gr[u] = u < na ? G + (a0 + u) * wp + b0 : zrow;
             for (int ri = s; ri < span; ri += 16) {
                 const int i = zlo + ri;
                 // P_u[p, a] A_u[a, i] for the row's coefficients a
-                float pal[BMAX], pah[BMAX];
+                float pll = 0.f, ph[BMAX], ps[BMAX];   // sum of the L parts; H part; L + H
 #pragma unroll
                 for (int u = 0; u < BMAX; ++u) {
-                    pal[u] = u < na ? P[u] * AHl[(a0 + u) * H + i] : 0.f;
-                    pah[u] = u < na ? P[BMAX + u] * AHh[(a0 + u) * H + i] : 0.f;
+                    const int at = min(a0 + u, hp - 1) * H + i;   // (P is 0 past the support)
+                    const float pl = P[u] * AHl[at];
+                    ph[u] = P[BMAX + u] * AHh[at];
+                    pll += pl;
+                    ps[u] = pl + ph[u];
                 }
-                // c_v[b] = Q_v[q, b] Y_v[b, i]
-                float cl[BMAX], ch[BMAX];
+                // c_v[b] = Q_v[q, b] Y_v[b, i], two b at a time, held twice as
+                // packed operands; what is read past the support in b is
+                // dropped by the select
+                f2_t cl[BMAX], ch[BMAX];
 #pragma unroll
-                for (int bb = 0; bb < BMAX; ++bb) {
-                    float yl = 0.f, yh = 0.f;
-                    if (bb < nb) {
+                for (int bb = 0; bb < BMAX; bb += 2) {
+                    const int b1 = bb + 1 < BMAX ? bb + 1 : bb;
+                    f2_t yl = pack2(pll, pll), yh = 0ull;
 #pragma unroll
-                        for (int u = 0; u < BMAX; ++u) {
-                            if (u < na) {
-                                const float gg = G[(a0 + u) * wp + b0 + bb];
-                                yl += pal[u] + pah[u] * gg;
-                                yh += (pal[u] + pah[u]) * gg;
-                            }
-                        }
+                    for (int u = 0; u < BMAX; ++u) {
+                        const f2_t gg = pack2(Gr[u][bb], Gr[u][b1]);
+                        yl = fma2(pack2(ph[u], ph[u]), gg, yl);
+                        yh = fma2(pack2(ps[u], ps[u]), gg, yh);
                     }
-                    cl[bb] = bb < nb ? Q[bb] * yl : 0.f;
-                    ch[bb] = bb < nb ? Q[BMAX + bb] * yh : 0.f;
+                    const float2 l = unpack2(yl), h2 = unpack2(yh);
+                    const float l0 = bb < nb ? Q[bb] * l.x : 0.f, h0 = bb < nb ? Q[BMAX + bb] * h2.x : 0.f;
+                    cl[bb] = pack2(l0, l0);
+                    ch[bb] = pack2(h0, h0);
+                    if (b1 > bb) {
+                        const float l1 = b1 < nb ? Q[b1] * l.y : 0.f, h1 = b1 < nb ? Q[BMAX + b1] * h2.y : 0.f;
+                        cl[b1] = pack2(l1, l1);
+                        ch[b1] = pack2(h1, h1);
+                    }
                 }
                 // row i of the operator row: columns 4 j4 .. 4 j4 + 3
                 for (int j4 = j4lo; j4 <= j4hi; ++j4) {
-                    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+                    f2_t a01 = 0ull, a23 = 0ull;
 #pragma unroll
                     for (int bb = 0; bb < BMAX; ++bb) {
-                        if (bb < nb) {
-                            const float4 a4 = reinterpret_cast<const float4 *>(AWl + (b0 + bb) * WP4)[j4];
-                            const float4 d4 = reinterpret_cast<const float4 *>(AWh + (b0 + bb) * WP4)[j4];
-                            acc.x = fmaf(cl[bb], a4.x, fmaf(ch[bb], d4.x, acc.x));
-                            acc.y = fmaf(cl[bb], a4.y, fmaf(ch[bb], d4.y, acc.y));
-                            acc.z = fmaf(cl[bb], a4.z, fmaf(ch[bb], d4.z, acc.z));
-                            acc.w = fmaf(cl[bb], a4.w, fmaf(ch[bb], d4.w, acc.w));
-                        }
+                        const int at = min(b0 + bb, wp - 1) * WP4 + 4 * j4;   // (c is 0 past the support)
+                        const ulonglong2 l = *reinterpret_cast<const ulonglong2 *>(AWl + at);
+                        const ulonglong2 h2 = *reinterpret_cast<const ulonglong2 *>(AWh + at);
+                        a01 = fma2(cl[bb], l.x, fma2(ch[bb], h2.x, a01));
+                        a23 = fma2(cl[bb], l.y, fma2(ch[bb], h2.y, a23));
                     }
+                    const float2 v01 = unpack2(a01), v23 = unpack2(a23);
+                    const float4 acc = make_float4(v01.x, v01.y, v23.x, v23.y);
                     stage_put4(shi, lo_off, t, i * W + 4 * j4, acc, min(4, W - 4 * j4));
                 }
             }
@@ -315,6 +327,7 @@ __global__ void __launch_bounds__(kSpatialThreads, BMAX <= 6 ? 3 : 2)
             if (wz_in_range(c.status, r0 + kTcRows <= c.w_rows)) ptx::tma_store_4d(&wmap, stg, 0, (int)(r0 >> 3), 0, 0);
             ptx::bulk_commit();
         }
+        claimed = next;
     }
     // rows past the produced count (tau > 0)
     const int tail = (int)(gridDim.x - 1 - blockIdx.x);
@@ -342,7 +355,10 @@ cudaError_t launch_spatial_tc(const Ctx &c, cudaStream_t s, bool *launched) {
     const int bmax = (c.F - 1) / 2 + 2;
     const void *fn;
     int bm;
-    if (bmax <= 6) {
+    if (bmax <= 5) {   // up to 8 taps
+        fn = (const void *)spatial_wsm_tc_kernel<5>;
+        bm = 5;
+    } else if (bmax == 6) {
         fn = (const void *)spatial_wsm_tc_kernel<6>;
         bm = 6;
     } else if (bmax <= 12) {
