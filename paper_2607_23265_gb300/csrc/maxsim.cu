@@ -40,16 +40,20 @@
 //   warp 10      TMA producer of the query rows (one thread)
 // Every mbarrier wait is bounded; on a timeout the kernel records a status
 // bit, drains what it issued, frees tensor memory and exits.
-// HBM bound up to Lq = 64 (256 frames of 27 x 27 x 3584: 0.243 ms at Lq = 16,
-// 0.26 at 64), then by the query rows' L2 reads (0.306 at 128).  On 8 videos of
-// 64 frames of 13 x 13 x 3584 and 8 to 119 rows one pass takes 0.185 ms where
+// HBM bound up to Lq = 64 (256 frames of 27 x 27 x 3584: 0.231 ms at Lq = 16,
+// 0.238 at 64), then by the query rows' L2 reads (0.298 at 128).  On 8 videos of
+// 64 frames of 13 x 13 x 3584 and 8 to 119 rows one pass takes 0.175 ms where
 // the relevance pass and one GEMM launch per video took 0.38; frame ends fall
-// inside most tiles there.  Measured and not taken: 16 channel-sum warps (0.196),
-// the sums in packed pairs (0.315), more query-row bytes in flight (0.19).
+// inside most tiles there.  The channel sums work on the rows of the tile's box
+// (a CTA's last tile is a short one), one K step per loop iteration: with all
+// 128 rows and four K steps unrolled 0.243, 0.265, 0.309 and 0.185 ms.  Measured
+// and not taken: 16 channel-sum warps (0.196), more query-row bytes in flight
+// (0.19).
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
 #include <algorithm>
+#include <type_traits>
 #include <cstring>
 
 #include "wz_internal.cuh"
@@ -364,7 +368,6 @@ __global__ void __launch_bounds__(kXThreads, 1) maxsim_pass_kernel(const __grid_
             // a frame starts inside the tile at row rb (frames have >= 128 tokens)
             const int to_end = (int)((int64_t)c.N - base % c.N);
             const int rb = to_end < nr ? to_end : nr;
-            const bool whole = rb == kXM;   // every row of the tile in the open frame
             float sq[16];                   // squares of this lane's two channels, row 8 i + re
 #pragma unroll
             for (int i = 0; i < 16; ++i) sq[i] = 0.f;
@@ -379,43 +382,59 @@ __global__ void __launch_bounds__(kXThreads, 1) maxsim_pass_kernel(const __grid_
                 }
                 // (indexed from the shared array itself: shared-memory loads)
                 const uint8_t *st0 = smem_raw + ring_off + (size_t)stage * p.stage_stride;
-#pragma unroll
+#pragma unroll 1
                 for (int g = 0; g < G; ++g) {
                     const uint8_t *lb = st0 + g * a_sub + lane_off;
-                    // s0 the open frame's rows, s1 the next's (whole tiles: even
-                    // and odd rows, shorter dependent chains)
+                    // s0 the open frame's rows, s1 the next's: NI rows per lane
+                    // (the tile's box), those past the tile as zeros; without a
+                    // frame end in the tile packed sums of even and odd rows,
+                    // else predicated ones (in PTX: as branches they take 1.4
+                    // times the kernel's time)
                     float s0x = 0.f, s0y = 0.f, s1x = 0.f, s1y = 0.f;
-                    if (whole) {
+                    auto rows = [&](auto ni, auto split) {
+                        constexpr int NI = decltype(ni)::value;
+                        uint32_t w[NI];
 #pragma unroll
-                        for (int i = 0; i < 16; ++i) {
-                            const uint32_t wv = *reinterpret_cast<const uint32_t *>(lb + 1024 * i);
-                            const float x = bf16_lo(wv), y = bf16_hi(wv);
-                            sq[i] = fmaf(x, x, fmaf(y, y, sq[i]));
-                            if (i & 1) {
-                                s1x += x;
-                                s1y += y;
-                            } else {
-                                s0x += x;
-                                s0y += y;
-                            }
+                        for (int i = 0; i < NI; ++i) {
+                            w[i] = *reinterpret_cast<const uint32_t *>(lb + 1024 * i);
+                            if (i >= NI - 4) w[i] = 8 * i < nrl ? w[i] : 0u;
                         }
-                        s0x += s1x;
-                        s0y += s1y;
-                        s1x = s1y = 0.f;
+                        f2_t e = 0ull, o = 0ull;
+#pragma unroll
+                        for (int i = 0; i < NI; ++i) {
+                            const float x = bf16_lo(w[i]), y = bf16_hi(w[i]);
+                            sq[i] = fmaf(x, x, fmaf(y, y, sq[i]));
+                            if constexpr (decltype(split)::value)
+                                asm("{\n"
+                                    ".reg .pred p;\n"
+                                    "setp.lt.s32 p, %6, %7;\n"
+                                    "@p add.f32 %0, %0, %4;\n"
+                                    "@p add.f32 %1, %1, %5;\n"
+                                    "@!p add.f32 %2, %2, %4;\n"
+                                    "@!p add.f32 %3, %3, %5;\n"
+                                    "}"
+                                    : "+f"(s0x), "+f"(s0y), "+f"(s1x), "+f"(s1y)
+                                    : "f"(x), "f"(y), "r"(8 * i), "r"(rbl));
+                            else if (i & 1) o = add2(o, pack2(x, y));
+                            else e = add2(e, pack2(x, y));
+                        }
+                        if constexpr (!decltype(split)::value) {
+                            const float2 s = unpack2(add2(e, o));
+                            s0x = s.x;
+                            s0y = s.y;
+                        }
+                    };
+                    using std::integral_constant;
+                    if (rb == nr) {
+                        if (nr > 96) rows(integral_constant<int, 16>(), std::false_type());
+                        else if (nr > 64) rows(integral_constant<int, 12>(), std::false_type());
+                        else if (nr > 32) rows(integral_constant<int, 8>(), std::false_type());
+                        else rows(integral_constant<int, 4>(), std::false_type());
                     } else {
-#pragma unroll
-                        for (int i = 0; i < 16; ++i) {
-                            const uint32_t wv = *reinterpret_cast<const uint32_t *>(lb + 1024 * i);
-                            const float x = bf16_lo(wv), y = bf16_hi(wv);
-                            sq[i] = fmaf(x, x, fmaf(y, y, sq[i]));
-                            if (8 * i < rbl) {
-                                s0x += x;
-                                s0y += y;
-                            } else if (8 * i < nrl) {
-                                s1x += x;
-                                s1y += y;
-                            }
-                        }
+                        if (nr > 96) rows(integral_constant<int, 16>(), std::true_type());
+                        else if (nr > 64) rows(integral_constant<int, 12>(), std::true_type());
+                        else if (nr > 32) rows(integral_constant<int, 8>(), std::true_type());
+                        else rows(integral_constant<int, 4>(), std::true_type());
                     }
                     if (g == G - 1) {   // the stage's last K step is in registers: hand the stage back
                         __syncwarp();
