@@ -796,156 +796,168 @@ __global__ void __launch_bounds__(kStatsThreads, 3) frame_stats_many_kernel(Ctx 
     }
 }
 
-// The max-over-query scorer's frame statistics: a CTA takes FPB consecutive
-// frames of one video (ceil(T / FPB) CTAs per video), whose sums stay in shared
-// memory ([FPB][D] floats); r_t = max_j <v_t, q_j> / ||q_j|| / ||v_t|| over the
-// video's query rows: every thread takes 16-byte vectors of the channels,
-// kRowBatch rows at a time (a row is read once for the FPB frames), the rows'
-// partial dots are reduced across the warp by one transpose-reduction, and the
-// warps' partials are added in a tree.  The gates are formed by further CTAs
-// (one per frame) beside them.  Bound by the latency of its steps and by
-// reading the query rows from L2 in every CTA (Lq D bf16 each): 512 frames of
-// 13 x 13 x 3584 and 8 to 119 rows (events around the kernel): 77 us with one
-// frame per CTA, a warp per row and the gate after the dots, 36 us now.
-constexpr int kRowBatch = 8;
+// The max-over-query scorer's frame statistics: a cluster of S CTAs takes
+// eight consecutive frames of one video (ceil(T / 8) clusters per video), each
+// CTA 1 / S of the channels: it forms the frames' sums there (shared
+// memory, [9][channels] with the frame before), their squares and neighbour
+// products (a warp per frame), and their dots with the video's query rows (a
+// warp per kMxRows rows: lanes over the channels, one transpose-reduction over
+// the 32 dots).  CTA k of the cluster then adds the parts of the dots of
+// frames k, k + S, .. and takes r_t = max_j <v_t, q_j> / ||q_j|| / ||v_t||.  The gates are
+// formed by further clusters beside them, a warp each where there are many
+// small frames.  The query rows are read once per eight frames, 1 / S by
+// each CTA: with CTAs of one to four whole frames their L2 reads bounded the
+// kernel (events around it: 512 frames of 13 x 13 x 3584 and 8 to 119 rows 35
+// us, 30 now; 128 rows 41 and 34; 128 frames of 16 x 16, 64 rows 18.0 and 16.4),
+// now the latency of its steps.  Eight CTAs per cluster there: 33 us (1.7 waves).
+constexpr int kMxFrames = 8;         // of a cluster
+constexpr int kMxRows = 4;
 
-template <int FPB>
-__global__ void __launch_bounds__(kStatsThreads, 2) frame_stats_maxsim_kernel(Ctx c) {
-    constexpr int NW = kStatsThreads / 32;
+template <int S>
+__global__ void __launch_bounds__(kStatsThreads, 2) frame_stats_maxsim_kernel(Ctx c, int gate_warps) {
+    __shared__ float part[kMxFrames][WZ_MAX_LQ_MAXSIM];   // <v_f, q_j> over this CTA's channels
+    __shared__ float wsum[kMxFrames][3];                  // vv, v.v_prev, v_prev.v_prev over them
+    __shared__ double best[kMxFrames / S][4], tot[kMxFrames / S][3];
+    __shared__ int slots[kMxFrames + 1], counts[kMxFrames + 1];
+    __shared__ float gate_map[WZ_MAX_HW * WZ_MAX_HW];
+    extern __shared__ float4 sfs[];   // [9][2 * per] frame sums: frame f0 - 1 + k of this CTA's channels
+    static_assert(kStatsThreads == 32 * kMxFrames && WZ_MAX_LQ_MAXSIM == 128, "a warp per frame, four for the rows");
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int per_video = (c.T + kMxFrames - 1) / kMxFrames, nstat = c.V * per_video * S;
+    const int group = (int)blockIdx.x / S, v = group / per_video, t0 = (group - v * per_video) * kMxFrames;
+    const int nf = min(kMxFrames, c.T - t0);
+    const int64_t f0 = (int64_t)v * c.T + t0;
+    // the column partials of frame f0 - 1 + k
+    if ((int)blockIdx.x < nstat && tid <= kMxFrames) {
+        int64_t at = 0;
+        int n = 0;
+        if ((tid > 0 || t0 > 0) && tid <= nf) frame_slots(c, f0 - 1 + tid, at, n);
+        slots[tid] = (int)at;   // < G1 + V T
+        counts[tid] = n;
+    }
+    __syncthreads();
     pdl_wait();
     pdl_trigger();
-    __shared__ float wsum[FPB][NW][3];                       // vv, v.v_prev, v_prev.v_prev
-    __shared__ float part[FPB][NW][WZ_MAX_LQ_MAXSIM];        // per warp: <v_f, q_j>
-    __shared__ double best[FPB][4];
-    __shared__ float gate_map[WZ_MAX_HW * WZ_MAX_HW];
-    extern __shared__ float4 sfs[];   // [FPB][D/4] frame sums
-    const int per_video = (c.T + FPB - 1) / FPB, nstat = c.V * per_video;
-    if ((int)blockIdx.x >= nstat) {
-        frame_gate<false>(c, (int64_t)blockIdx.x - nstat, gate_map);
+    if ((int)blockIdx.x >= nstat) {   // whole clusters
+        const int b = (int)blockIdx.x - nstat;
+        if (gate_warps || b < c.V * c.T) frame_gates(c, b, gate_warps, gate_map);
         return;
     }
-    const int v = (int)blockIdx.x / per_video, t0 = ((int)blockIdx.x - v * per_video) * FPB;
-    const int nf = min(FPB, c.T - t0);
-    const int64_t f0 = (int64_t)v * c.T + t0;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const VideoPar par = c.vpar[v];
-    const int nv = c.D / 4;
-    const float4 *P = reinterpret_cast<const float4 *>(c.part);
-    // the column partials of frame f0 - 1 + k
-    int64_t slot[FPB + 1];
-    int cnt[FPB + 1];
-#pragma unroll
-    for (int k = 0; k <= FPB; ++k) {
-        slot[k] = cnt[k] = 0;
-        if ((k > 0 || t0 > 0) && k <= nf) frame_slots(c, f0 - 1 + k, slot[k], cnt[k]);
-    }
-    auto dot4 = [](const float4 &a, const float4 &b, float s) {
-        return fmaf(a.x, b.x, fmaf(a.y, b.y, fmaf(a.z, b.z, fmaf(a.w, b.w, s))));
-    };
-    float vv[FPB], vp[FPB], pp[FPB];
-#pragma unroll
-    for (int k = 0; k < FPB; ++k) vv[k] = vp[k] = pp[k] = 0.f;
-    for (int i = threadIdx.x; i < nv; i += kStatsThreads) {
-        float4 sf[FPB + 1];
-#pragma unroll
-        for (int k = 0; k <= FPB; ++k) {
-            sf[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-            for (int q = 0; q < cnt[k]; q += 2) {   // two partial rows in flight, summed in order
-                const float4 x = P[(size_t)(slot[k] + q) * nv + i];
-                const float4 y = q + 1 < cnt[k] ? P[(size_t)(slot[k] + q + 1) * nv + i] : make_float4(0.f, 0.f, 0.f, 0.f);
-                sf[k].x += x.x; sf[k].y += x.y; sf[k].z += x.z; sf[k].w += x.w;
-                if (q + 1 < cnt[k]) { sf[k].x += y.x; sf[k].y += y.y; sf[k].z += y.z; sf[k].w += y.w; }
+    const int rank = (int)ptx::cluster_rank();
+    const int Lq = c.vpar[v].Lq, q_row0 = c.vpar[v].q_row0;
+    // this CTA's channels: 16-byte vectors v0 .. v0 + nvec - 1 of a row
+    const int n8 = c.D / 8, per = (n8 + S - 1) / S, v0 = min(rank * per, n8), nvec = min(per, n8 - v0);
+    const int nq = 2 * nvec;
+    {
+        const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+        const float4 *P = reinterpret_cast<const float4 *>(c.part) + 2 * v0;
+        const size_t nv = (size_t)c.D / 4;
+#pragma unroll 4
+        for (int idx = tid; idx < (kMxFrames + 1) * nq; idx += kStatsThreads) {
+            const int k = idx / nq, i = idx - k * nq, n = counts[k];
+            const float4 *src = P + (size_t)slots[k] * nv + i;
+            float4 s = n > 0 ? src[0] : zero;
+            const float4 y = n > 1 ? src[nv] : zero;
+            s.x += y.x; s.y += y.y; s.z += y.z; s.w += y.w;
+            for (int q = 2; q < n; ++q) {
+                const float4 z = src[(size_t)q * nv];
+                s.x += z.x; s.y += z.y; s.z += z.z; s.w += z.w;
             }
-        }
-#pragma unroll
-        for (int k = 0; k < FPB; ++k) {
-            sfs[k * nv + i] = sf[k + 1];
-            vv[k] = dot4(sf[k + 1], sf[k + 1], vv[k]);
-            vp[k] = dot4(sf[k + 1], sf[k], vp[k]);
-            pp[k] = dot4(sf[k], sf[k], pp[k]);
+            sfs[k * 2 * per + i] = s;
         }
     }
-#pragma unroll
-    for (int k = 0; k < FPB; ++k) {
+    __syncthreads();
+    {
+        auto dot4 = [](const float4 &a, const float4 &b, float s) {
+            return fmaf(a.x, b.x, fmaf(a.y, b.y, fmaf(a.z, b.z, fmaf(a.w, b.w, s))));
+        };
+        float vv = 0.f, vp = 0.f, pp = 0.f;
+        for (int i = lane; i < nq; i += 32) {
+            const float4 s = sfs[(warp + 1) * 2 * per + i], p = sfs[warp * 2 * per + i];
+            vv = dot4(s, s, vv);
+            vp = dot4(s, p, vp);
+            pp = dot4(p, p, pp);
+        }
         for (int o = 16; o > 0; o >>= 1) {
-            vv[k] += __shfl_xor_sync(0xffffffffu, vv[k], o);
-            vp[k] += __shfl_xor_sync(0xffffffffu, vp[k], o);
-            pp[k] += __shfl_xor_sync(0xffffffffu, pp[k], o);
+            vv += __shfl_xor_sync(0xffffffffu, vv, o);
+            vp += __shfl_xor_sync(0xffffffffu, vp, o);
+            pp += __shfl_xor_sync(0xffffffffu, pp, o);
         }
         if (lane == 0) {
-            wsum[k][warp][0] = vv[k];
-            wsum[k][warp][1] = vp[k];
-            wsum[k][warp][2] = pp[k];
+            wsum[warp][0] = vv;
+            wsum[warp][1] = vp;
+            wsum[warp][2] = pp;
         }
     }
-    __syncthreads();   // sfs complete
-    const int n8 = c.D / 8;
-    const uint4 *Qr = reinterpret_cast<const uint4 *>(static_cast<const __nv_bfloat16 *>(c.Q) + (size_t)par.q_row0 * c.D);
-    // CTAs start on different rows: no hot L2 lines
-    const int nbatch = (par.Lq + kRowBatch - 1) / kRowBatch, rot = (int)(blockIdx.x % nbatch);
-    for (int bi = 0; bi < nbatch; ++bi) {
-        const int j0 = (bi + rot < nbatch ? bi + rot : bi + rot - nbatch) * kRowBatch;
-        float acc[FPB][kRowBatch];
+    const uint4 *Qr = reinterpret_cast<const uint4 *>(static_cast<const __nv_bfloat16 *>(c.Q) + (size_t)q_row0 * c.D) + v0;
+    for (int j0 = warp * kMxRows; j0 < Lq; j0 += kStatsThreads / 32 * kMxRows) {
+        f2_t acc[kMxFrames][kMxRows];
 #pragma unroll
-        for (int k = 0; k < FPB; ++k)
+        for (int k = 0; k < kMxFrames; ++k)
 #pragma unroll
-            for (int u = 0; u < kRowBatch; ++u) acc[k][u] = 0.f;
-        for (int i = threadIdx.x; i < n8; i += kStatsThreads) {
-            uint4 qv[kRowBatch];
+            for (int u = 0; u < kMxRows; ++u) acc[k][u] = 0ull;
+#pragma unroll 1
+        for (int i = lane; i < nvec; i += 32) {
+            f2_t q[kMxRows][4];
 #pragma unroll
-            for (int u = 0; u < kRowBatch; ++u)
-                qv[u] = j0 + u < par.Lq ? __ldg(Qr + (size_t)(j0 + u) * n8 + i) : make_uint4(0u, 0u, 0u, 0u);
-            float4 s[FPB][2];
-#pragma unroll
-            for (int k = 0; k < FPB; ++k) {
-                s[k][0] = sfs[k * nv + 2 * i];
-                s[k][1] = sfs[k * nv + 2 * i + 1];
+            for (int u = 0; u < kMxRows; ++u) {
+                const uint4 x = j0 + u < Lq ? __ldg(Qr + (size_t)(j0 + u) * n8 + i) : make_uint4(0u, 0u, 0u, 0u);
+                unpack_pairs(x, q[u], (__nv_bfloat16 *)nullptr);
             }
 #pragma unroll
-            for (int u = 0; u < kRowBatch; ++u) {
-                float q[8];
-                unpack(qv[u], q, (__nv_bfloat16 *)nullptr);
+            for (int k = 0; k < kMxFrames; ++k) {
+                const ulonglong2 *sk = reinterpret_cast<const ulonglong2 *>(sfs + (k + 1) * 2 * per + 2 * i);
+                const ulonglong2 a = sk[0], b = sk[1];
 #pragma unroll
-                for (int k = 0; k < FPB; ++k)
-                    acc[k][u] = dot4(s[k][0], make_float4(q[0], q[1], q[2], q[3]),
-                                     dot4(s[k][1], make_float4(q[4], q[5], q[6], q[7]), acc[k][u]));
+                for (int u = 0; u < kMxRows; ++u)
+                    acc[k][u] = fma2(q[u][0], a.x, fma2(q[u][1], a.y, fma2(q[u][2], b.x, fma2(q[u][3], b.y, acc[k][u]))));
             }
         }
+        float d[kMxFrames * kMxRows];
 #pragma unroll
-        for (int k = 0; k < FPB; ++k) {
-            const float tot = transpose_reduce<kRowBatch>(acc[k]);   // lane l holds row l >> 2
-            if ((lane & 3) == 0) part[k][warp][j0 + (lane >> 2)] = tot;
-        }
+        for (int k = 0; k < kMxFrames; ++k)
+#pragma unroll
+            for (int u = 0; u < kMxRows; ++u) {
+                const float2 x = unpack2(acc[k][u]);
+                d[k * kMxRows + u] = x.x + x.y;
+            }
+        const float r = transpose_reduce<kMxFrames * kMxRows>(d);   // lane l holds value l
+        part[lane / kMxRows][j0 + lane % kMxRows] = r;
     }
-    __syncthreads();
-    // the dots with row j over the warps, over ||q_j||; 128 rows of a frame per
-    // four warps
-    static_assert(WZ_MAX_LQ_MAXSIM == 128 && NW == 8, "two frames per round");
-#pragma unroll
-    for (int k0 = 0; k0 < FPB; k0 += 2) {
-        const int k = k0 + (int)(threadIdx.x >> 7), j = threadIdx.x & 127;
-        if (k < FPB) {
+    __syncwarp();
+    ptx::cluster_sync();   // every CTA's parts
+    for (int m = 0, f = rank; f < nf; ++m, f += S) {
+        if (warp < 4) {
+            const int j = tid;
             double x = -INFINITY;
-            if (k < nf && j < par.Lq) {
+            if (j < Lq) {
                 const double qn = (double)c.qnorm[(size_t)v * WZ_MAX_LQ_MAXSIM + j];
-                const float d = ((part[k][0][j] + part[k][1][j]) + (part[k][2][j] + part[k][3][j])) +
-                                ((part[k][4][j] + part[k][5][j]) + (part[k][6][j] + part[k][7][j]));
-                x = qn > 0.0 ? (double)d / qn : 0.0;
+                float p[S];
+#pragma unroll
+                for (int r = 0; r < S; ++r) p[r] = ptx::ld_cluster(ptx::map_cluster(&part[f][j], (uint32_t)r));
+#pragma unroll
+                for (int o = 1; o < S; o <<= 1)
+#pragma unroll
+                    for (int r = 0; r < S; r += 2 * o) p[r] += p[r + o];
+                x = qn > 0.0 ? (double)p[0] / qn : 0.0;
             }
             for (int o = 16; o > 0; o >>= 1) x = fmax(x, __shfl_xor_sync(0xffffffffu, x, o));
-            if (lane == 0) best[k][warp & 3] = x;
+            if (lane == 0) best[m][warp] = x;
+        } else if (warp == 4) {   // lane S q + r: quantity q of CTA r
+            double s = 0.0;
+            if (lane < 3 * S)
+                s = (double)ptx::ld_cluster(ptx::map_cluster(&wsum[f][lane / S], (uint32_t)(lane % S)));
+            for (int o = 1; o < S; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            if (lane < 3 * S && lane % S == 0) tot[m][lane / S] = s;
         }
     }
-    __syncthreads();
-    if (warp < nf) {   // a warp per frame: lane q < 3 sums quantity q over the warps
-        double acc = 0.0;
-        if (lane < 3)
-            for (int w = 0; w < NW; ++w) acc += (double)wsum[warp][w][lane];
-        const double s0 = __shfl_sync(0xffffffffu, acc, 0), s1 = __shfl_sync(0xffffffffu, acc, 1);
-        const double s2 = __shfl_sync(0xffffffffu, acc, 2);
+    __syncwarp();
+    ptx::cluster_sync();   // the parts have been read (and best, tot are written)
+    const int f = rank + warp * S;   // a warp per frame
+    if (warp < kMxFrames / S && f < nf) {
         const double m = fmax(fmax(best[warp][0], best[warp][1]), fmax(best[warp][2], best[warp][3]));
-        const double den2 = lane == 0 ? s0 : s0 * s2, num = lane == 0 ? m : s1;
-        frame_result(c, f0 + warp, v, t0 + warp, lane, den2 > 0.0 ? num * rsqrt(den2) : 0.0);
+        const double den2 = lane == 0 ? tot[warp][0] : tot[warp][0] * tot[warp][2], num = lane == 0 ? m : tot[warp][1];
+        frame_result(c, f0 + f, v, t0 + f, lane, den2 > 0.0 ? num * rsqrt(den2) : 0.0);
     }
 }
 
@@ -1105,17 +1117,18 @@ cudaError_t launch_frame_stats(const Ctx &c, cudaStream_t s) {
     if (e != cudaSuccess) return e;
     const int64_t frames = (int64_t)c.V * c.T, gates = c.gate && c.spatial_mode == WZ_SPATIAL_WSM ? frames : 0;
     if (c.relevance_mode == WZ_RELEVANCE_MAXSIM) {
-        // frames share a CTA's reads of the query rows once every SM has work
-        // without that (and their sums fit)
-        const int fpb = frames > 4 * (int64_t)sms && c.D <= 8192 ? 4 : frames > sms && c.D <= 16384 ? 2 : 1;
-        const size_t smem = (size_t)fpb * c.D * 4;
-        const void *fn = fpb == 4 ? (const void *)frame_stats_maxsim_kernel<4>
-                         : fpb == 2 ? (const void *)frame_stats_maxsim_kernel<2>
-                                    : (const void *)frame_stats_maxsim_kernel<1>;
+        // eight CTAs per eight frames, four where that is one wave and eight are not
+        const int64_t octets = c.V * (int64_t)((c.T + kMxFrames - 1) / kMxFrames);
+        const int S = 8 * octets > 2 * (int64_t)sms && c.D <= 8192 ? 4 : 8;
+        const void *fn = S == 4 ? (const void *)frame_stats_maxsim_kernel<4> : (const void *)frame_stats_maxsim_kernel<8>;
+        const size_t smem = (size_t)(kMxFrames + 1) * 2 * ((c.D / 8 + S - 1) / S) * 16;
         e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
-        return launch_kernel(fn, dim3((unsigned)(c.V * ((c.T + fpb - 1) / fpb) + gates)), dim3(kStatsThreads), smem,
-                             s, args, c.pdl != 0);
+        int gate_warps = frames > sms && c.N <= kWarpGateTokens;
+        const int64_t per = gate_warps ? kStatsThreads / 32 : 1, gate_ctas = (gates + per - 1) / per;
+        void *margs[] = {const_cast<Ctx *>(&c), &gate_warps};
+        return launch_kernel(fn, dim3((unsigned)((octets + (gate_ctas + S - 1) / S) * S)), dim3(kStatsThreads), smem, s,
+                             margs, c.pdl != 0, (unsigned)S);
     }
     if (frames > 4 * (int64_t)sms && c.T >= kStatsFrames) {
         // more than two waves of a CTA per frame and gate

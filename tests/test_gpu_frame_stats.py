@@ -1,4 +1,4 @@
-"""Frame statistics of many frames: several frames per CTA (the last CTA of a video not full, rows
+"""Frame statistics of many frames: several frames per CTA or cluster (the last of a video not full, rows
 of more vectors than threads), gates by warps and by CTAs."""
 
 import pytest
@@ -14,8 +14,8 @@ CASES = [
     (1, 650, 8, 9, 72, 2, "mean"),
     (10, 64, 8, 8, 1032, 4, "mean"),      # two vectors per thread
     (9, 70, 23, 23, 64, 2, "mean"),       # 529 tokens: a CTA per gate
-    (1, 201, 8, 8, 2112, 9, "maxsim"),    # two frames per CTA, two steps per row batch
-    (33, 19, 12, 12, 64, 17, "maxsim"),   # four frames per CTA
+    (1, 201, 8, 8, 2112, 9, "maxsim"),    # clusters of eight, one frame in the last
+    (33, 19, 12, 12, 64, 17, "maxsim"),   # clusters of four
 ]
 
 
