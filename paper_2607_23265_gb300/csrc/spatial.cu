@@ -518,9 +518,9 @@ cudaError_t launch_spatial(const Ctx &c, cudaStream_t s) {
         void *args[] = {const_cast<Ctx *>(&c), &S};
         return launch_kernel(fn, dim3(blocks), dim3(kSpatialThreads), smem, s, args, c.pdl != 0);
     }
-    // persistent: every resident CTA pulls grid rows; at least kTailBlocks
-    // CTAs so that the tail rows are covered
-    const unsigned blocks = (unsigned)std::max(resident, kTailBlocks);
+    // persistent; a grid row holds at least one token of the budget
+    const int64_t rows = std::min<int64_t>((int64_t)c.V * c.T * c.H, c.rows_total);
+    const unsigned blocks = spatial_blocks(c, sms, per_sm > 0 ? per_sm : 1, rows);
     void *args[] = {const_cast<Ctx *>(&c), &compact};
     return launch_kernel(fn, dim3(blocks), dim3(kSpatialThreads), compact ? smem_c : smem, s, args, c.pdl != 0);
 }

@@ -392,9 +392,9 @@ cudaError_t launch_spatial_tc(const Ctx &c, cudaStream_t s, bool *launched) {
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kSpatialThreads, smem)) != cudaSuccess)
         return e;
     if (per_sm < 1) return cudaSuccess;
-    // persistent: every resident CTA pulls groups; at least kTailBlocks CTAs
-    // so that the tail rows are covered
-    const unsigned blocks = (unsigned)std::max(sms * per_sm, kTailBlocks);
+    // persistent; at most the groups (a frame's last one not full) and, beside
+    // them, the frames' unit records
+    const unsigned blocks = spatial_blocks(c, sms, per_sm, c.rows_total / kTcRows + 2 * (int64_t)c.V * c.T);
     void *args[] = {&wmap, const_cast<Ctx *>(&c)};
     *launched = true;
     return launch_kernel(fn, dim3(blocks), dim3(kSpatialThreads), smem, s, args, c.pdl != 0);

@@ -6,6 +6,8 @@
 // parameters at the head of its shared-memory block.
 #pragma once
 
+#include <algorithm>
+
 #include "wz_internal.cuh"
 
 namespace wz {
@@ -154,6 +156,18 @@ __device__ __forceinline__ void write_rows(const Ctx &c, const float *stg, int k
 
 constexpr int kSpatialThreads = 256;
 constexpr int kTailBlocks = 64;
+
+// CTAs of a persistent spatial kernel for at most `work` work items: all that
+// fit, or fewer when there are fewer items and the SMs that the temporal
+// kernel's V + 1 CTAs do not hold take those.  The CTAs form their tables
+// while that kernel runs; a full grid's last ones start only when it has ended
+// and delay small calls by the tables (64 frames of 13 x 13 x 3584 54.3 -> 53.9
+// us, 16 of 14 x 14 x 896 fp32 50.6 -> 49.0).  A full grid cut to the free SMs
+// lost more than it gave (256 frames of 27 x 27 411.7 -> 414.7).
+inline unsigned spatial_blocks(const Ctx &c, int sms, int per_sm, int64_t work) {
+    const int64_t free = (int64_t)(sms - (c.V + 1)) * per_sm;
+    return (unsigned)std::max<int64_t>(work <= free ? work : (int64_t)sms * per_sm, kTailBlocks);
+}
 constexpr int kCompactFrames = 2048;   // frames whose work prefix a spatial CTA keeps in shared memory
 
 // pre[f] = sum of count(f') over the frames f' < f, pre[F] = the total
