@@ -46,55 +46,70 @@ __device__ __forceinline__ void video_init(const Ctx &c, int v, const VideoPar &
     }
 }
 
-// u_q = mean of the query rows: a block covers 32 channels with 8 row
-// slices; compensated fp32 sums (TwoSum) per slice, combined in a fixed
-// order, stored as fp64 and fp32.
+__device__ __forceinline__ float2 load_two(const __nv_bfloat16 *p) {
+    const uint32_t v = *reinterpret_cast<const uint32_t *>(p);
+    return make_float2(bf16_lo(v), bf16_hi(v));
+}
+__device__ __forceinline__ float2 load_two(const float *p) { return *reinterpret_cast<const float2 *>(p); }
+
+// u_q = mean of the query rows: a block covers 64 channels, two per thread (a
+// warp reads 128 bytes or more of a row), with 8 row slices; compensated fp32
+// sums (TwoSum) per slice, combined in a fixed order, stored as fp64 and fp32.
+// Latency bound; half the CTAs of one channel per thread also leave the SMs to
+// the relevance pass sooner (whole calls: 128 frames of 16 x 16, 64 rows 103.4
+// -> 101.3 us, 32 videos of 64 frames 739.9 -> 738.0; 16 slices of 512 threads
+// 100.6 and 740.5).
 template <typename T, int NPAR>
 __global__ void __launch_bounds__(256) query_pool_kernel(Ctx c, VideoParBlock<NPAR> par) {
-    __shared__ float ps[8][32], pe[8][32];
+    __shared__ float2 ps[8][32], pe[8][32];
     pdl_wait();
     pdl_trigger();
     const int v = blockIdx.y;
     const VideoPar vp = par.v[v];
     if (blockIdx.x == 0 && threadIdx.x == 0) video_init(c, v, vp);
     const int cl = threadIdx.x & 31, slice = threadIdx.x >> 5;
-    const int d = blockIdx.x * 32 + cl;
-    float s = 0.f, e = 0.f;
+    const int d = (blockIdx.x * 32 + cl) * 2;   // (D is even)
+    float2 s = make_float2(0.f, 0.f), e = s;
+    auto add = [](float2 &s, float2 &e, const float2 &x) {
+        float t, err;
+        two_sum(s.x, x.x, t, err);
+        s.x = t;
+        e.x += err;
+        two_sum(s.y, x.y, t, err);
+        s.y = t;
+        e.y += err;
+    };
     if (d < c.D) {
         const T *Q = static_cast<const T *>(c.Q) + (size_t)vp.q_row0 * c.D + d;
         // rows slice, slice + 8, ...: loaded 8 at a time, then summed in order
         for (int j0 = slice; j0 < vp.Lq; j0 += 64) {
-            float x[8];
+            float2 x[8];
 #pragma unroll
             for (int k = 0; k < 8; ++k) {
                 const int j = j0 + 8 * k;
-                x[k] = j < vp.Lq ? load_scalar<T>(Q + (size_t)j * c.D) : 0.f;
+                x[k] = j < vp.Lq ? load_two(Q + (size_t)j * c.D) : make_float2(0.f, 0.f);
             }
 #pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                if (j0 + 8 * k < vp.Lq) {
-                    float t, err;
-                    two_sum(s, x[k], t, err);
-                    s = t;
-                    e += err;
-                }
-            }
+            for (int k = 0; k < 8; ++k)
+                if (j0 + 8 * k < vp.Lq) add(s, e, x[k]);
         }
     }
     ps[slice][cl] = s;
     pe[slice][cl] = e;
     __syncthreads();
-    if (slice == 0 && d < c.D) {
+    if (slice < 2 && d < c.D) {   // warp h: the threads' channel h
+        const bool h = slice != 0;
         float S = 0.f, E = 0.f;
         for (int k = 0; k < 8; ++k) {
+            const float2 s2 = ps[k][cl], e2 = pe[k][cl];
             float t, err;
-            two_sum(S, ps[k][cl], t, err);
+            two_sum(S, h ? s2.y : s2.x, t, err);
             S = t;
-            E += err + pe[k][cl];
+            E += err + (h ? e2.y : e2.x);
         }
         const double m = ((double)S + (double)E) / (double)vp.Lq;
-        c.qbar64[(size_t)v * c.D + d] = m;
-        c.qbar32[(size_t)v * c.D + d] = (float)m;
+        c.qbar64[(size_t)v * c.D + d + slice] = m;
+        c.qbar32[(size_t)v * c.D + d + slice] = (float)m;
     }
 }
 
@@ -974,7 +989,7 @@ VideoParBlock<N> par_block(const VideoPar *hpar, int n) {
 template <int N>
 cudaError_t query_pool_n(const Ctx &c, const VideoPar *hpar, cudaStream_t s) {
     VideoParBlock<N> blk = par_block<N>(hpar, c.V);   // copied into the launch parameters
-    const dim3 grid((unsigned)((c.D + 31) / 32), (unsigned)c.V);
+    const dim3 grid((unsigned)((c.D + 63) / 64), (unsigned)c.V);
     void *args[] = {const_cast<Ctx *>(&c), &blk};
     const void *fn = c.dtype == WZ_DTYPE_BF16 ? (const void *)query_pool_kernel<__nv_bfloat16, N>
                                               : (const void *)query_pool_kernel<float, N>;
