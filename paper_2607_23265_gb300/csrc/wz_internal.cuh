@@ -191,20 +191,6 @@ __device__ __forceinline__ void unpack(const uint4 &v, float (&f)[4], float *) {
     f[2] = __uint_as_float(v.z); f[3] = __uint_as_float(v.w);
 }
 
-__device__ __forceinline__ uint4 ldg_stream(const uint4 *p) {
-    uint4 r;
-    asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
-                 : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w) : "l"(p));
-    return r;
-}
-
-template <typename T>
-__device__ __forceinline__ float load_scalar(const T *p);
-template <> __device__ __forceinline__ float load_scalar<float>(const float *p) { return *p; }
-template <> __device__ __forceinline__ float load_scalar<__nv_bfloat16>(const __nv_bfloat16 *p) {
-    return __bfloat162float(*p);
-}
-
 template <typename T>
 __device__ __forceinline__ T from_float(float v);
 template <> __device__ __forceinline__ float from_float<float>(float v) { return v; }
