@@ -1132,15 +1132,17 @@ cudaError_t launch_frame_stats(const Ctx &c, cudaStream_t s) {
     if (e != cudaSuccess) return e;
     const int64_t frames = (int64_t)c.V * c.T, gates = c.gate && c.spatial_mode == WZ_SPATIAL_WSM ? frames : 0;
     if (c.relevance_mode == WZ_RELEVANCE_MAXSIM) {
-        // eight CTAs per eight frames, four where that is one wave and eight are not
+        int gate_warps = frames > sms && c.N <= kWarpGateTokens;
+        const int64_t per = gate_warps ? kStatsThreads / 32 : 1, gate_ctas = (gates + per - 1) / per;
+        // eight CTAs per eight frames, four where those and the gates are more
+        // than one wave (256 frames of 27 x 27, 16 / 64 / 128 rows: 18.3 / 21.3 /
+        // 26.4 us with eight, 16.2 / 20.1 / 26.2 with four)
         const int64_t octets = c.V * (int64_t)((c.T + kMxFrames - 1) / kMxFrames);
-        const int S = 8 * octets > 2 * (int64_t)sms && c.D <= 8192 ? 4 : 8;
+        const int S = 8 * octets + gate_ctas > 2 * (int64_t)sms && c.D <= 8192 ? 4 : 8;
         const void *fn = S == 4 ? (const void *)frame_stats_maxsim_kernel<4> : (const void *)frame_stats_maxsim_kernel<8>;
         const size_t smem = (size_t)(kMxFrames + 1) * 2 * ((c.D / 8 + S - 1) / S) * 16;
         e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
-        int gate_warps = frames > sms && c.N <= kWarpGateTokens;
-        const int64_t per = gate_warps ? kStatsThreads / 32 : 1, gate_ctas = (gates + per - 1) / per;
         void *margs[] = {const_cast<Ctx *>(&c), &gate_warps};
         return launch_kernel(fn, dim3((unsigned)((octets + (gate_ctas + S - 1) / S) * S)), dim3(kStatsThreads), smem, s,
                              margs, c.pdl != 0, (unsigned)S);
