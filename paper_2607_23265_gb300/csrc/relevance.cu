@@ -636,7 +636,8 @@ __device__ __forceinline__ void partial_sums(const float4 *P, int nv, int i, con
 // r_t = cos(v_bar_t, u_q) and delta_t = 1 - cos(v_bar_t, v_bar_{t-1})
 // clamped to [0, 2] (Eq. 7) in fp64.  Another CTA per frame forms its gate
 // (where there is one).  Bound by the latency of these steps: 64 frames of
-// 13 x 13 x 3584 take 6.0 us (first CTA past its wait to the last one's end);
+// 13 x 13 x 3584 take 4.6 us (first CTA past its wait to the last one's end);
+// 6.0 us with the slots' divisions after the wait,
 // 8.2 us with the partials of the two frames read one after the other, two at
 // a time, 64-bit divisions, and the gate in the other half of the CTA.
 __global__ void __launch_bounds__(512, 2) frame_stats_kernel(Ctx c) {

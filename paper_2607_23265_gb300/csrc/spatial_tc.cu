@@ -24,6 +24,16 @@
 // wait for the temporal kernel.  Tensor path, at most kCompactFrames frames
 // and maps whose 16-row group fits in shared memory; spatial_wsm_kernel
 // serves the rest.
+//
+// Bound by instruction issue on many frames (2048 of 13 x 13 x 3584: 38.9 M
+// warp instructions, 55 % issue at 24 warps per SM, 66 us under the profiler),
+// by the latency of one group on few (64 frames: 5.9 us past the wait).  Rows
+// in packed pairs over the exact support, zero weights instead of tests, and
+// the group's frame found by every warp: 32 videos of 64 frames 746.8 -> 740.0
+// us per call, 256 of 27 x 27 415.1 -> 412.0, 64 of 13 x 13 55.2 -> 54.5.
+// Measured and not taken: a group formed before the wait to have its
+// instructions at hand (+4 us: the last CTAs start when the temporal kernel has
+// ended), odd map rows staged from a shifted copy of A' (-0.2 % for 4 KB).
 #include <algorithm>
 
 #include "wz_ptx.cuh"
