@@ -585,7 +585,13 @@ __device__ __forceinline__ void frame_slots(const Ctx &c, int64_t f, int64_t &sl
 
 // r_t and delta_t of frame f = (v, t) from r's and delta's cosines (lanes 0 and
 // 1 of a warp hold them, so that the two inverse square roots run side by
-// side).
+// side).  The cosine num * rsqrt(den2) of equal frames may miss 1 by its own
+// rounding (an ulp of rsqrt, a half each of the products: less than 2^-51), so
+// up to that delta_t is 0: a still video's gamma_t, min-max normalised, would be
+// 1 otherwise.  (The square root and the division, whose cosine of equal frames
+// is exactly 1, take 0.8 us more on 64 frames.)
+constexpr double kCosineRounding = 1.0 / (1ull << 51);
+
 __device__ __forceinline__ void frame_result(const Ctx &c, int64_t f, int v, int t, int lane, double cosine) {
     if (lane == 0) {
         const double r = c.ext_r ? (double)c.ext_r[f] : cosine;   // an external scorer's r_t
@@ -593,7 +599,8 @@ __device__ __forceinline__ void frame_result(const Ctx &c, int64_t f, int v, int
         if (c.frame_scores) c.frame_scores[f] = (float)r;
     }
     if (lane == 1) {
-        const double d = t > 0 ? fmin(2.0, fmax(0.0, 1.0 - cosine)) + 0.0 : 0.0;   // + 0.0: never -0
+        const double away = 1.0 - cosine;
+        const double d = t > 0 && away > kCosineRounding ? fmin(2.0, away) : 0.0;   // (NaN: 0)
         c.fr[4 * f + 1] = d;
         if (c.drange) {   // non-negative doubles order like their bit patterns
             const unsigned long long bits = (unsigned long long)__double_as_longlong(d);
