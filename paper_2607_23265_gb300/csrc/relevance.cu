@@ -610,6 +610,24 @@ __device__ __forceinline__ void frame_result(const Ctx &c, int64_t f, int v, int
     }
 }
 
+// <a, b> over four channels as two sums (even and odd ones).  A thread adds one
+// number per vector to its running sums, so that these are short chains.
+__device__ __forceinline__ f2_t dot4(const float4 &a, const float4 &b) {
+    return fma2(pack2(a.x, a.y), pack2(b.x, b.y), fma2(pack2(a.z, a.w), pack2(b.z, b.w), 0ull));
+}
+__device__ __forceinline__ float pair_sum(f2_t v) {
+    const float2 s = unpack2(v);
+    return s.x + s.y;
+}
+
+// The squares and products of a frame's sums are fp32 within kStatsParts parts
+// of the channels (trees that stop there) and fp64 over the parts: delta_t of a
+// quiet video is a small difference of them, and gamma_t magnifies it.  Its rms
+// error there, in 1e-8: 1.3 to 1.4 at D = 3584 and 1.4 to 3.3 at 8192 to 32768
+// in every kernel below; 2.0 to 2.7 and 4.7 to 14 with chains over all of a
+// thread's channels and one part per warp.
+constexpr int kStatsParts = 32;
+
 // Channels 4 i .. 4 i + 3 of the sums of FPB + 1 frames: the first two partials
 // of every frame in flight together, further ones (frames of more than two
 // CTAs' tokens) after them, in slot order.
@@ -638,17 +656,16 @@ __device__ __forceinline__ void partial_sums(const float4 *P, int nv, int i, con
 
 // One CTA per frame: the frame sums (fixed list of CTA partials) for all
 // channels, read as 16-byte vectors, up to four partials of the frame and four
-// of the one before it in flight; fp32 products summed over each thread's
-// channels and across each warp, the warp totals in fp64; then
-// r_t = cos(v_bar_t, u_q) and delta_t = 1 - cos(v_bar_t, v_bar_{t-1})
-// clamped to [0, 2] (Eq. 7) in fp64.  Another CTA per frame forms its gate
+// of the one before it in flight; fp32 products summed to kStatsParts parts,
+// these in fp64; then r_t = cos(v_bar_t, u_q) and delta_t = 1 - cos(v_bar_t,
+// v_bar_{t-1}) clamped to [0, 2] (Eq. 7) in fp64.  Another CTA per frame forms its gate
 // (where there is one).  Bound by the latency of these steps: 64 frames of
 // 13 x 13 x 3584 take 4.6 us (first CTA past its wait to the last one's end);
 // 6.0 us with the slots' divisions after the wait,
 // 8.2 us with the partials of the two frames read one after the other, two at
 // a time, 64-bit divisions, and the gate in the other half of the CTA.
 __global__ void __launch_bounds__(512, 2) frame_stats_kernel(Ctx c) {
-    __shared__ float wsum[16][5];
+    __shared__ float wsum[kStatsParts][5];
     __shared__ float gate_map[WZ_MAX_HW * WZ_MAX_HW];   // the frame's saliency map
     const int VT = c.V * c.T, f = (int)blockIdx.x;
     const int v = f / c.T, t = f - v * c.T;
@@ -666,7 +683,7 @@ __global__ void __launch_bounds__(512, 2) frame_stats_kernel(Ctx c) {
     const float4 *Pf = reinterpret_cast<const float4 *>(c.part) + (size_t)sf_at * nv;
     const float4 *Pp = reinterpret_cast<const float4 *>(c.part) + (size_t)sp_at * nv;
     const float4 *Qv = reinterpret_cast<const float4 *>(c.qbar32 + (size_t)v * c.D);
-    float p0 = 0.f, p1 = 0.f, p2 = 0.f, p3 = 0.f, p4 = 0.f;
+    f2_t s0 = 0ull, s1 = 0ull, s2 = 0ull, s3 = 0ull, s4 = 0ull;
     const int nmax = max(nf, np);
     for (int i = threadIdx.x; i < nv; i += blockDim.x) {
         const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -692,34 +709,42 @@ __global__ void __launch_bounds__(512, 2) frame_stats_kernel(Ctx c) {
             fm[2] = sf.z / (float)c.N;
             fm[3] = sf.w / (float)c.N;
         }
-        p0 = fmaf(sf.x, q.x, fmaf(sf.y, q.y, fmaf(sf.z, q.z, fmaf(sf.w, q.w, p0))));
-        p1 = fmaf(sf.x, sf.x, fmaf(sf.y, sf.y, fmaf(sf.z, sf.z, fmaf(sf.w, sf.w, p1))));
-        p2 = fmaf(sf.x, sp.x, fmaf(sf.y, sp.y, fmaf(sf.z, sp.z, fmaf(sf.w, sp.w, p2))));
-        p3 = fmaf(q.x, q.x, fmaf(q.y, q.y, fmaf(q.z, q.z, fmaf(q.w, q.w, p3))));
-        p4 = fmaf(sp.x, sp.x, fmaf(sp.y, sp.y, fmaf(sp.z, sp.z, fmaf(sp.w, sp.w, p4))));
+        s0 = add2(s0, dot4(sf, q));
+        s1 = add2(s1, dot4(sf, sf));
+        s2 = add2(s2, dot4(sf, sp));
+        s3 = add2(s3, dot4(q, q));
+        s4 = add2(s4, dot4(sp, sp));
     }
-    for (int o = 16; o > 0; o >>= 1) {
+    float p0 = pair_sum(s0), p1 = pair_sum(s1), p2 = pair_sum(s2), p3 = pair_sum(s3), p4 = pair_sum(s4);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    auto halve = [&](int o) {
         p0 += __shfl_xor_sync(0xffffffffu, p0, o);
         p1 += __shfl_xor_sync(0xffffffffu, p1, o);
         p2 += __shfl_xor_sync(0xffffffffu, p2, o);
         p3 += __shfl_xor_sync(0xffffffffu, p3, o);
         p4 += __shfl_xor_sync(0xffffffffu, p4, o);
-    }
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    if (lane == 0) {
-        wsum[warp][0] = p0;
-        wsum[warp][1] = p1;
-        wsum[warp][2] = p2;
-        wsum[warp][3] = p3;
-        wsum[warp][4] = p4;
+    };
+    halve(16);
+    halve(8);
+    halve(4);
+    if (nw == 16) halve(2);
+    const int parts = kStatsParts / nw;   // of a warp: 2 of 16 warps, 4 of 8
+    if (lane < parts) {
+        float *w = wsum[warp * parts + lane];
+        w[0] = p0;
+        w[1] = p1;
+        w[2] = p2;
+        w[3] = p3;
+        w[4] = p4;
     }
     __syncthreads();
     if (warp == 0) {
-        // lane 4 k + h (k < 5) sums quantity k over the warps h, h + 4, ..; the
-        // four parts in a tree
+        // lane 4 k + h (k < 5) sums quantity k over the parts h, h + 4, ..; the
+        // four sums in a tree
         double acc = 0.0;
         if (lane < 20)
-            for (int w = lane & 3; w < nw; w += 4) acc += (double)wsum[w][lane >> 2];
+#pragma unroll
+            for (int w = 0; w < kStatsParts; w += 4) acc += (double)wsum[w + (lane & 3)][lane >> 2];
         acc += __shfl_xor_sync(0xffffffffu, acc, 1);
         acc += __shfl_xor_sync(0xffffffffu, acc, 2);
         const double vq = __shfl_sync(0xffffffffu, acc, 0), vv = __shfl_sync(0xffffffffu, acc, 4);
@@ -742,7 +767,8 @@ constexpr int kStatsFrames = 4;
 template <int FPB>
 __global__ void __launch_bounds__(kStatsThreads, 3) frame_stats_many_kernel(Ctx c, int gate_warps) {
     constexpr int NW = kStatsThreads / 32, NQ = 3 * FPB + 2;   // vq, vv, vp of each frame; qq, the first pp
-    __shared__ float wsum[NW][NQ];
+    constexpr int PW = kStatsParts / NW;   // parts of a warp
+    __shared__ float wsum[kStatsParts][NQ];
     __shared__ float gate_map[WZ_MAX_HW * WZ_MAX_HW];
     static_assert(NW * kWarpGateTokens <= WZ_MAX_HW * WZ_MAX_HW && FPB <= NW, "a map and a frame per warp");
     const int per_video = (c.T + FPB - 1) / FPB, nstat = c.V * per_video;
@@ -770,9 +796,6 @@ __global__ void __launch_bounds__(kStatsThreads, 3) frame_stats_many_kernel(Ctx 
     float acc[NQ];
 #pragma unroll
     for (int k = 0; k < NQ; ++k) acc[k] = 0.f;
-    auto dot4 = [](const float4 &a, const float4 &b, float s) {
-        return fmaf(a.x, b.x, fmaf(a.y, b.y, fmaf(a.z, b.z, fmaf(a.w, b.w, s))));
-    };
 #pragma unroll 1
     for (int i = threadIdx.x; i < nv; i += kStatsThreads) {
         const float4 q = Qv[i];
@@ -787,28 +810,29 @@ __global__ void __launch_bounds__(kStatsThreads, 3) frame_stats_many_kernel(Ctx 
                 fm[2] = sf[k + 1].z / (float)c.N;
                 fm[3] = sf[k + 1].w / (float)c.N;
             }
-            acc[3 * k] = dot4(sf[k + 1], q, acc[3 * k]);
-            acc[3 * k + 1] = dot4(sf[k + 1], sf[k + 1], acc[3 * k + 1]);
-            acc[3 * k + 2] = dot4(sf[k + 1], sf[k], acc[3 * k + 2]);
+            acc[3 * k] += pair_sum(dot4(sf[k + 1], q));
+            acc[3 * k + 1] += pair_sum(dot4(sf[k + 1], sf[k + 1]));
+            acc[3 * k + 2] += pair_sum(dot4(sf[k + 1], sf[k]));
         }
-        acc[3 * FPB] = dot4(q, q, acc[3 * FPB]);
-        acc[3 * FPB + 1] = dot4(sf[0], sf[0], acc[3 * FPB + 1]);
+        acc[3 * FPB] += pair_sum(dot4(q, q));
+        acc[3 * FPB + 1] += pair_sum(dot4(sf[0], sf[0]));
     }
-    for (int o = 16; o > 0; o >>= 1)
+    for (int o = 16; o >= PW; o >>= 1)
 #pragma unroll
         for (int k = 0; k < NQ; ++k) acc[k] += __shfl_xor_sync(0xffffffffu, acc[k], o);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (lane == 0)
+    if (lane < PW)
 #pragma unroll
-        for (int k = 0; k < NQ; ++k) wsum[warp][k] = acc[k];
+        for (int k = 0; k < NQ; ++k) wsum[warp * PW + lane][k] = acc[k];
     __syncthreads();
     if (warp < nf) {
-        // warp k's frame: lane 4 m + h (m < 5) sums quantity m over the warps h, h + 4
+        // warp k's frame: lane 4 m + h (m < 5) sums quantity m over the parts h, h + 4, ..
         const int m = lane >> 2;
         const int col = m < 3 ? 3 * warp + m : m == 3 ? 3 * FPB : warp == 0 ? 3 * FPB + 1 : 3 * (warp - 1) + 1;
         double s = 0.0;
         if (lane < 20)
-            for (int w = lane & 3; w < NW; w += 4) s += (double)wsum[w][col];
+#pragma unroll
+            for (int w = 0; w < kStatsParts; w += 4) s += (double)wsum[w + (lane & 3)][col];
         s += __shfl_xor_sync(0xffffffffu, s, 1);
         s += __shfl_xor_sync(0xffffffffu, s, 2);
         const double vq = __shfl_sync(0xffffffffu, s, 0), vv = __shfl_sync(0xffffffffu, s, 4);
@@ -839,7 +863,8 @@ constexpr int kMxRows = 4;
 template <int S>
 __global__ void __launch_bounds__(kStatsThreads, 2) frame_stats_maxsim_kernel(Ctx c, int gate_warps) {
     __shared__ float part[kMxFrames][WZ_MAX_LQ_MAXSIM];   // <v_f, q_j> over this CTA's channels
-    __shared__ float wsum[kMxFrames][3];                  // vv, v.v_prev, v_prev.v_prev over them
+    constexpr int PW = kStatsParts / S;   // parts of a warp
+    __shared__ float wsum[kMxFrames][3][PW];              // vv, v.v_prev, v_prev.v_prev over them
     __shared__ double best[kMxFrames / S][4], tot[kMxFrames / S][3];
     __shared__ int slots[kMxFrames + 1], counts[kMxFrames + 1];
     __shared__ float gate_map[WZ_MAX_HW * WZ_MAX_HW];
@@ -891,25 +916,28 @@ __global__ void __launch_bounds__(kStatsThreads, 2) frame_stats_maxsim_kernel(Ct
     }
     __syncthreads();
     {
-        auto dot4 = [](const float4 &a, const float4 &b, float s) {
-            return fmaf(a.x, b.x, fmaf(a.y, b.y, fmaf(a.z, b.z, fmaf(a.w, b.w, s))));
-        };
-        float vv = 0.f, vp = 0.f, pp = 0.f;
-        for (int i = lane; i < nq; i += 32) {
-            const float4 s = sfs[(warp + 1) * 2 * per + i], p = sfs[warp * 2 * per + i];
-            vv = dot4(s, s, vv);
-            vp = dot4(s, p, vp);
-            pp = dot4(p, p, pp);
-        }
-        for (int o = 16; o > 0; o >>= 1) {
+        const float4 *cur = sfs + (warp + 1) * 2 * per, *prev = sfs + warp * 2 * per;
+        f2_t sum[3][2] = {};   // by vector parity: a lane's chains are as short as those of 512 threads
+        for (int i = lane; i < nq; i += 64)
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+                if (i + 32 * h < nq) {
+                    const float4 s = cur[i + 32 * h], p = prev[i + 32 * h];
+                    sum[0][h] = add2(sum[0][h], dot4(s, s));
+                    sum[1][h] = add2(sum[1][h], dot4(s, p));
+                    sum[2][h] = add2(sum[2][h], dot4(p, p));
+                }
+        float vv = pair_sum(add2(sum[0][0], sum[0][1])), vp = pair_sum(add2(sum[1][0], sum[1][1]));
+        float pp = pair_sum(add2(sum[2][0], sum[2][1]));
+        for (int o = 16; o >= PW; o >>= 1) {
             vv += __shfl_xor_sync(0xffffffffu, vv, o);
             vp += __shfl_xor_sync(0xffffffffu, vp, o);
             pp += __shfl_xor_sync(0xffffffffu, pp, o);
         }
-        if (lane == 0) {
-            wsum[warp][0] = vv;
-            wsum[warp][1] = vp;
-            wsum[warp][2] = pp;
+        if (lane < PW) {
+            wsum[warp][0][lane] = vv;
+            wsum[warp][1][lane] = vp;
+            wsum[warp][2][lane] = pp;
         }
     }
     const uint4 *Qr = reinterpret_cast<const uint4 *>(static_cast<const __nv_bfloat16 *>(c.Q) + (size_t)q_row0 * c.D) + v0;
@@ -968,8 +996,14 @@ __global__ void __launch_bounds__(kStatsThreads, 2) frame_stats_maxsim_kernel(Ct
             if (lane == 0) best[m][warp] = x;
         } else if (warp == 4) {   // lane S q + r: quantity q of CTA r
             double s = 0.0;
-            if (lane < 3 * S)
-                s = (double)ptx::ld_cluster(ptx::map_cluster(&wsum[f][lane / S], (uint32_t)(lane % S)));
+            if (lane < 3 * S) {
+                const uint32_t at = ptx::map_cluster(wsum[f][lane / S], (uint32_t)(lane % S));
+                float w[PW];
+#pragma unroll
+                for (int k = 0; k < PW; ++k) w[k] = ptx::ld_cluster(at + 4u * k);
+#pragma unroll
+                for (int k = 0; k < PW; ++k) s += (double)w[k];
+            }
             for (int o = 1; o < S; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
             if (lane < 3 * S && lane % S == 0) tot[m][lane / S] = s;
         }
