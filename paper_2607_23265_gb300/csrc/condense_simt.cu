@@ -172,7 +172,7 @@ cudaError_t launch_simt(const Ctx &c, int sms, cudaStream_t s) {
     const int64_t frames = (int64_t)c.V * c.T;
     int compact = frames <= kCompactFrames ? 1 : 0;
     const size_t smem = kSimtStages * simt_stage_bytes<Tin, TM, TN>() + (compact ? (size_t)(frames + 1) * 4 : 0);
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(fn, smem);
     if (e != cudaSuccess) return e;
     int per_sm = 0;
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, smem)) != cudaSuccess) return e;

@@ -616,7 +616,7 @@ cudaError_t launch_condense_tc(const Ctx &c, cudaStream_t s) {
     if (e != cudaSuccess) return e;
     e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(condense_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
+    e = allow_smem((const void *)condense_tc_kernel, kSmemBytes);
     if (e != cudaSuccess) return e;
     void *args[] = {&maps, const_cast<Ctx *>(&c)};
     return launch_kernel((const void *)condense_tc_kernel, dim3(sms), dim3(kThreads), kSmemBytes, s, args,

@@ -455,7 +455,7 @@ cudaError_t launch_dwt2d(const void *X, int dtype, int T, int H, int W, int D, i
     int vec = ((uintptr_t)X % 16 == 0 && (size_t)D * esz % 16 == 0) ? 1 : 0;
     const void *fn = bf ? pick_dwt2d<__nv_bfloat16>(F, vc) : pick_dwt2d<float>(F, vc);
     if (!fn) return cudaErrorInvalidValue;
-    const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k.smem);
+    const cudaError_t e = allow_smem(fn, k.smem);
     if (e != cudaSuccess) return e;
     Taps t = make_taps(dlo, dhi, F);
     int ct = k.ct;
@@ -471,7 +471,7 @@ cudaError_t launch_idwt2d(const float *LL, const float *LH, const float *HL, con
     const DwtCfg k = dwt_config((size_t)H * dwt_row(2 * wp) * 4, std::max(H, 2 * wp), vc, kIdwtThreads);
     const void *fn = pick_idwt2d(F, vc);
     if (!fn) return cudaErrorInvalidValue;
-    const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k.smem);
+    const cudaError_t e = allow_smem(fn, k.smem);
     if (e != cudaSuccess) return e;
     Taps t = make_taps(rlo, rhi, F);
     int ct = k.ct;

@@ -626,7 +626,7 @@ cudaError_t launch_maxsim_pass(const Ctx &c, int Lqp, int64_t qrows, cudaStream_
     const void *fn = L.G == 4 ? (const void *)maxsim_pass_kernel<4>
                      : L.G == 2 ? (const void *)maxsim_pass_kernel<2>
                                 : (const void *)maxsim_pass_kernel<1>;
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.smem);
+    cudaError_t e = allow_smem(fn, L.smem);
     if (e != cudaSuccess) return e;
     void *args[] = {&maps, const_cast<Ctx *>(&c), &p};
     return launch_kernel(fn, dim3(c.G1), dim3(kXThreads), L.smem, s, args, c.pdl != 0);

@@ -526,7 +526,7 @@ cudaError_t launch_project_gemm(const void *A, int M, int K, const void *B, int 
     p.clear_status = clear_status ? 1 : 0;
     void *args[] = {&maps, &p};
     if (shape.pair) {
-        e = cudaFuncSetAttribute(project_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPairSmemBytes);
+        e = allow_smem((const void *)project_pair_kernel, kPairSmemBytes);
         if (e != cudaSuccess) return e;
         const int tiles = ((M + 2 * kPM - 1) / (2 * kPM)) * ((N + kPN - 1) / kPN);
         const int pairs = tiles < sms / 2 ? tiles : sms / 2;
@@ -537,7 +537,7 @@ cudaError_t launch_project_gemm(const void *A, int M, int K, const void *B, int 
     p.stage_stride = (kPM + p.tileN) * kPK * 2;   // a multiple of 4 KB
     p.stages = (kPStages * kPStageBytes) / p.stage_stride;
     if (p.stages > kPMaxStages) p.stages = kPMaxStages;
-    e = cudaFuncSetAttribute(project_gemm_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPSmemBytes);
+    e = allow_smem((const void *)project_gemm_kernel<0>, kPSmemBytes);
     if (e != cudaSuccess) return e;
     const int tiles = ((M + kPM - 1) / kPM) * ((N + p.tileN - 1) / p.tileN);
     const int grid = tiles < sms ? tiles : sms;
@@ -570,7 +570,7 @@ cudaError_t launch_maxsim_gemm(const void *X, int M, int K, const void *QHL, int
     if (e != cudaSuccess) return e;
     e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(project_gemm_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPSmemBytes);
+    e = allow_smem((const void *)project_gemm_kernel<1>, kPSmemBytes);
     if (e != cudaSuccess) return e;
     const int tiles = (M + kPM - 1) / kPM;
     const int grid = tiles < sms ? tiles : sms;

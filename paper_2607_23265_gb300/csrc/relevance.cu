@@ -1146,7 +1146,7 @@ int relevance_grid(const Ctx &c) {
     int dev = 0, sms = 0, per_sm = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
-    if (cudaFuncSetAttribute(r.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)r.smem) != cudaSuccess) return 0;
+    if (allow_smem(r.fn, r.smem) != cudaSuccess) return 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, r.fn, r.threads, r.smem) != cudaSuccess) return 0;
     if (per_sm < 1) per_sm = 1;
     const int64_t total = (int64_t)c.V * c.T * c.N;
@@ -1160,7 +1160,7 @@ int relevance_grid(const Ctx &c) {
 cudaError_t launch_relevance_pass(const Ctx &c, cudaStream_t s) {
     RelCfg r;
     if (!pick_any(c, r)) return cudaErrorInvalidValue;
-    cudaError_t e = cudaFuncSetAttribute(r.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)r.smem);
+    cudaError_t e = allow_smem(r.fn, r.smem);
     if (e != cudaSuccess) return e;
     void *args[] = {const_cast<Ctx *>(&c), &r.sh};
     return launch_kernel(r.fn, dim3(c.G1), dim3(r.threads), r.smem, s, args, c.pdl != 0);
@@ -1183,7 +1183,7 @@ cudaError_t launch_frame_stats(const Ctx &c, cudaStream_t s) {
         const int S = 8 * octets + gate_ctas > 2 * (int64_t)sms && c.D <= 8192 ? 4 : 8;
         const void *fn = S == 4 ? (const void *)frame_stats_maxsim_kernel<4> : (const void *)frame_stats_maxsim_kernel<8>;
         const size_t smem = (size_t)(kMxFrames + 1) * 2 * ((c.D / 8 + S - 1) / S) * 16;
-        e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        e = allow_smem(fn, smem);
         if (e != cudaSuccess) return e;
         void *margs[] = {const_cast<Ctx *>(&c), &gate_warps};
         return launch_kernel(fn, dim3((unsigned)((octets + (gate_ctas + S - 1) / S) * S)), dim3(kStatsThreads), smem, s,

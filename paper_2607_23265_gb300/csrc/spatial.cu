@@ -500,7 +500,7 @@ cudaError_t launch_spatial(const Ctx &c, cudaStream_t s) {
     // the compact row list when its prefix fits without costing a resident CTA
     const size_t smem_c = spatial_compact_smem_bytes(c);
     const size_t smem_max = plain || (int64_t)c.V * c.T > kCompactFrames ? smem : smem_c;
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_max);
+    cudaError_t e = allow_smem(fn, smem_max);
     if (e != cudaSuccess) return e;
     int dev = 0, sms = 0, per_sm = 0, per_sm_c = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;

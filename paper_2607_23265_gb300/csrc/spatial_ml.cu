@@ -238,7 +238,7 @@ cudaError_t launch_spatial_ml(const Ctx &c, cudaStream_t s) {
     else if (c.H <= 32) fn = (const void *)spatial_ml_kernel<32>;
     else if (c.H <= 64) fn = (const void *)spatial_ml_kernel<64>;
     else return cudaErrorInvalidValue;
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(fn, smem);
     if (e != cudaSuccess) return e;
     int dev = 0, sms = 0, per_sm = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;

@@ -557,7 +557,7 @@ __global__ void __launch_bounds__(kTemporalThreads) temporal_kernel(Ctx c) {
 
 cudaError_t launch_temporal(const Ctx &c, cudaStream_t s) {
     const size_t smem = temporal_smem_bytes(c.T, c.wta_levels);
-    cudaError_t e = cudaFuncSetAttribute(temporal_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem((const void *)temporal_kernel, smem);
     if (e != cudaSuccess) return e;
     void *args[] = {const_cast<Ctx *>(&c)};
     return launch_kernel((const void *)temporal_kernel, dim3(c.V + (c.wsm_levels > 1 ? kMLParts : 1)), dim3(temporal_threads(c.T)), smem, s, args,

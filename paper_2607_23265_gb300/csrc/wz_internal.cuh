@@ -159,6 +159,22 @@ inline cudaError_t launch_kernel(const void *fn, dim3 grid, dim3 block, size_t s
     return cudaLaunchKernelExC(&cfg, fn, args);
 }
 
+// Lets launches of fn have `need` bytes of dynamic shared memory.  The limit
+// belongs to the function, not to a call, and calls on other threads may need
+// other sizes: it is set once, to all that a CTA of fn can have, and never
+// lowered between another thread's setting and its launch.
+inline cudaError_t allow_smem(const void *fn, size_t need) {
+    cudaFuncAttributes a;
+    cudaError_t e = cudaFuncGetAttributes(&a, fn);
+    if (e != cudaSuccess || need <= (size_t)a.maxDynamicSharedSizeBytes) return e;
+    int dev = 0, most = 0;
+    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+    if ((e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess) return e;
+    most -= (int)a.sharedSizeBytes;
+    if (need > (size_t)most) return cudaErrorInvalidValue;
+    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+}
+
 __device__ __forceinline__ int ext_index(int i, int n, int mode) {
     if (i >= 0 && i < n) return i;
     if (mode == WZ_MODE_ZERO) return -1;
