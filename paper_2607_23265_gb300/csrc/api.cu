@@ -348,6 +348,7 @@ int run_condense(const CondenseRequest &r) {
     c.out_rel = r.out_relevance;
     if (r.device_status) c.status = r.device_status;
     else c.clear_status = 1;
+    c.sms = sm_count();
     c.G1 = relevance_grid(c);
     if (c.G1 < 1) {
         cudaGetLastError();
@@ -814,6 +815,7 @@ int wz_relevance(const void *features, int T, int H, int W, int D, int dtype, co
     c.a = token_scores;
     c.frame_scores = frame_scores;
     c.frame_mean = frame_mean;
+    c.sms = sm_count();
     c.G1 = relevance_grid(c);
     if (c.G1 < 1) {
         cudaGetLastError();

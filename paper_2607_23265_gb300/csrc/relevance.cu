@@ -1090,7 +1090,7 @@ void relevance_config(const Ctx &c, RelCfg &r) {
     const int w = sh.gthreads / 32;
     sh.groups = 1;
     if (kNarrow) sh.groups = std::max(1, (16 / w) * w >= 15 ? 16 / w : kRelMaxWarps / w);
-    const int64_t per_cta = ((int64_t)c.V * c.T * c.N + 151) / 152;
+    const int64_t per_cta = ((int64_t)c.V * c.T * c.N + c.sms - 1) / c.sms;
     sh.groups = (int)std::min<int64_t>(sh.groups, std::max<int64_t>(1, per_cta / 32));
     const size_t wpart = (size_t)2 * w * 2 * kRelWindow * 4;
     size_t csum = 0, ring = 0;
@@ -1142,15 +1142,13 @@ bool pick_any(const Ctx &c, RelCfg &r) {
 
 int relevance_grid(const Ctx &c) {
     RelCfg r;
-    if (!pick_any(c, r)) return 0;
-    int dev = 0, sms = 0, per_sm = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return 0;
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
+    if (c.sms < 1 || !pick_any(c, r)) return 0;
+    int per_sm = 0;
     if (allow_smem(r.fn, r.smem) != cudaSuccess) return 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, r.fn, r.threads, r.smem) != cudaSuccess) return 0;
     if (per_sm < 1) per_sm = 1;
     const int64_t total = (int64_t)c.V * c.T * c.N;
-    int64_t g = (int64_t)sms * per_sm;
+    int64_t g = (int64_t)c.sms * per_sm;
     const int64_t min_tokens = 16;
     g = std::min<int64_t>(g, (total + min_tokens - 1) / min_tokens);
     g = std::min<int64_t>(g, kG1Max);
@@ -1168,10 +1166,7 @@ cudaError_t launch_relevance_pass(const Ctx &c, cudaStream_t s) {
 
 cudaError_t launch_frame_stats(const Ctx &c, cudaStream_t s) {
     void *args[] = {const_cast<Ctx *>(&c)};
-    int dev = 0, sms = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return e;
+    const int sms = c.sms;
     const int64_t frames = (int64_t)c.V * c.T, gates = c.gate && c.spatial_mode == WZ_SPATIAL_WSM ? frames : 0;
     if (c.relevance_mode == WZ_RELEVANCE_MAXSIM) {
         int gate_warps = frames > sms && c.N <= kWarpGateTokens;
@@ -1183,7 +1178,7 @@ cudaError_t launch_frame_stats(const Ctx &c, cudaStream_t s) {
         const int S = 8 * octets + gate_ctas > 2 * (int64_t)sms && c.D <= 8192 ? 4 : 8;
         const void *fn = S == 4 ? (const void *)frame_stats_maxsim_kernel<4> : (const void *)frame_stats_maxsim_kernel<8>;
         const size_t smem = (size_t)(kMxFrames + 1) * 2 * ((c.D / 8 + S - 1) / S) * 16;
-        e = allow_smem(fn, smem);
+        const cudaError_t e = allow_smem(fn, smem);
         if (e != cudaSuccess) return e;
         void *margs[] = {const_cast<Ctx *>(&c), &gate_warps};
         return launch_kernel(fn, dim3((unsigned)((octets + (gate_ctas + S - 1) / S) * S)), dim3(kStatsThreads), smem, s,

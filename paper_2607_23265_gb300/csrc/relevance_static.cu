@@ -114,6 +114,7 @@ extern "C" int wz_relevance_static(const void *features, int T, int H, int W, in
     c.D = D;
     c.N = H * W;
     c.dtype = dtype;
+    c.sms = sm_count();
     c.G1 = relevance_grid(c);
     if (c.G1 < 1) {
         cudaGetLastError();

@@ -521,7 +521,7 @@ __global__ void __launch_bounds__(kTemporalThreads) temporal_kernel(Ctx c) {
     }
     int pre[6], tot[6];
     block_excl_scan<6>(part, iscr, pre, tot);
-    const int narrow = c.V == 1 && tot[2] + tot[3] <= kNarrowUnits ? 1 : 0;
+    const int narrow = c.V == 1 && tot[2] + tot[3] <= kNarrowUnits * c.sms ? 1 : 0;
     const int utot = narrow ? tot[4] + tot[5] : tot[2] + tot[3];
     int o = pre[0], wo = pre[1], u = narrow ? pre[4] : pre[2], uB = narrow ? tot[4] + pre[5] : tot[2] + pre[3];
     for (int t = t0; t < t1; ++t) {

@@ -35,6 +35,7 @@ struct Ctx {
     int dtype;            // WZ_DTYPE_*
     int hp, wp;           // WSM subband sizes
     int K_pad;            // N rounded up to 32 (row length of the operator)
+    int sms;              // SMs of the device
     int G1;               // relevance CTAs actually launched
     int n_ct;             // 128-channel tiles
     int max_units_v;      // unit-list capacity per video
@@ -157,6 +158,13 @@ inline cudaError_t launch_kernel(const void *fn, dim3 grid, dim3 block, size_t s
     cfg.attrs = attr;
     cfg.numAttrs = n;
     return cudaLaunchKernelExC(&cfg, fn, args);
+}
+
+// SMs of the current device; 0 on an error.
+inline int sm_count() {
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+    return cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess ? sms : 0;
 }
 
 // Lets launches of fn have `need` bytes of dynamic shared memory.  The limit
@@ -291,10 +299,6 @@ __host__ __device__ __forceinline__ size_t tile_index(int64_t r, int k, int64_t 
            (size_t)(r & 7) * 8 + (size_t)(k & 7);
 }
 
-// Channel tiles per tensor-core work unit for a column block of ncp (padded)
-// output tokens.  Up to 128 tokens, hi and lo are one MMA of N = 2*ncp and
-// take 2*ncp accumulator columns per tile; above, they accumulate into the
-// same ncp columns.  Either way a unit fits one 256-column buffer.
 // Subband length after l cascaded levels of an F-tap DWT: n_l = (n_{l-1} + F - 1) / 2.
 __host__ __device__ __forceinline__ int level_size(int n, int F, int l) {
     for (int k = 0; k < l; ++k) n = (n + F - 1) / 2;
@@ -313,13 +317,15 @@ __host__ __device__ __forceinline__ int gate_floats(int H, int W, int F, int J) 
 // ncp <= 64, else two MMAs of N = ncp; a unit spans as many 128-channel tiles
 // (at most 4) as the 512 accumulator columns of tensor memory hold, so each
 // operator tile in shared memory serves 2-4 channel tiles.  Narrow units (one
-// video with at most kNarrowUnits wide ones; the temporal kernel
+// video with at most kNarrowUnits wide ones per SM; the temporal kernel
 // decides) take, for blocks of up to 128 tokens, the tiles of half of the
 // columns: more, smaller units whose epilogue overlaps the next unit's main
-// loop.  Calls, wide / narrow: 64 frames of 13 x 13 x 3584 (224 wide units)
-// 58.8 / 57.0 us, 128 of 16 x 16 (448) 103.6 / 101.8; with the max-over-query
-// scorer (896) 146.0 / 147.1, 256 of 27 x 27 413 / 420, 32 videos of 64 frames
-// 763 / 779 (there the operator's extra reads cost more).
+// loop, and a shorter last wave; the operator is read more often.  Calls of one
+// video, 3584 channels, wide / narrow: 64 frames of 13 x 13 (224 wide units)
+// 53.8 / 53.3 us, 128 (455) 74.4 / 74.2, 128 of 16 x 16 (455) 93.7 / 90.6; above
+// the line 160 of 16 x 16 (560) 113.2 / 109.3 and 256 (903) 161.6 / 159.2, but
+// with the max-over-query scorer (896) 146.0 / 147.1, 256 of 27 x 27 (1,400) 413 /
+// 420 and 32 videos of 64 frames 763 / 779: a line that no measured call loses by.
 __host__ __device__ __forceinline__ bool unit_fused(int ncp) { return ncp <= 64; }
 
 __host__ __device__ __forceinline__ int unit_tiles(int ncp, bool narrow) {
@@ -328,7 +334,7 @@ __host__ __device__ __forceinline__ int unit_tiles(int ncp, bool narrow) {
     return cg < 1 ? 1 : (cg > 4 ? 4 : cg);
 }
 
-constexpr int kNarrowUnits = 456;   // three per SM
+constexpr int kNarrowUnits = 3;   // wide units per SM
 
 // ---- launchers (one per kernel family) -------------------------------------
 
