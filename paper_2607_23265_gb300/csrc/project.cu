@@ -14,8 +14,8 @@
 //       each CTA of a cluster of two holds 128 rows of A and 128 of B, so an SM
 //       reads half of what a 128 x 256 tile of its own takes, which bounds the
 //       other kernel; six stages of 32 KB per CTA
-//   project_gemm_kernel   tiles of 128 x tileN on one SM, tileN 256, 128, 64 or
-//       32, so that few rows still spread over the SMs
+//   project_gemm_kernel   tiles of 128 x tileN on one SM, tileN 256, 64 or 32, so
+//       that few rows still spread over the SMs
 // Warps of either:
 //   warp 0     TMA producer (one thread)
 //   warp 1     TMEM allocation and the MMA issuer (one thread; the even CTA's)
@@ -478,8 +478,10 @@ namespace {
 
 // Tile shape of Out[M][N]: what a K step costs an SM in shared-memory cycles
 // (the tile's operands written by TMA and read by the MMA, 2 (128 + tileN); a
-// pair 512 for 256 x 256) times the rounds of tiles over the SMs.  Both layers,
-// against 128 x 256 tiles on one SM everywhere: 18,662 x 3584 x 3584 x 3584
+// pair 512 for 256 x 256) times the rounds of tiles over the SMs.  (128 x 128
+// tiles cost what a pair's do and never take fewer rounds; 128 x 256 ones save
+// the half that an odd number of row blocks leaves empty in pairs, as with 300
+// rows of 10,000 columns.)  Both layers, against 128 x 256 tiles on one SM everywhere: 18,662 x 3584 x 3584 x 3584
 // 595 -> 565 us (1,698 TFLOP/s), 2704 rows 135 -> 128, 300 x 2048 x 2048 x 2048
 // 37.6 -> 27.4, 64 x 3584 x 3584 x 3584 51.6 -> 39.6.
 struct PShape {
@@ -491,7 +493,7 @@ PShape project_shape(int M, int N, int sms) {
     auto ceil_div = [](int64_t a, int64_t b) { return (a + b - 1) / b; };
     PShape best{true, kPN};
     int64_t cost = ceil_div(ceil_div(M, 2 * kPM) * ceil_div(N, kPN), sms / 2) * 512;
-    for (int tn = kPN; tn >= 32; tn >>= 1) {
+    for (const int tn : {kPN, 64, 32}) {
         const int64_t x = ceil_div(ceil_div(M, kPM) * ceil_div(N, tn), sms) * 2 * (kPM + tn);
         if (x < cost) {
             cost = x;
@@ -580,3 +582,14 @@ cudaError_t launch_maxsim_gemm(const void *X, int M, int K, const void *QHL, int
 }
 
 }  // namespace wz
+
+#ifdef WZ_CHECKED
+// Test hook: the tile columns that a layer of the projector takes on the current
+// device, 2 kPN for pairs; negative on an error.
+extern "C" __attribute__((visibility("default"))) int wz_check_project_tile(int rows, int cols) {
+    const int sms = wz::sm_count();
+    if (sms < 1 || rows < 1 || cols < 1) return -1;
+    const wz::PShape shape = wz::project_shape(rows, cols, sms);
+    return shape.pair ? 2 * wz::kPN : shape.tileN;
+}
+#endif

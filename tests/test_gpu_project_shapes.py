@@ -1,6 +1,8 @@
-"""The projector in each of its tile shapes: 128 x 32 .. 256 on one SM and 256 x 256 on a pair of
+"""The projector in each of its tile shapes: 128 x 32, 64 and 256 on one SM and 256 x 256 on a pair of
 SMs, with rows and columns that end inside a tile (and inside either half of a pair's), one K step
 and more K steps than the ring has stages."""
+
+import ctypes as C
 
 import pytest
 
@@ -8,17 +10,27 @@ from test_gpu_project import _case, _check, _hidden_ok, _np, _run, wz  # noqa: F
 
 pytestmark = pytest.mark.gpu
 
+PAIR = 512   # the library's name for 256 x 256 on a pair
 
-@pytest.mark.parametrize("B,D,C,E", [
-    (4100, 64, 320, 512),       # pairs: one K step; columns end in the second tile's first half
-    (300, 192, 3584, 3584),     # pairs: rows end in the first half of the second tile
-    (1500, 640, 1152, 576),     # pairs, then 128 x 64
-    (129, 128, 3584, 64),       # 128 x 64, then 128 x 32
-    (1000, 448, 1152, 3520),    # 128 x 64, then pairs
-    (2500, 128, 320, 4864),     # 128 x 64, then pairs with more tiles than pairs
-    (9800, 64, 256, 256),       # pairs in two rounds' reach, 39 tiles of 256 rows
+
+def _tile(wz, rows, cols):
+    """The tile columns that a layer of `rows` x `cols` takes (the checked library says)."""
+    return C.CDLL(wz.LIB_CHECKED_PATH).wz_check_project_tile(rows, cols)
+
+
+@pytest.mark.parametrize("B,D,C,E,tiles", [
+    (4100, 64, 320, 512, (PAIR, PAIR)),       # one K step; columns end in the second tile's first half
+    (300, 192, 3584, 3584, (PAIR, PAIR)),     # rows end in the first half of the second tile
+    (1500, 640, 1152, 576, (PAIR, 64)),
+    (129, 128, 3584, 64, (64, 32)),
+    (1000, 448, 1152, 3520, (64, PAIR)),
+    (2500, 128, 320, 4864, (64, PAIR)),       # more tiles than pairs
+    (9800, 64, 256, 256, (PAIR, PAIR)),       # 39 tiles of 256 rows: within one round of the pairs
+    (100, 64, 64, 20480, (32, 256)),          # fewer rows than a tile's, 80 tiles of 256 columns
+    (300, 128, 10048, 192, (256, 32)),        # rows and columns end inside the last tiles
 ])
-def test_project_tiles(wz, B, D, C, E):  # noqa: F811
+def test_project_tiles(wz, B, D, C, E, tiles):  # noqa: F811
+    assert (_tile(wz, B, C), _tile(wz, B, E)) == tiles
     Z, W1, b1, W2, b2 = _case(B, D, C, E, seed=B + C)
     out, hidden = _run(wz, Z, W1, b1, W2, b2)
     hg = _np(hidden)
