@@ -314,6 +314,26 @@ int validate(const CondenseRequest &r, std::vector<int64_t> &B, int64_t &rows) {
     return WZ_OK;
 }
 
+// Where the unit query rows of a call with the max-over-query scorer go.  The
+// one pass over the features (token norms, channel sums, token x query-row
+// maxima) wants those of all videos at once: in their own buffer, in the partial
+// slots past the ones in use, or in the operator's memory, which the spatial
+// kernel writes later.  Without room, or where the pass does not apply, the
+// scorer runs video by video through the own buffer.
+enum class QueryRows { kByVideo, kOwn, kSlots, kOperator };
+
+// Lqp: the longest query, padded to 16; qrows: the rows of all videos (qhl_row).
+// *at: their offset in the workspace (kSlots, kOperator).
+QueryRows place_query_rows(const Ctx &c, const Shape &s, const Layout &L, int Lqp, int64_t qrows, size_t *at) {
+    if (!maxsim_pass_supported(c, Lqp)) return QueryRows::kByVideo;
+    const size_t need = (size_t)qrows * s.D * 2;
+    if (need <= (size_t)2 * WZ_MAX_LQ_MAXSIM * s.D * 2) return QueryRows::kOwn;
+    *at = L.part + align_up(((size_t)c.G1 + (size_t)s.V * s.T) * s.D * 4);
+    if (*at + need <= L.fr) return QueryRows::kSlots;
+    *at = L.Wop;
+    return *at + need <= L.total ? QueryRows::kOperator : QueryRows::kByVideo;
+}
+
 int run_condense(const CondenseRequest &r) {
     std::vector<int64_t> B;
     int64_t rows = 0;
@@ -373,26 +393,17 @@ int run_condense(const CondenseRequest &r) {
         return r.events ? cudaEventRecord((cudaEvent_t)r.events[k], r.stream) : cudaSuccess;
     };
     Nvtx whole("wz::condense");
-    // max-over-query scorer: one pass over the features computes the token
-    // norms, the channel sums and the token x query-row maxima where it applies
-    // and the videos' unit query rows have room: in their own buffer, in the
-    // partial slots past the ones in use, or in the operator's memory (written
-    // by the spatial kernel, later)
     const bool maxsim = c.relevance_mode == WZ_RELEVANCE_MAXSIM;
     const int Lq_max = *std::max_element(r.Lq.begin(), r.Lq.end()), Lqp_max = (Lq_max + 15) / 16 * 16;
     bool fused_maxsim = false;
-    const int64_t qrows = qhl_row(qrow, r.V);   // rows of all videos
-    if (maxsim && maxsim_pass_supported(c, Lqp_max)) {
-        const size_t need = (size_t)qrows * s.D * 2;
-        const size_t used = align_up(((size_t)c.G1 + (size_t)s.V * s.T) * s.D * 4);
-        if (need <= (size_t)2 * WZ_MAX_LQ_MAXSIM * s.D * 2) fused_maxsim = true;
-        else if (L.part + used + need <= L.fr) {
-            c.qhl = reinterpret_cast<__nv_bfloat16 *>(ws.ptr + L.part + used);
-            fused_maxsim = true;
-        } else if (L.Wop + need <= L.total) {
-            c.qhl = reinterpret_cast<__nv_bfloat16 *>(ws.ptr + L.Wop);
-            fused_maxsim = true;
-        }
+    int64_t qrows = 0;   // unit query rows of all videos
+    if (maxsim) {
+        qrows = qhl_row(qrow, r.V);
+        size_t at = 0;
+        const QueryRows place = place_query_rows(c, s, L, Lqp_max, qrows, &at);
+        fused_maxsim = place != QueryRows::kByVideo;
+        if (place == QueryRows::kSlots || place == QueryRows::kOperator)
+            c.qhl = reinterpret_cast<__nv_bfloat16 *>(ws.ptr + at);
     }
     WZ_CUDA(mark(2 * WZ_KERNEL_QUERY_POOL));
     if (fused_maxsim) {   // needs no pooled query
@@ -943,5 +954,30 @@ const char *wz_status_string(int status) {
 }
 
 int wz_version(void) { return 100; }
+
+#ifdef WZ_CHECKED
+// Test hook: the QueryRows of a bf16 batch with the max-over-query scorer on the
+// current device, as an int; negative on an error.
+__attribute__((visibility("default"))) int wz_check_query_rows(int V, int T, int H, int W, int D, const int32_t *Lq,
+                                                               const float *ratio) {
+    if (!Lq || !ratio || check_sizes(V, T, H, W, D, WZ_DTYPE_BF16) != WZ_OK) return -1;
+    std::vector<int64_t> B(V);
+    int rows = 0;
+    for (int v = 0; v < V; ++v) {
+        B[v] = budget(T, H * W, ratio[v]);
+        rows += Lq[v];
+    }
+    const Shape s = make_shape(V, T, H, W, D, WZ_DTYPE_BF16, 2, B.data());
+    const Layout L = make_layout(s, true, true);
+    Ctx c{};
+    bind(c, s, L, nullptr);
+    c.relevance_mode = WZ_RELEVANCE_MAXSIM;
+    c.sms = sm_count();
+    c.G1 = relevance_grid(c);
+    size_t at = 0;
+    return c.G1 < 1 ? -1
+                    : (int)place_query_rows(c, s, L, (*std::max_element(Lq, Lq + V) + 15) / 16 * 16, qhl_row(rows, V), &at);
+}
+#endif
 
 }  // extern "C"

@@ -1,32 +1,42 @@
 """The max-over-query scorer on batches: the fused pass with every place its unit query rows can
-take in the workspace, tiles cut at video ends, odd frame counts with two frames per statistics
-CTA, and the per-video path where the fused pass does not apply."""
+take in the workspace, tiles cut at video ends, clusters of the statistics kernel with fewer than
+eight frames, and the per-video path where the fused pass does not apply."""
 
-import numpy as np
+import ctypes as C
+
 import pytest
 import torch
 
-from helpers import accepted_random, compare_condense, oracle_run, to_np64
+from helpers import accepted_random, compare_condense, oracle_run
 
 pytestmark = pytest.mark.gpu
 
+BY_VIDEO, OWN, SLOTS, OPERATOR = range(4)   # where the unit query rows go
+
 CASES = [
-    # V, T, H, W, D, query rows
-    (2, 3, 11, 12, 128, [5, 64]),                          # own query-row buffer
-    (3, 5, 12, 12, 192, [1, 128, 33]),                     # past the column partials in use
-    (16, 11, 12, 12, 64, [128] * 16),                      # in the operator's memory; 176 frames
-    (16, 4, 12, 12, 512, [128, 120] * 8),                  # no room: video by video
-    (5, 4, 9, 9, 128, [3, 17, 128, 64, 1]),                # frames of fewer than 128 tokens
-    (4, 45, 13, 10, 64, [16, 15, 90, 2]),                  # several videos inside a CTA's range
-    (2, 9, 16, 16, 1024, [127, 100]),                      # long queries: small query-row stages
-    (2, 4, 13, 13, 4160, [40, 24]),                        # too wide for the fused pass
+    # V, T, H, W, D, query rows, their place
+    (2, 3, 11, 12, 128, [5, 64], OWN),
+    (3, 5, 12, 12, 192, [1, 128, 33], SLOTS),              # past the column partials in use
+    (16, 11, 12, 12, 64, [128] * 16, OPERATOR),            # 176 frames
+    (16, 4, 12, 12, 512, [128, 120] * 8, BY_VIDEO),        # no room
+    (5, 4, 9, 9, 128, [3, 17, 128, 64, 1], BY_VIDEO),      # frames of fewer than 128 tokens
+    (4, 45, 13, 10, 64, [16, 15, 90, 2], SLOTS),           # several videos inside a CTA's range
+    (2, 9, 16, 16, 1024, [127, 100], SLOTS),               # long queries: small query-row stages
+    (2, 4, 13, 13, 4160, [40, 24], BY_VIDEO),              # too wide for the fused pass
 ]
 
 
-@pytest.mark.parametrize("V,T,H,W,D,Lqs", CASES)
-def test_maxsim_batch_shapes(V, T, H, W, D, Lqs):
+def _place(wz, V, T, H, W, D, Lqs, ratios):
+    """The place that the library chooses (the checked build says)."""
+    fn = C.CDLL(wz.LIB_CHECKED_PATH).wz_check_query_rows
+    return fn(V, T, H, W, D, (C.c_int32 * V)(*Lqs), (C.c_float * V)(*ratios))
+
+
+@pytest.mark.parametrize("V,T,H,W,D,Lqs,place", CASES)
+def test_maxsim_batch_shapes(V, T, H, W, D, Lqs, place):
     import paper_2607_23265_gb300 as wz
     ratios = [(0.2, 0.1, 0.3)[v % 3] for v in range(V)]
+    assert _place(wz, V, T, H, W, D, Lqs, ratios) == place
     vids = [accepted_random(T, H, W, D, lq, r, seed=500 + 7 * k, relevance="maxsim")
             for k, (lq, r) in enumerate(zip(Lqs, ratios))]
     X = torch.stack([x for x, _ in vids]).cuda()
