@@ -7,11 +7,12 @@
 // ring of kSimtStages cp.async stages; a thread forms RT rows x 4 CG columns,
 // products in f32x2 (column pairs), every output one chain in ascending K.
 // Bound by latency for few frames and by the FMA pipe (43 of 75 TFLOP/s) for
-// many.  Before, with one unpipelined 16-token step at a time, 64 x 64 tiles
-// and a grid over every possible tile: 64 frames of 13 x 13 x 3584 96 us (57
-// now), 64 of 27 x 27 x 2048 1.07 ms (0.81 now).
+// many: 64 frames of 13 x 13 x 3584 57 us (96 with one unpipelined 16-token step
+// at a time, 64 x 64 tiles and a grid over every possible tile), 64 of 27 x 27 x
+// 2048 0.81 ms (1.07).
 #include <algorithm>
 
+#include "wz_ptx.cuh"
 #include "wz_spatial.cuh"
 
 namespace wz {
@@ -25,13 +26,6 @@ constexpr int kSimtWRow = kSimtK + 4; // staged operator row: the rows of a warp
 template <typename Tin, int TM, int TN>
 __host__ __device__ constexpr size_t simt_stage_bytes() {
     return (size_t)TM * kSimtWRow * 4 + (size_t)kSimtK * TN * sizeof(Tin);
-}
-
-// 16 bytes global -> shared, zeros when !on (nothing is read then).
-__device__ __forceinline__ void copy16(void *dst, const void *src, bool on) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)),
-                 "l"(src), "r"(on ? 16 : 0)
-                 : "memory");
 }
 
 __device__ __forceinline__ void cols4(const float *p, f2_t (&x)[2]) {
@@ -103,12 +97,12 @@ __global__ void __launch_bounds__((TM / RT) * (TN / (4 * CG))) condense_simt_ker
             constexpr int WQ = kSimtK / 4;                 // 16-byte pieces of an operator row
             for (int k = tid; k < TM * WQ; k += NT) {
                 const int r = k / WQ, q = (k % WQ) * 4;
-                copy16(ws + r * kSimtWRow + q, Wr + (size_t)r * c.K_pad + kc * kSimtK + q, r < n);
+                ptx::copy_async16(ws + r * kSimtWRow + q, Wr + (size_t)r * c.K_pad + kc * kSimtK + q, r < n);
             }
             constexpr int XE = 16 / (int)sizeof(Tin), XQ = TN / XE;   // pieces of a token row
             for (int k = tid; k < kSimtK * XQ; k += NT) {
                 const int r = k / XQ, q = (k % XQ) * XE, tok = kc * kSimtK + r;
-                copy16(xs + r * TN + q, Xf + (size_t)tok * D + q, tok < N && c0 + q < D);
+                ptx::copy_async16(xs + r * TN + q, Xf + (size_t)tok * D + q, tok < N && c0 + q < D);
             }
         };
         f2_t acc[RT][2 * CG];
@@ -119,13 +113,13 @@ __global__ void __launch_bounds__((TM / RT) * (TN / (4 * CG))) condense_simt_ker
 #pragma unroll
         for (int s = 0; s < kSimtStages - 1; ++s) {
             if (s < KC) load(s);
-            asm volatile("cp.async.commit_group;" ::: "memory");
+            ptx::copy_async_commit();
         }
         for (int kc = 0; kc < KC; ++kc) {
-            asm volatile("cp.async.wait_group %0;" ::"n"(kSimtStages - 2) : "memory");
+            ptx::copy_async_wait<kSimtStages - 2>();
             __syncthreads();   // step kc has landed for every thread; step kc - 1 has been read
             if (kc + kSimtStages - 1 < KC) load(kc + kSimtStages - 1);
-            asm volatile("cp.async.commit_group;" ::: "memory");
+            ptx::copy_async_commit();
             const unsigned char *st = ssm + (kc % kSimtStages) * simt_stage_bytes<Tin, TM, TN>();
             const float *ws = reinterpret_cast<const float *>(st) + ty * kSimtWRow;
             const Tin *xs = reinterpret_cast<const Tin *>(st + (size_t)TM * kSimtWRow * 4) + tx * 4;

@@ -12,6 +12,7 @@
 #include <initializer_list>
 
 #include "wz_internal.cuh"
+#include "wz_ptx.cuh"
 
 namespace wz {
 
@@ -224,11 +225,6 @@ constexpr int dwt_ctas(int F) { return F <= 10 ? 3 : F <= 14 ? 2 : 1; }
 // rows that a warp's lanes work on start in different banks (CT = 16).
 __host__ __device__ __forceinline__ int dwt_row(int n) { return n | 1; }
 
-__device__ __forceinline__ void copy_async16(void *dst, const void *src) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
-                 : "memory");
-}
-
 // The CTA's map goes to shared memory in one go (every read in flight at
 // once; cp.async where `vec` says that 16-byte pieces are aligned), then for
 // the width-low and the width-high half: width pass of every row into the
@@ -256,9 +252,9 @@ dwt2d_kernel(const Tin *X, int H, int W, int D, int CT, int mode, int vec, Taps 
         const int nv = nc * (int)sizeof(Tin) / 16, ve = 16 / (int)sizeof(Tin);
         for (int k = threadIdx.x; k < H * W * nv; k += blockDim.x) {
             const int p = k / nv, q = (k - p * nv) * ve, i = p / W;
-            copy_async16(sx + (i * ws + p - i * W) * CT + q, Xf + (size_t)p * D + q);
+            ptx::copy_async16(sx + (i * ws + p - i * W) * CT + q, Xf + (size_t)p * D + q);
         }
-        asm volatile("cp.async.wait_all;" ::: "memory");
+        ptx::copy_async_wait_all();
     } else {
         for (int k = threadIdx.x; k < H * W * nc; k += blockDim.x) {
             const int p = k / nc, q = k - p * nc, i = p / W;
