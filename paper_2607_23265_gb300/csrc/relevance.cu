@@ -237,9 +237,11 @@ struct RelShape {
 template <typename T, int VPT, int MAXTHREADS>
 __global__ void __launch_bounds__(MAXTHREADS, 1) relevance_pass_kernel(Ctx c, RelShape sh) {
     // The producer streams only the features, which the kernels before this
-    // one do not write, so it starts before the wait for the previous grid
-    // (the query pooling) and fills the ring meanwhile; the consumers wait
-    // for it before they read u_q or write anything.
+    // one do not write, so where the launches overlap (the condensation calls;
+    // wz_relevance and wz_relevance_static launch one after the other) it starts
+    // before the wait for the previous grid (the query pooling) and fills the
+    // ring meanwhile; the consumers wait for it before they read u_q or write
+    // anything.
     pdl_trigger();
     constexpr int VEC = VecOf<T>::kElems;
     constexpr int GROUP = kRelGroupTokens;
@@ -1157,7 +1159,7 @@ int relevance_grid(const Ctx &c) {
 
 cudaError_t launch_relevance_pass(const Ctx &c, cudaStream_t s) {
     RelCfg r;
-    if (!pick_any(c, r)) return cudaErrorInvalidValue;
+    if (!pick_any(c, r) || r.sh.stages % r.sh.groups != 0) return cudaErrorInvalidValue;   // (see RelShape)
     cudaError_t e = allow_smem(r.fn, r.smem);
     if (e != cudaSuccess) return e;
     void *args[] = {const_cast<Ctx *>(&c), &r.sh};
