@@ -80,10 +80,10 @@ typedef struct CUstream_st *wz_stream_t;
 #define WZ_PATH_SIMT   2 /* fp32 CUDA-core GEMM                              */
 
 /* Kernels of one condensation call, in launch order (for kernel_events). */
-#define WZ_KERNEL_QUERY_POOL     0 /* u_q                                      */
+#define WZ_KERNEL_QUERY_POOL     0 /* u_q, or the unit query rows (max-over-query, one pass) */
 #define WZ_KERNEL_RELEVANCE      1 /* streaming pass: a_{t,n}, column sums     */
-#define WZ_KERNEL_FRAME_STATS    2 /* fp64 frame sums and dot products          */
-#define WZ_KERNEL_TEMPORAL       3 /* r, delta, gamma, WTA, budgets, offsets    */
+#define WZ_KERNEL_FRAME_STATS    2 /* frame sums, r, delta, gates               */
+#define WZ_KERNEL_TEMPORAL       3 /* gamma, WTA, budgets, offsets              */
 #define WZ_KERNEL_SPATIAL        4 /* operator rows W_m, index map, tail rows   */
 #define WZ_KERNEL_CONDENSE       5 /* Z_m = W_m X_m, packed                     */
 #define WZ_NUM_KERNELS           6
@@ -337,7 +337,7 @@ WZ_API size_t wz_relevance_workspace_size(int T, int H, int W, int D);
  *     SM) is the relevance grid (152 on a GB300 at D = 3584: about T <= 1000
  *     frames fit at that width).
  *   - device_status [1] int32, nullable: as for wz_relevance.  Without it the
- *     array's own status word is zeroed on `stream` (cudaMemsetAsync) and
+ *     array's own status word is zeroed by the call's first kernel and
  *     takes the bits, so a timed-out wait is not reported.
  *   - Every call shares the one array; apart from that status word nothing
  *     in it must start at zero and no state passes from one call to the next,
