@@ -630,6 +630,13 @@ __device__ __forceinline__ float pair_sum(f2_t v) {
 // thread's channels and one part per warp.
 constexpr int kStatsParts = 32;
 
+// Sum of N parts at p, p + stride, .. in fp64, as a tree (N a power of two).
+template <int N>
+__device__ __forceinline__ double parts_sum(const float *p, int stride) {
+    if constexpr (N == 1) return (double)*p;
+    else return parts_sum<N / 2>(p, stride) + parts_sum<N / 2>(p + N / 2 * stride, stride);
+}
+
 // Channels 4 i .. 4 i + 3 of the sums of FPB + 1 frames: the first two partials
 // of every frame in flight together, further ones (frames of more than two
 // CTAs' tokens) after them, in slot order.
@@ -743,10 +750,7 @@ __global__ void __launch_bounds__(512, 2) frame_stats_kernel(Ctx c) {
     if (warp == 0) {
         // lane 4 k + h (k < 5) sums quantity k over the parts h, h + 4, ..; the
         // four sums in a tree
-        double acc = 0.0;
-        if (lane < 20)
-#pragma unroll
-            for (int w = 0; w < kStatsParts; w += 4) acc += (double)wsum[w + (lane & 3)][lane >> 2];
+        double acc = lane < 20 ? parts_sum<kStatsParts / 4>(&wsum[lane & 3][lane >> 2], 4 * 5) : 0.0;
         acc += __shfl_xor_sync(0xffffffffu, acc, 1);
         acc += __shfl_xor_sync(0xffffffffu, acc, 2);
         const double vq = __shfl_sync(0xffffffffu, acc, 0), vv = __shfl_sync(0xffffffffu, acc, 4);
@@ -831,10 +835,7 @@ __global__ void __launch_bounds__(kStatsThreads, 3) frame_stats_many_kernel(Ctx 
         // warp k's frame: lane 4 m + h (m < 5) sums quantity m over the parts h, h + 4, ..
         const int m = lane >> 2;
         const int col = m < 3 ? 3 * warp + m : m == 3 ? 3 * FPB : warp == 0 ? 3 * FPB + 1 : 3 * (warp - 1) + 1;
-        double s = 0.0;
-        if (lane < 20)
-#pragma unroll
-            for (int w = 0; w < kStatsParts; w += 4) s += (double)wsum[w + (lane & 3)][col];
+        double s = lane < 20 ? parts_sum<kStatsParts / 4>(&wsum[lane & 3][col], 4 * NQ) : 0.0;
         s += __shfl_xor_sync(0xffffffffu, s, 1);
         s += __shfl_xor_sync(0xffffffffu, s, 2);
         const double vq = __shfl_sync(0xffffffffu, s, 0), vv = __shfl_sync(0xffffffffu, s, 4);
@@ -1003,8 +1004,7 @@ __global__ void __launch_bounds__(kStatsThreads, 2) frame_stats_maxsim_kernel(Ct
                 float w[PW];
 #pragma unroll
                 for (int k = 0; k < PW; ++k) w[k] = ptx::ld_cluster(at + 4u * k);
-#pragma unroll
-                for (int k = 0; k < PW; ++k) s += (double)w[k];
+                s = parts_sum<PW>(w, 1);
             }
             for (int o = 1; o < S; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
             if (lane < 3 * S && lane % S == 0) tot[m][lane / S] = s;
