@@ -25,8 +25,8 @@
 // and maps whose 16-row group fits in shared memory; spatial_wsm_kernel
 // serves the rest.
 //
-// Bound by instruction issue on many frames (2048 of 13 x 13 x 3584: 38.9 M
-// warp instructions, 55 % issue at 24 warps per SM, 66 us under the profiler),
+// Bound by instruction issue on many frames (2048 of 13 x 13 x 3584: 38.7 M
+// warp instructions, 54 % issue at 23 warps per SM, 65 us under the profiler),
 // by the latency of one group on few (64 frames: 5.9 us past the wait).  Rows
 // in packed pairs over the exact support, zero weights instead of tests, and
 // the group's frame found by every warp: 32 videos of 64 frames 746.8 -> 740.0
