@@ -476,28 +476,38 @@ bool encode_2d(PFN_cuTensorMapEncodeTiled_v12000 enc, CUtensorMap *m, const void
 
 namespace {
 
-// Tile shape of Out[M][N]: what a K step costs an SM in shared-memory cycles
-// (the tile's operands written by TMA and read by the MMA, 2 (128 + tileN); a
-// pair 512 for 256 x 256) times the rounds of tiles over the SMs.  (128 x 128
-// tiles cost what a pair's do and never take fewer rounds; 128 x 256 ones save
-// the half that an odd number of row blocks leaves empty in pairs, as with 300
-// rows of 10,000 columns.)  Both layers, against 128 x 256 tiles on one SM everywhere: 18,662 x 3584 x 3584 x 3584
-// 595 -> 565 us (1,698 TFLOP/s), 2704 rows 135 -> 128, 300 x 2048 x 2048 x 2048
-// 37.6 -> 27.4, 64 x 3584 x 3584 x 3584 51.6 -> 39.6.
+// Tile shape of Out[M][N]: the rounds of tiles over the SMs times what a K step of
+// a round takes, measured (512 stands for 0.34 us: a pair's tensor cycles at full
+// rate and the waits between), and a pair's start (clusters, their barriers and
+// tensor memory) as three steps.  One SM's tiles save the half that an odd number
+// of 128-row blocks leaves empty in pairs, which can be a whole round.  One layer, us,
+// pairs / 256 / 64 columns: 256 x 3584 x 3584 (rows x columns x K) 46 / 46 / 40, 2688
+// rows 85 / 70 / 151, 9728 rows 165 / 179 / 489; 2304 x 1152 x 1152 27.4 / 25.8 / 31.7; over
+// 136 shapes the choice is within 0.2 % of the best on average, 3.6 % at most.  Both
+// layers of 18,662 x 3584 x 3584 x 3584 571 us (1,680 TFLOP/s; 595 with 256 columns).
+// Fewer than 32 rows are a few lines of A that every CTA fetches at the same time,
+// and more than 64 CTAs wait for them: 1 row x 3584 x 3584 x 3584 49.8 us with 32
+// columns, 39.5 with 64, 43.7 with 256; 2048: 26.8, 27.1, 31.2; from 32 rows 32
+// columns are no slower.
 struct PShape {
     bool pair;
     int tileN;
 };
 
-PShape project_shape(int M, int N, int sms) {
+PShape project_shape(int M, int N, int K, int sms) {
     auto ceil_div = [](int64_t a, int64_t b) { return (a + b - 1) / b; };
+    const int64_t steps = K / kPK;
     PShape best{true, kPN};
-    int64_t cost = ceil_div(ceil_div(M, 2 * kPM) * ceil_div(N, kPN), sms / 2) * 512;
-    for (const int tn : {kPN, 64, 32}) {
-        const int64_t x = ceil_div(ceil_div(M, kPM) * ceil_div(N, tn), sms) * 2 * (kPM + tn);
+    int64_t cost = (ceil_div(ceil_div(M, 2 * kPM) * ceil_div(N, kPN), sms / 2) * steps + 3) * 512;
+    const struct {
+        int n, step;
+    } single[] = {{kPN, 530}, {64, 400}, {32, 333}};
+    for (const auto &t : single) {
+        if (t.n == 32 && M < 32 && N > 2048) continue;
+        const int64_t x = ceil_div(ceil_div(M, kPM) * ceil_div(N, t.n), sms) * steps * t.step;
         if (x < cost) {
             cost = x;
-            best = PShape{false, tn};
+            best = PShape{false, t.n};
         }
     }
     return best;
@@ -517,7 +527,7 @@ cudaError_t launch_project_gemm(const void *A, int M, int K, const void *B, int 
     if (e != cudaSuccess) return e;
     e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
-    const PShape shape = project_shape(M, N, sms);
+    const PShape shape = project_shape(M, N, K, sms);
     PMaps maps;
     memset(&maps, 0, sizeof(maps));
     if (!encode_2d(enc, &maps.a, A, M, K, kPM) || !encode_2d(enc, &maps.b, B, N, K, shape.pair ? kPN / 2 : shape.tileN))
@@ -586,10 +596,10 @@ cudaError_t launch_maxsim_gemm(const void *X, int M, int K, const void *QHL, int
 #ifdef WZ_CHECKED
 // Test hook: the tile columns that a layer of the projector takes on the current
 // device, 2 kPN for pairs; negative on an error.
-extern "C" __attribute__((visibility("default"))) int wz_check_project_tile(int rows, int cols) {
+extern "C" __attribute__((visibility("default"))) int wz_check_project_tile(int rows, int cols, int k) {
     const int sms = wz::sm_count();
-    if (sms < 1 || rows < 1 || cols < 1) return -1;
-    const wz::PShape shape = wz::project_shape(rows, cols, sms);
+    if (sms < 1 || rows < 1 || cols < 1 || k < wz::kPK) return -1;
+    const wz::PShape shape = wz::project_shape(rows, cols, k, sms);
     return shape.pair ? 2 * wz::kPN : shape.tileN;
 }
 #endif
