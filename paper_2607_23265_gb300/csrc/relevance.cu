@@ -244,8 +244,12 @@ __global__ void __launch_bounds__(MAXTHREADS, 1) relevance_pass_kernel(Ctx c, Re
     // anything.
     pdl_trigger();
     constexpr int VEC = VecOf<T>::kElems;
-    constexpr int GROUP = kRelGroupTokens;
+    // tokens per transpose-reduction: chunks of long rows hold no more (1 or 2
+    // tokens with 8 vectors per thread, at most 4 with 4); with 8 for all, the
+    // widest rows spilled and took 2 % longer
+    constexpr int GROUP = VPT == 8 ? 1 : VPT == 4 ? 4 : kRelGroupTokens;
     constexpr int NV = 2 * GROUP;            // GROUP dots + GROUP squared norms
+    constexpr int HOLD = 32 / NV;            // lanes that end with the same value
     extern __shared__ __align__(128) uint8_t rsm[];
     __shared__ float qsum[kRelMaxWarps];
     __shared__ uint64_t full[kRelMaxStages], empty[kRelMaxStages];
@@ -406,8 +410,8 @@ __global__ void __launch_bounds__(MAXTHREADS, 1) relevance_pass_kernel(Ctx c, Re
                         acc[k + GROUP] = n2.x + n2.y;
                     }
                     const float tot = transpose_reduce<NV>(acc);
-                    const int kk = (lane >> 1) & (GROUP - 1);   // lane l holds value l >> 1: token kk, dot or norm
-                    if ((lane & 1) == 0 && kk < left) wp[(lane >> 4) * kRelWindow + wcount + g0 + kk] = tot;
+                    const int kk = (lane / HOLD) & (GROUP - 1);   // lane l holds value l / HOLD: token kk, dot or norm
+                    if (lane % HOLD == 0 && kk < left) wp[(lane >> 4) * kRelWindow + wcount + g0 + kk] = tot;
                 }
             }
             // hand the stage back once this warp's reads are done
@@ -1078,7 +1082,12 @@ struct RelCfg {
 // (16 x 16 maps), one group / 16 / 24 warps: D = 512: 181 / 119 / 120 us;
 // 1152: 212 / 161 / 158; 2304: 146 / - / 122; 2816: 127 / - / 116; 3072 (12
 // warps a row): 120.3 / - / 120.1.  A thread holds at most 8 elements of a row
-// in groups of more than one.  CTAs of fewer than 64 tokens (short clips) stay
+// in groups of more than one.  Rows of one warp take four groups: their chunks
+// are short work, and with more groups (or more than 8 tokens a chunk) the
+// barriers and the merge of the groups' sums at every frame end cost more than
+// they hide.  wz_relevance, one / four / sixteen groups (sixteen with chunks of 32
+// tokens): 4096 frames of 16 x 16 x 128 147 / 144 / 278 us, of 6 x 6 x 256 56 / 54 /
+// 91, 3000 of 7 x 7 x 64 fp32 40 / 42 / 91.  CTAs of fewer than 64 tokens (short clips) stay
 // with one group: the groups' column sums cost more than they save there (16
 // frames of 13 x 13 x 896: 27 us with one group, 30 us with three).
 template <typename T, int VPT>
@@ -1091,17 +1100,16 @@ void relevance_config(const Ctx &c, RelCfg &r) {
     sh.gthreads = std::max(32, ((n_vec + VPT - 1) / VPT + 31) / 32 * 32);
     const int w = sh.gthreads / 32;
     sh.groups = 1;
-    if (kNarrow) sh.groups = std::max(1, (16 / w) * w >= 15 ? 16 / w : kRelMaxWarps / w);
+    if (kNarrow) sh.groups = w == 1 ? 4 : std::max(1, (16 / w) * w >= 15 ? 16 / w : kRelMaxWarps / w);
     const int64_t per_cta = ((int64_t)c.V * c.T * c.N + c.sms - 1) / c.sms;
     sh.groups = (int)std::min<int64_t>(sh.groups, std::max<int64_t>(1, per_cta / 32));
     const size_t wpart = (size_t)2 * w * 2 * kRelWindow * 4;
     size_t csum = 0, ring = 0;
     for (; sh.groups > 1; --sh.groups) {
-        // chunks of 8 tokens (up to 32 and 8 KB: short rows), at least two
-        // stages per group
+        // chunks of 8 tokens, at least two stages per group
         csum = (size_t)(sh.groups - 1) * c.D * 4;
         ring = kRelSmem - wpart - csum;
-        sh.ch = 8 * (int)std::max<size_t>(1, std::min<size_t>(4, 8192 / (8 * rowb)));
+        sh.ch = 8;
         sh.stages = (int)std::min<size_t>(kRelMaxStages, ring / (sh.ch * rowb)) / sh.groups * sh.groups;
         if (sh.stages >= 2 * sh.groups) break;
     }

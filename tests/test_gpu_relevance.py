@@ -28,6 +28,13 @@ CASES = [
     (6, 9, 9, 4104, "bf16"),       # two vectors per thread
     (4, 8, 9, 8200, "bf16"),
     (5, 8, 9, 2056, "f32"),
+    (2100, 4, 4, 64, "f32"),       # rows of one warp: four groups, frames of two chunks
+    (700, 6, 6, 256, "bf16"),
+    (300, 7, 9, 136, "bf16"),
+    (4, 5, 5, 16392, "bf16"),      # eight vectors per thread: two tokens per chunk, then one
+    (3, 6, 7, 32768, "bf16"),
+    (3, 7, 7, 16384, "f32"),
+    (5, 6, 6, 8192, "f32"),        # four vectors per thread
 ]
 
 
