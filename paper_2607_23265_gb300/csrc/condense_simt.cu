@@ -167,6 +167,7 @@ cudaError_t launch_simt(const Ctx &c, int sms, cudaStream_t s) {
     int compact = frames <= kCompactFrames ? 1 : 0;
     const size_t smem = kSimtStages * simt_stage_bytes<Tin, TM, TN>() + (compact ? (size_t)(frames + 1) * 4 : 0);
     cudaError_t e = allow_smem(fn, smem);
+    if (e == cudaSuccess) e = prefer_smem(fn);
     if (e != cudaSuccess) return e;
     int per_sm = 0;
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, smem)) != cudaSuccess) return e;
@@ -184,11 +185,13 @@ cudaError_t launch_simt(const Ctx &c, int sms, cudaStream_t s) {
 // 32 x 128 / 64 x 128 / 128 x 128 tiles: 64 frames of 13 x 13 x 3584, 17 rows:
 // 57 / 61 / - / - us; 128 of 16 x 16 x 2048, 25 rows: - / 127 / 149 / 199; 32 of
 // 27 x 27 x 3584, 73 rows: - / - / 354 / 411; 64 of 27 x 27 x 2048, 182 rows:
-// - / - / 873 / 811 (43 TFLOP/s).
+// - / - / 873 / 811 (43 TFLOP/s).  Up to 64 channels wider tiles are half empty:
+// calls on 128 frames of 16 x 16 x 8, every token, 96 / 141 / 117 / 108.
 template <typename Tin>
 cudaError_t launch_simt_tiles(const Ctx &c, int sms, cudaStream_t s) {
     const int64_t rows = c.rows_total / ((int64_t)c.V * c.T), full = 2 * (int64_t)sms;
     auto tiles = [&](int tm, int tn) { return (c.rows_total + tm - 1) / tm * ((c.D + tn - 1) / tn); };
+    if (c.D <= 64) return launch_simt<Tin, 32, 64, 4, 1>(c, sms, s);
     if (rows >= 128 && tiles(128, 128) >= full) return launch_simt<Tin, 128, 128, 8, 2>(c, sms, s);
     if (rows >= 48 && tiles(64, 128) >= full) return launch_simt<Tin, 64, 128, 8, 2>(c, sms, s);
     if (tiles(32, 128) >= 2 * full) return launch_simt<Tin, 32, 128, 4, 2>(c, sms, s);

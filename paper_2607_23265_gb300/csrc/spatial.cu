@@ -501,6 +501,7 @@ cudaError_t launch_spatial(const Ctx &c, cudaStream_t s) {
     const size_t smem_c = spatial_compact_smem_bytes(c);
     const size_t smem_max = plain || (int64_t)c.V * c.T > kCompactFrames ? smem : smem_c;
     cudaError_t e = allow_smem(fn, smem_max);
+    if (e == cudaSuccess) e = prefer_smem(fn);
     if (e != cudaSuccess) return e;
     int dev = 0, sms = 0, per_sm = 0, per_sm_c = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
