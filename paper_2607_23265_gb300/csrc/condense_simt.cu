@@ -167,7 +167,6 @@ cudaError_t launch_simt(const Ctx &c, int sms, cudaStream_t s) {
     int compact = frames <= kCompactFrames ? 1 : 0;
     const size_t smem = kSimtStages * simt_stage_bytes<Tin, TM, TN>() + (compact ? (size_t)(frames + 1) * 4 : 0);
     cudaError_t e = allow_smem(fn, smem);
-    if (e == cudaSuccess) e = prefer_smem(fn);
     if (e != cudaSuccess) return e;
     int per_sm = 0;
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, smem)) != cudaSuccess) return e;

@@ -120,7 +120,7 @@ __device__ void plain_operator_rows(const Ctx &c, const SpatialSmem &L, float *s
 // Ablation modes without the WSM: S CTAs per frame, grid rows p = s0, s0 + S, ...
 __global__ void __launch_bounds__(kSpatialThreads) spatial_plain_kernel(Ctx c, int S) {
     pdl_wait();
-    pdl_trigger();
+    operator_trigger(c);
     extern __shared__ float sm[];
     const int64_t nblk_frames = (int64_t)c.V * c.T * S;
     if ((int64_t)blockIdx.x >= nblk_frames) {
@@ -157,7 +157,7 @@ __device__ __forceinline__ int frame_rows(const Ctx &c, int f) {
 // the rows that exist; otherwise it runs over all V*T*H (frame, row) pairs.
 template <int BMAX>
 __global__ void __launch_bounds__(kSpatialThreads, 4) spatial_wsm_kernel(Ctx c, int compact) {
-    pdl_trigger();
+    operator_trigger(c);
     extern __shared__ float sm[];
     __shared__ int s_item, s_f, s_wsum[kSpatialThreads / 32];
     const int tid = threadIdx.x;
@@ -501,7 +501,6 @@ cudaError_t launch_spatial(const Ctx &c, cudaStream_t s) {
     const size_t smem_c = spatial_compact_smem_bytes(c);
     const size_t smem_max = plain || (int64_t)c.V * c.T > kCompactFrames ? smem : smem_c;
     cudaError_t e = allow_smem(fn, smem_max);
-    if (e == cudaSuccess) e = prefer_smem(fn);
     if (e != cudaSuccess) return e;
     int dev = 0, sms = 0, per_sm = 0, per_sm_c = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;

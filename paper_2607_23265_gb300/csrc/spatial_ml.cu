@@ -20,7 +20,7 @@ namespace wz {
 template <int HMAX>
 __global__ void __launch_bounds__(kSpatialThreads) spatial_ml_kernel(Ctx c, int S) {
     pdl_wait();
-    pdl_trigger();
+    operator_trigger(c);
     extern __shared__ float sm[];
     const int tid = threadIdx.x;
     const int64_t nblk_frames = (int64_t)c.V * c.T * S;

@@ -183,16 +183,6 @@ inline cudaError_t allow_smem(const void *fn, size_t need) {
     return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
 }
 
-// All of an SM's L1 as shared memory while CTAs of fn run there.  An SM keeps its
-// split until it is empty, so CTAs of the next kernel that come beside the last
-// ones of this find the room that their occupancy says.  For the operator kernels
-// ahead of the CUDA-core condensation, whose CTAs hold fixed shares of its tiles:
-// 16 frames of 64 x 64 x 256 fp32 1016 us without, 764 with (the launches one after
-// the other 779); 16 of 14 x 14 x 896 49.9 and 44.5.
-inline cudaError_t prefer_smem(const void *fn) {
-    return cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-}
-
 __device__ __forceinline__ int ext_index(int i, int n, int mode) {
     if (i >= 0 && i < n) return i;
     if (mode == WZ_MODE_ZERO) return -1;

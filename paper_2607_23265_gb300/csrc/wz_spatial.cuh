@@ -154,6 +154,17 @@ __device__ __forceinline__ void write_rows(const Ctx &c, const float *stg, int k
     }
 }
 
+// The tensor-core condensation (one CTA per SM, claims its units) may come to the
+// SMs while an operator kernel runs.  The CUDA-core one may not: its CTAs hold fixed
+// shares of its tiles, and those that came early would share the few SMs with room
+// beside operator CTAs, two or more on an SM while others get none.  There the
+// operator kernel's CTAs let it start by their exit.  Calls in fp32 with both / with
+// this: 6 frames of 48 x 48 x 1024 650 / 499 us, 16 of 64 x 64 x 256 1060 / 807, 64 of 13
+// x 13 x 1024 67.6 / 57.4, 16 of 14 x 14 x 896 55.2 / 49.4.
+__device__ __forceinline__ void operator_trigger(const Ctx &c) {
+    if (c.path == WZ_PATH_TENSOR) pdl_trigger();
+}
+
 constexpr int kSpatialThreads = 256;
 constexpr int kTailBlocks = 64;
 
