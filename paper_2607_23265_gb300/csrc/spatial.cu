@@ -148,8 +148,8 @@ __device__ __forceinline__ int frame_rows(const Ctx &c, int f) {
 }
 
 // The WSM operator rows (single level), persistent: every CTA copies the
-// frame-independent tables once, then takes grid rows (frame f, row p) from
-// a global counter until none is left; a row whose frame changes reloads
+// frame-independent tables once, then takes its own grid row (frame f, row p) and
+// further ones from a global counter until none is left; a row whose frame changes reloads
 // the frame's gate and width rows.  Rows of frames with a small budget cost
 // as much as others, so the dynamic order keeps the SMs evenly loaded.  With
 // compact != 0 (at most kCompactFrames frames) every CTA first forms the
@@ -169,9 +169,11 @@ __global__ void __launch_bounds__(kSpatialThreads, 4) spatial_wsm_kernel(Ctx c, 
     // while it runs
     build_spatial_tables_smem(c, L, sm);
     pdl_wait();
-    // thread 0 claims the next row while the current one is formed, so the
-    // counter's round trip overlaps the work
-    int claimed = tid == 0 ? atomicAdd(c.spatial_next, 1) : 0;
+    // the first row is the CTA's own index, so that few rows go to different SMs (6
+    // frames of 48 x 48 x 1024 160 us a call; 206 to 219 with claims, where the CTAs
+    // of an SM came one after the other); thread 0 claims the next row while the
+    // current one is formed, so the counter's round trip overlaps the work
+    int claimed = (int)blockIdx.x;
     if ((int)blockIdx.x < kTailBlocks) tail_rows(c, (int)blockIdx.x);
     float *G = sm + L.G;
     float *AHl = sm + L.AHl, *AHh = sm + L.AHh, *AWl = sm + L.AWl, *AWh = sm + L.AWh;
@@ -207,7 +209,7 @@ __global__ void __launch_bounds__(kSpatialThreads, 4) spatial_wsm_kernel(Ctx c, 
         __syncthreads();   // the previous row's reads of shared memory
         if (tid == 0) {
             const int it = claimed;
-            if (it < items) claimed = atomicAdd(c.spatial_next, 1);
+            if (it < items) claimed = (int)gridDim.x + atomicAdd(c.spatial_next, 1);
             int fi = 0;
             if (compact && it < items) {
                 // the last frame whose first row is <= it (frames without
