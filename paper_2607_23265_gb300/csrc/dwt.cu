@@ -365,16 +365,18 @@ Taps make_taps(const float *lo, const float *hi, int F) {
 }
 
 // Launch shape of the 2D kernels: CT channels per CTA (the most of 64, 32, 16
-// whose shared memory is at most 72 KB, so that three CTAs share an SM, and
-// whose longer pass is at most one round of the CTA's threads; else 8, which
-// fits at the largest map and filter), one thread per run of that pass.
+// whose shared memory is at most 72 KB, so that three CTAs share an SM, whose
+// longer pass is at most one round of the CTA's threads, and which D fills to more
+// than a half; else 8, which fits at the largest map and filter), one thread per
+// run of that pass.
 struct DwtCfg {
     int ct, threads;
     size_t smem;
 };
 
-DwtCfg dwt_config(size_t bytes_per_channel, int runs_per_channel, int vc, int max_threads) {
+DwtCfg dwt_config(size_t bytes_per_channel, int runs_per_channel, int D, int vc, int max_threads) {
     int ct = 64;
+    while (ct > 8 && 2 * D <= ct) ct >>= 1;
     while (ct > 8 && (bytes_per_channel * ct > 72 * 1024 || runs_per_channel * ct / vc > max_threads)) ct >>= 1;
     return {ct, std::min(max_threads, (runs_per_channel * ct / vc + 31) / 32 * 32), bytes_per_channel * ct};
 }
@@ -447,7 +449,8 @@ cudaError_t launch_dwt2d(const void *X, int dtype, int T, int H, int W, int D, i
     const int vc = pair_ok(D, {LL, LH, HL, HH}, X, bf ? 2 : 4) ? 2 : 1;
     const int wp = (W + F - 1) / 2;
     const size_t esz = bf ? 2 : 4;
-    const DwtCfg k = dwt_config((size_t)(H + 1) * dwt_row(wp) * 4 + (size_t)H * dwt_row(W + 1) * esz, std::max(H, wp), vc, kDwtThreads);
+    const DwtCfg k = dwt_config((size_t)(H + 1) * dwt_row(wp) * 4 + (size_t)H * dwt_row(W + 1) * esz, std::max(H, wp), D, vc,
+                                kDwtThreads);
     int vec = ((uintptr_t)X % 16 == 0 && (size_t)D * esz % 16 == 0) ? 1 : 0;
     const void *fn = bf ? pick_dwt2d<__nv_bfloat16>(F, vc) : pick_dwt2d<float>(F, vc);
     if (!fn) return cudaErrorInvalidValue;
@@ -464,7 +467,7 @@ cudaError_t launch_idwt2d(const float *LL, const float *LH, const float *HL, con
                           float *out, cudaStream_t s) {
     const int vc = pair_ok(D, {LL, LH, HL, HH, out}, nullptr, 4) ? 2 : 1;
     const int wp = (W + F - 1) / 2;
-    const DwtCfg k = dwt_config((size_t)H * dwt_row(2 * wp) * 4, std::max(H, 2 * wp), vc, kIdwtThreads);
+    const DwtCfg k = dwt_config((size_t)H * dwt_row(2 * wp) * 4, std::max(H, 2 * wp), D, vc, kIdwtThreads);
     const void *fn = pick_idwt2d(F, vc);
     if (!fn) return cudaErrorInvalidValue;
     const cudaError_t e = allow_smem(fn, k.smem);

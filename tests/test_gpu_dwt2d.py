@@ -27,6 +27,12 @@ CASES = [
     (64, 64, 11, 10, "symmetric", "f32", 0),
     (64, 63, 10, 10, "periodic", "bf16", 0),
     (27, 26, 34, 44, "symmetric", "bf16", 0),
+    (4, 4, 1, 1, "symmetric", "bf16", 0),        # few channels: chunks of 8, 16, 32, 64
+    (4, 5, 3, 1, "zero", "f32", 0),
+    (2, 4, 8, 4, "symmetric", "bf16", 0),
+    (4, 4, 9, 1, "periodic", "f32", 0),
+    (3, 2, 17, 2, "symmetric", "bf16", 0),
+    (4, 2, 32, 1, "symmetric", "f32", 0),
 ]
 
 
